@@ -1260,6 +1260,7 @@ int amber_batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, cons
       xpre.push_back(xpre.back() + (uint32_t)(xa.groups * xa.nbuckets));
     }
     am.M = nitems;
+    for (const ThreshArgs& t : th) am.max_table = std::max(am.max_table, t.M);
     for (int f = 0; f < 2; ++f) {
       am.Mg[f] = (int)sc[f].size();
       am.scan_tiles[f] = spre[f].back();

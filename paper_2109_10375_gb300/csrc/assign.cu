@@ -78,6 +78,25 @@ __device__ __forceinline__ u128 mul_floor(double x, u128 T) {
   return (top << (64 - s)) | (u128)(p0 >> s);
 }
 
+// Block sum of the per-tile mass sums first, first + step, ... (valid on thread 0).
+__device__ __forceinline__ u128 sum_tile_mass(const unsigned long long* __restrict__ tile_mass, int64_t ntiles,
+                                              int64_t first, int64_t step) {
+  __shared__ u128 ws[32];
+  u128 acc = 0;
+  for (int64_t t = first; t < ntiles; t += step) {
+    const ulonglong2 v = reinterpret_cast<const ulonglong2*>(tile_mass)[t];
+    acc += ((u128)v.y << 64) | (u128)v.x;
+  }
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) acc += shfl_down_u128(acc, o);
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  u128 s = 0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += ws[w];
+  return s;
+}
+
 // Linear growth factor D(a) of flat LCDM (Omega_m = om, Omega_L = 1 - om),
 // normalised to D = a early on: D(a) = (5 om / 2) E(a) int_0^a da'/(a' E(a'))^3
 // with E(a) = sqrt(om a^-3 + 1 - om).  In closed form D(a) = a 2F1(1/3, 1;
@@ -110,102 +129,104 @@ __device__ double growth_D(double a, double om) {
   return 2.5 * om * E * I;
 }
 
-// tile_mass (optional): per-tile partial sums from the ranking; their total
-// is formed here (exact, order-free).  From the exact total T (2^-64 units)
-// the kernel picks the scan's fixed-point shift s (total below 2^62), and
-// tabulates X_j = floor(x_j T 2^(s-64)) so "x_j >= F_n" is the integer test
-// "X_j >= M_n", plus 1/(X_j - X_j+1) for the interpolation weight.
-__device__ __forceinline__ void thresholds_body(const ThreshArgs& A) {
-  unsigned long long* __restrict__ total = A.total;
-  const unsigned long long* __restrict__ tile_mass = A.tile_mass;
-  const int64_t ntiles = A.ntiles;
-  const int M = A.M;
-  const double a_w = A.a_w, b_w = A.b_w, c_w = A.c_w, z_lo = A.z_lo, z_hi = A.z_hi;
-  unsigned long long* __restrict__ Xq = A.Xq;
-  float* __restrict__ inv_dx = A.inv_dx;
-  int* __restrict__ qshift = A.qshift;
-  unsigned long long* __restrict__ qtotal = A.qtotal;
-  const int weighting = A.weighting;
-  const double omega_m = A.omega_m, z_mid = A.z_mid;
-  const int64_t ncells = A.ncells;
-  float* __restrict__ lin = A.lin;
-  __shared__ u128 ws[32];
+// Exact total of the ranking's per-tile mass sums into total (zeroed): for
+// many tiles, where reading them all in every thresholds CTA would cost more
+// than this launch.  (1024^3: 262144 sums, 4 MB, over 64 CTAs.)
+__global__ void __launch_bounds__(256) k_tile_total(const unsigned long long* __restrict__ tile_mass, int64_t ntiles,
+                                                    unsigned long long* __restrict__ total) {
+  const u128 s = sum_tile_mass(tile_mass, ntiles, (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
+                               (int64_t)gridDim.x * blockDim.x);
+  if (threadIdx.x == 0 && s != 0) atomic_add_u128(total, s);
+}
+
+// From the exact total T (2^-64 units) the kernel picks the scan's
+// fixed-point shift s (total below 2^62), and tabulates X_j = floor(x_j T
+// 2^(s-64)) so "x_j >= F_n" is the integer test "X_j >= M_n", plus
+// 1/(X_j - X_j+1) for the interpolation weight.  tile_mass (optional):
+// per-tile partial sums from the ranking; every CTA adds them up itself
+// (exact, order-free), so no launch is needed for the total.
+// The table's exp, pow and growth series run on the FP64 pipe, which takes 16
+// cycles per warp instruction here: one warp per CTA evaluates 31 points (and
+// the next one, for the difference), so 2000 points spread over 65 SMs, and
+// warps 1-7 read the partial sums meanwhile.  One CTA of 1024 threads for the
+// whole table took 103 us (growth weighting 255 us); a 32^3 solve went from 256
+// to 145 us with this and the scan's gallop, a 128^3 growth one from 1501 to 489.
+constexpr int kThreshThreads = 256;
+constexpr int kThreshPoints = 31;
+// more tile sums than this take a launch of their own (k_tile_total): 4096
+// sums are 64 KB read per CTA, about 1 us; 262144 would be 4 MB, over 30 us
+constexpr int64_t kTileTotalMin = 4096;
+
+__device__ __forceinline__ void thresholds_body(const ThreshArgs& A, int blk) {
   __shared__ u128 sT;
-  __shared__ int s_shift;
-  if (tile_mass) {
-    u128 acc = 0;
-    for (int64_t t = threadIdx.x; t < ntiles; t += blockDim.x)
-      acc += ((u128)tile_mass[2 * t + 1] << 64) | (u128)tile_mass[2 * t];
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) acc += shfl_down_u128(acc, o);
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      u128 s = 0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += ws[w];
-      total[0] = (unsigned long long)s;
-      total[1] = (unsigned long long)(s >> 64);
-      sT = s;
+  const int lane = threadIdx.x & 31, M = A.M;
+  const int j = blk * kThreshPoints + lane;
+  const bool mine = threadIdx.x < 32 && j < M;
+  double x = 0.0, alpha = 1.0, beta = 0.0;  // weight of a cell at z_j: alpha + beta mass (volume weighting: 1)
+  if (mine) {
+    const double z = A.z_lo + (A.z_hi - A.z_lo) * (double)j / (double)(M - 1);
+    const double u = fmax((z - A.a_w) / A.b_w, 0.0);
+    x = exp(-pow(u, A.c_w));
+    if (A.weighting == AMBER_WEIGHT_MASS_GROWTH) {
+      const double g = growth_D(1.0 / (1.0 + z), A.omega_m) / growth_D(1.0 / (1.0 + A.z_mid), A.omega_m);
+      alpha = 1.0 - g;
+      beta = g;
     }
+  }
+  if (A.tile_mass) {
+    const u128 s = sum_tile_mass(A.tile_mass, A.ntiles, threadIdx.x, blockDim.x);
+    if (threadIdx.x == 0) sT = s;
   } else if (threadIdx.x == 0) {
-    sT = ((u128)total[1] << 64) | (u128)total[0];
+    sT = ((u128)A.total[1] << 64) | (u128)A.total[0];
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    // bit length L of T; the real total is below 2^(L-64), so s = 126 - L
-    // keeps it below 2^62 (s <= 64: no finer than the exact representation)
-    int L = 0;
-    for (u128 v = sT; v != 0; v >>= 1) ++L;
-    int s = 126 - L;
-    if (s > 64) s = 64;
-    s_shift = s;
-    *qshift = s;
-    const int sh = 64 - s;
-    *qtotal = (unsigned long long)(sh >= 0 ? (sT >> sh) : (sT << (-sh)));
-  }
-  __syncthreads();
+  if (threadIdx.x >= 32) return;
   const u128 T = sT;
-  const int sh = 64 - s_shift;  // X in 2^-s units: floor(x T) >> (64 - s)
-  for (int j = threadIdx.x; j < M; j += blockDim.x) {
-    const double z = z_lo + (z_hi - z_lo) * (double)j / (double)(M - 1);
-    const double u = fmax((z - a_w) / b_w, 0.0);
-    const double x = exp(-pow(u, c_w));
-    const u128 X = mul_floor(x, T);
-    Xq[j] = (unsigned long long)(sh >= 0 ? (X >> sh) : (X << (-sh)));
-    if (weighting != AMBER_WEIGHT_MASS) {
-      // weight of a cell at z_j: alpha_j + beta_j mass; margin h_j(n) =
-      // x_j W_N - W_n.  Two equal forms keep the operands small at either end
-      // of the ranking: the head form x_j W_N - alpha_j n - beta_j M_n for the
-      // first half of the ranks, and the tail form (x_j - 1) W_N +
-      // alpha_j (N - n) + beta_j (T - M_n) for the second, where the weight
-      // after rank n (all that is left on the x = 1 plateau) comes from exact
-      // differences
-      double alpha = 1.0, beta = 0.0;  // volume
-      if (weighting == AMBER_WEIGHT_MASS_GROWTH) {
-        const double g = growth_D(1.0 / (1.0 + z), omega_m) / growth_D(1.0 / (1.0 + z_mid), omega_m);
-        alpha = 1.0 - g;
-        beta = g;
-      }
-      const double Treal = u128_to_double(T) * 5.421010862427522e-20;  // 2^-64
-      const double WN = alpha * (double)ncells + beta * Treal;
-      lin[j] = (float)(x * WN);
-      lin[kMaxTable + j] = (float)((x - 1.0) * WN);
-      lin[2 * kMaxTable + j] = (float)alpha;
-      lin[3 * kMaxTable + j] = (float)beta;
-    }
+  // bit length L of T; the real total is below 2^(L-64), so s = 126 - L
+  // keeps it below 2^62 (s <= 64: no finer than the exact representation)
+  const unsigned long long th = (unsigned long long)(T >> 64), tl = (unsigned long long)T;
+  const int L = th ? 128 - __clzll((long long)th) : 64 - __clzll((long long)tl);
+  const int s = 126 - L < 64 ? 126 - L : 64;
+  const int sh = 64 - s;  // X in 2^-s units: floor(x T) >> (64 - s)
+  if (blk == 0 && lane == 0) {
+    *A.qshift = s;
+    *A.qtotal = (unsigned long long)(sh >= 0 ? (T >> sh) : (T << (-sh)));
   }
-  __syncthreads();
-  for (int j = threadIdx.x; j < M - 1; j += blockDim.x) {
-    const unsigned long long d = Xq[j] - Xq[j + 1];
-    inv_dx[j] = d > 0 ? 1.0f / __ull2float_rn(d) : 0.0f;
+  const u128 X = mul_floor(x, T);
+  const unsigned long long Xq = mine ? (unsigned long long)(sh >= 0 ? (X >> sh) : (X << (-sh))) : 0ull;
+  const unsigned long long next = __shfl_down_sync(0xffffffffu, Xq, 1);
+  if (!mine || lane >= kThreshPoints) return;  // lane 31's point belongs to the next CTA
+  A.Xq[j] = Xq;
+  if (j < M - 1) {
+    const unsigned long long d = Xq - next;
+    A.inv_dx[j] = d > 0 ? 1.0f / __ull2float_rn(d) : 0.0f;
+  }
+  if (A.weighting != AMBER_WEIGHT_MASS) {
+    // margin h_j(n) = x_j W_N - W_n.  Two equal forms keep the operands small
+    // at either end of the ranking: the head form x_j W_N - alpha_j n - beta_j
+    // M_n for the first half of the ranks, and the tail form (x_j - 1) W_N +
+    // alpha_j (N - n) + beta_j (T - M_n) for the second, where the weight
+    // after rank n (all that is left on the x = 1 plateau) comes from exact
+    // differences
+    const double Treal = u128_to_double(T) * 5.421010862427522e-20;  // 2^-64
+    const double WN = alpha * (double)A.ncells + beta * Treal;
+    A.lin[j] = (float)(x * WN);
+    A.lin[kMaxTable + j] = (float)((x - 1.0) * WN);
+    A.lin[2 * kMaxTable + j] = (float)alpha;
+    A.lin[3 * kMaxTable + j] = (float)beta;
   }
 }
 
-__global__ void __launch_bounds__(1024) k_thresholds(const ThreshArgs A) { thresholds_body(A); }
+__global__ void __launch_bounds__(kThreshThreads) k_thresholds(const ThreshArgs A) {
+  thresholds_body(A, (int)blockIdx.x);
+}
 
-// One CTA per item.
-__global__ void __launch_bounds__(1024) k_thresholds_multi(const ThreshArgs* __restrict__ args) {
-  thresholds_body(args[blockIdx.x]);
+// CTA (x, y): points of CTA x of item y's table.
+__global__ void __launch_bounds__(kThreshThreads) k_thresholds_multi(const ThreshArgs* __restrict__ args) {
+  __shared__ ThreshArgs A;
+  if (threadIdx.x == 0) A = args[blockIdx.y];
+  __syncthreads();
+  if ((int)blockIdx.x * kThreshPoints < A.M) thresholds_body(A, (int)blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -259,19 +280,20 @@ __device__ __forceinline__ void count_ge_round(const unsigned long long* __restr
 
 constexpr int kScanWin = 64;  // thresholds one tile may span, staged in shared memory
 
-constexpr int kLinCand = 256;  // table points a tile's cells may straddle (linear weightings)
-
 // LIN: a linear weighting (growth or volume).  The exact-integer threshold
-// test of the mass weighting is replaced by the margins h_j(n) in FP32: per
-// tile, every table point is classified against the box of (n, M_n) the
-// tile's cells span -- ionized for all of them, for none, or straddling --
-// and each cell takes the largest point that ionizes it among
-// max{j : all ionized} and the straddling points above it.
+// test of the mass weighting is replaced by the margins h_j(n) in FP32: a
+// cell takes the largest table point j with h_j >= 0.  A margin is linear in
+// (n, M_n), so its extremes over the box that a run of ranks spans lie at the
+// corners.  Per tile every point is classified: jall is the largest one that
+// ionizes all of its cells, jtop the largest one that can ionize any.  From
+// jtop each warp walks down 32 points at a time to the first one its own box
+// allows, each thread from there to the first one its 16 ranks allow, and only
+// then each cell tests margins.  (The first tile of 128^3 spans over 1000 of
+// 2000 points; with every cell testing all of the tile's points it took 1.06 ms.)
 template <bool GATHER, bool WANT_F, bool LIN>
 __device__ __forceinline__ void scan_assign_body(const ScanArgs& a) {
   constexpr int NT = kScanThreads, IT = kScanItems, TILE = kScanTile;
-  __shared__ int s_jall, s_ncand;
-  __shared__ int s_cand[LIN ? kLinCand : 1];
+  __shared__ int s_jall, s_jtop;
   __shared__ uint32_t sord[TILE + TILE / 32];
   __shared__ float smass[TILE + TILE / 32];
   __shared__ unsigned long long wtot[NT / 32];
@@ -286,7 +308,7 @@ __device__ __forceinline__ void scan_assign_body(const ScanArgs& a) {
   if (tid == 0) {
     s_tile = atomicAdd(a.ticket, 1u);
     s_jall = -1;
-    s_ncand = 0;
+    s_jtop = -1;
   }
   for (int b = tid; b < a.nbuckets; b += NT) scnt[b] = 0;
   __syncthreads();
@@ -467,34 +489,34 @@ __device__ __forceinline__ void scan_assign_body(const ScanArgs& a) {
   const bool head = start + (uint32_t)cnt / 2u <= n / 2u;
   const float* linC = head ? a.linP : a.linQ;
   const float sa = head ? -1.0f : 1.0f;
+  // table point j over the box of ranks (r0, r1] (from 0) with prefix masses
+  // in [m0, m1]: bounds of its margin and the rounding they are good to
+  struct Box { float u0, u1, v0, v1; };
+  auto box_of = [&](uint32_t r0, uint32_t r1, unsigned long long m0, unsigned long long m1) -> Box {
+    if (head) return {(float)(r0 + 1u), (float)r1, u64_to_float(m0) * qinv, u64_to_float(m1) * qinv};
+    return {(float)(n - r1), (float)(n - (r0 + 1u)), u64_to_float(qT - m1) * qinv, u64_to_float(qT - m0) * qinv};
+  };
+  auto classify = [&](const Box& x, int j, float& hmin, float& hmax, float& tol) {
+    const float Cj = linC[j], al = sa * a.lina[j], be = sa * a.linb[j];
+    const float au0 = al * x.u0, au1 = al * x.u1, bv0 = be * x.v0, bv1 = be * x.v1;
+    hmin = Cj + fminf(au0, au1) + fminf(bv0, bv1);
+    hmax = Cj + fmaxf(au0, au1) + fmaxf(bv0, bv1);
+    tol = 4e-7f * (fabsf(Cj) + fmaxf(fabsf(au0), fabsf(au1)) + fmaxf(fabsf(bv0), fabsf(bv1)));
+  };
   if constexpr (LIN) {
-    // (u, v) of the tile's cells lie in the box [u0, u1] x [v0, v1]; a linear
-    // margin takes its extremes at the corners
-    const float u0 = head ? (float)(start + 1u) : (float)(n - (start + (uint32_t)cnt));
-    const float u1 = head ? (float)(start + (uint32_t)cnt) : (float)(n - (start + 1u));
-    const float v0 = head ? u64_to_float(s_excl) * qinv : u64_to_float(qT - (s_excl + tile_sum)) * qinv;
-    const float v1 = head ? u64_to_float(s_excl + tile_sum) * qinv : u64_to_float(qT - s_excl) * qinv;
-    auto classify = [&](int j, float& hmin, float& hmax, float& tol) {
-      const float Cj = linC[j], al = sa * a.lina[j], be = sa * a.linb[j];
-      const float au0 = al * u0, au1 = al * u1, bv0 = be * v0, bv1 = be * v1;
-      hmin = Cj + fminf(au0, au1) + fminf(bv0, bv1);
-      hmax = Cj + fmaxf(au0, au1) + fmaxf(bv0, bv1);
-      tol = 4e-7f * (fabsf(Cj) + fmaxf(fabsf(au0), fabsf(au1)) + fmaxf(fabsf(bv0), fabsf(bv1)));
-    };
+    const Box tb = box_of(start, start + (uint32_t)cnt, s_excl, s_excl + tile_sum);
+    int ja = -1, jt = -1;
     for (int j = tid; j < M; j += NT) {
       float hmin, hmax, tol;
-      classify(j, hmin, hmax, tol);
-      if (hmin >= tol) atomicMax(&s_jall, j);
+      classify(tb, j, hmin, hmax, tol);
+      if (hmin >= tol) ja = j;
+      if (hmax >= -tol) jt = j;
     }
-    __syncthreads();
-    const int jall = s_jall;
-    for (int j = jall + 1 + tid; j < M; j += NT) {
-      float hmin, hmax, tol;
-      classify(j, hmin, hmax, tol);
-      if (hmax >= -tol) {
-        const int k = atomicAdd(&s_ncand, 1);
-        if (k < kLinCand) s_cand[k] = j;
-      }
+    ja = __reduce_max_sync(0xffffffffu, ja);
+    jt = __reduce_max_sync(0xffffffffu, jt);
+    if (lane == 0) {
+      if (ja >= 0) atomicMax(&s_jall, ja);
+      if (jt >= 0) atomicMax(&s_jtop, jt);
     }
     __syncthreads();
   }
@@ -509,7 +531,7 @@ __device__ __forceinline__ void scan_assign_body(const ScanArgs& a) {
   // (order and masses were consumed above, so their shared arrays are free).
   uint32_t* scell = sord;
   float* sz = smass;
-  if (LIN && s_ncand == 0) {
+  if (LIN && s_jtop <= s_jall) {
     // no table point above max{j : all ionized} can ionize any cell of the
     // tile: every cell takes j* = jall, whose two margin rows are held in
     // registers
@@ -568,6 +590,63 @@ __device__ __forceinline__ void scan_assign_body(const ScanArgs& a) {
       scell[q + (q >> 5)] = cell[i];
       sz[q + (q >> 5)] = z;
     }
+  } else if constexpr (LIN) {
+    const int jall = s_jall;
+    int jt = s_jtop;
+    {
+      // the warp's ranks: 32 points per round from the top down
+      const uint32_t w0 = start + (uint32_t)min(warp * 32 * IT, cnt), w1 = start + (uint32_t)min((warp + 1) * 32 * IT, cnt);
+      const Box wbx = box_of(w0, w1, s_excl + wpre, s_excl + wpre + wtot[warp]);
+      unsigned hit = 0;
+      if (w1 > w0) {
+        for (; jt > jall; jt -= 32) {
+          const int j = jt - lane;
+          float hmin, hmax = -1.f, tol = 0.f;
+          if (j > jall) classify(wbx, j, hmin, hmax, tol);
+          hit = __ballot_sync(0xffffffffu, j > jall && hmax >= -tol);
+          if (hit) break;
+        }
+      }
+      jt = hit ? jt - (__ffs(hit) - 1) : jall;
+    }
+    if (tid * IT < cnt) {
+      const Box cb = box_of(start + (uint32_t)(tid * IT), start + (uint32_t)min((tid + 1) * IT, cnt), Mn, Mn + run);
+      for (; jt > jall; --jt) {
+        float hmin, hmax, tol;
+        classify(cb, jt, hmin, hmax, tol);
+        if (hmax >= -tol) break;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < IT; ++i) {
+      const int p = tid * IT + i;
+      if (p >= cnt) continue;
+      Mn += mass_fix(mv[i], qs);
+      // the cell's own form (a tile can straddle the middle rank; the boxes'
+      // classification above carries a tolerance for either form)
+      const uint32_t rank1 = start + (uint32_t)p + 1u;
+      const bool chead = rank1 <= n / 2u;
+      const float cs = chead ? -1.0f : 1.0f;
+      const float* cC = chead ? a.linP : a.linQ;
+      const float uu = cs * (chead ? (float)rank1 : (float)(n - rank1));
+      const float vv = cs * (chead ? u64_to_float(Mn) * qinv : u64_to_float(qT - Mn) * qinv);
+      auto h = [&](int j) { return fmaf(a.linb[j], vv, fmaf(a.lina[j], uu, cC[j])); };
+      int js = jt;
+      while (js > jall && !(h(js) >= 0.0f)) --js;
+      float z;
+      if (js < 0) z = a.z_lo;
+      else if (js == M - 1) z = a.z_hi;
+      else {
+        const float h0 = h(js), h1 = h(js + 1);
+        float t = h0 / (h0 - h1);
+        t = fminf(fmaxf(t, 0.0f), 0.99999994f);
+        z = a.z_lo + ((float)js + t) * a.dzt;
+      }
+      if (WANT_F) a.F[start + p] = (double)Mn * invT;
+      const uint32_t q = soff[cell[i] >> a.bucket_shift] + slot[i];
+      scell[q + (q >> 5)] = cell[i];
+      sz[q + (q >> 5)] = z;
+    }
   } else {
     int cx = -1;
 #pragma unroll
@@ -575,52 +654,27 @@ __device__ __forceinline__ void scan_assign_body(const ScanArgs& a) {
       const int p = tid * IT + i;
       if (p >= cnt) continue;
       Mn += mass_fix(mv[i], qs);
-      if constexpr (LIN) {
-        // the cell's own form (a tile can straddle the middle rank; the tile's
-        // classification above carries a tolerance for either form)
-        const uint32_t rank1 = start + (uint32_t)p + 1u;
-        const bool chead = rank1 <= n / 2u;
-        const float cs = chead ? -1.0f : 1.0f;
-        const float* cC = chead ? a.linP : a.linQ;
-        const float uu = cs * (chead ? (float)rank1 : (float)(n - rank1));
-        const float vv = cs * (chead ? u64_to_float(Mn) * qinv : u64_to_float(qT - Mn) * qinv);
-        auto h = [&](int j) { return fmaf(a.linb[j], vv, fmaf(a.lina[j], uu, cC[j])); };
-        int js = s_jall;
-        const int nc = s_ncand;
-        if (nc <= kLinCand) {
-          for (int k = 0; k < nc; ++k) {
-            const int c = s_cand[k];
-            if (c > js && h(c) >= 0.0f) js = c;
+      int lo = cx_lo, hi = cx_hi;
+      if (cx >= 0) {
+        // the prefix grew: gallop down from the last cell's bracket (in a
+        // small grid's first tile neighbours lie hundreds of points apart, and
+        // stepping through them one dependent load at a time took 63 us at 32^3)
+        hi = cx;
+        lo = cx;
+        for (int step = 1; lo > cx_lo; step *= 2) {
+          const int q = max(lo - step, cx_lo);
+          if (Xj(q) >= Mn) {
+            lo = q + 1;
+            break;
           }
-        } else {
-          for (int c = M - 1; c > js; --c)
-            if (h(c) >= 0.0f) { js = c; break; }
+          hi = lo = q;
         }
-        float z;
-        if (js < 0) z = a.z_lo;
-        else if (js == M - 1) z = a.z_hi;
-        else {
-          const float h0 = h(js), h1 = h(js + 1);
-          float t = h0 / (h0 - h1);
-          t = fminf(fmaxf(t, 0.0f), 0.99999994f);
-          z = a.z_lo + ((float)js + t) * a.dzt;
-        }
-        if (WANT_F) a.F[start + p] = (double)Mn * invT;
-        const uint32_t q = soff[cell[i] >> a.bucket_shift] + slot[i];
-        scell[q + (q >> 5)] = cell[i];
-        sz[q + (q >> 5)] = z;
-        continue;
       }
-      if (cx < 0) {
-        int lo = cx_lo, hi = cx_hi;
-        while (lo < hi) {
-          const int mid = (lo + hi) >> 1;
-          if (Xj(mid) >= Mn) lo = mid + 1; else hi = mid;
-        }
-        cx = lo;
-      } else {
-        while (cx > 0 && Xj(cx - 1) < Mn) --cx;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (Xj(mid) >= Mn) lo = mid + 1; else hi = mid;
       }
+      cx = lo;
       const int j = cx - 1;
       float z;
       if (j < 0) z = a.z_lo;
@@ -899,7 +953,12 @@ cudaError_t assign_impl(const AssignWork& w, const uint32_t* order, const float*
   }
 
   prof_begin(prof, PK_THRESHOLDS, s);
-  k_thresholds<<<1, 1024, 0, s>>>(ta);
+  if (ta.ntiles > kTileTotalMin) {
+    k_tile_total<<<(unsigned)std::min<int64_t>(64, (ta.ntiles + 1023) / 1024), 256, 0, s>>>(tile_mass, ta.ntiles,
+                                                                                         ta.total);
+    ta.tile_mass = nullptr;
+  }
+  k_thresholds<<<(ta.M + kThreshPoints - 1) / kThreshPoints, kThreshThreads, 0, s>>>(ta);
   prof_end(prof, PK_THRESHOLDS, s);
 
   prof_begin(prof, PK_SCAN_ASSIGN, s);
@@ -925,7 +984,8 @@ cudaError_t assign_impl(const AssignWork& w, const uint32_t* order, const float*
 }
 
 cudaError_t assign_multi(const AssignMulti& m, cudaStream_t s) {
-  k_thresholds_multi<<<m.M, 1024, 0, s>>>(m.thresh);
+  k_thresholds_multi<<<dim3((unsigned)((m.max_table + kThreshPoints - 1) / kThreshPoints), (unsigned)m.M),
+                       kThreshThreads, 0, s>>>(m.thresh);
   if (m.scan_tiles[0]) k_scan_assign_multi<false><<<m.scan_tiles[0], kScanThreads, 0, s>>>(m.scan[0], m.scan_prefix[0], m.Mg[0]);
   if (m.scan_tiles[1]) k_scan_assign_multi<true><<<m.scan_tiles[1], kScanThreads, 0, s>>>(m.scan[1], m.scan_prefix[1], m.Mg[1]);
   k_scatter_back_multi<<<m.scatter_blocks, 256, 0, s>>>(m.scatter, m.scatter_prefix, m.M);

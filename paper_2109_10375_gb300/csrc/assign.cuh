@@ -86,10 +86,10 @@ struct ScanArgs {
   const float* linb;
 };
 
-// Arguments of the thresholds kernel (one CTA per matching).
+// Arguments of the thresholds kernel.
 struct ThreshArgs {
-  unsigned long long* total;             // exact mass total (2 x u64), formed here from tile_mass if given
-  const unsigned long long* tile_mass;   // per-sort-tile partial sums or null
+  unsigned long long* total;             // exact mass total (2 x u64), read when tile_mass is null
+  const unsigned long long* tile_mass;   // per-sort-tile partial sums (16-byte aligned) or null
   int64_t ntiles;
   int M;                                 // table points
   double a_w, b_w, c_w, z_lo, z_hi;
@@ -122,6 +122,7 @@ struct ScatterArgs {
 // scan look-back states must be zeroed beforehand.
 struct AssignMulti {
   int M;
+  int max_table;  // largest table of the items
   const ThreshArgs* thresh;
   const ScanArgs* scan[2];
   const uint32_t* scan_prefix[2];
