@@ -572,13 +572,12 @@ static LptWork lpt_work(amber_ctx* c, int n) {
   const Plan& p = c->plan;
   LptWork w{};
   // three half spectra (4 + 16/n bytes per cell each): the transform buffer
-  // and the key and index ping-pong pairs (8 bytes per cell each); two fields
-  // in the mass pair
+  // and the key and index ping-pong pairs (8 bytes per cell each); a field in
+  // the first mass array
   w.H0 = c->ws + p.off_spec;
   w.H1 = c->sortw.keysA;
   w.H2 = c->sortw.idxA;
   w.F0 = c->sortw.massA;
-  w.F1 = c->sortw.massB;
   w.acc = reinterpret_cast<double*>(c->ws + p.off_pow);
   w.tw = c->ws + p.off_tw32 + p.tw32_off[ilog2i(n)];
   w.status = c->status;

@@ -19,6 +19,8 @@
 
 #include <cuda.h>  // CUtensorMap (the z pass's TMA descriptor)
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "keys.cuh"
 
@@ -122,12 +124,19 @@ enum { PASS_FWD = 0, PASS_INV = 1, PASS_CONV = 2 };
 #ifndef AMBER_YPASS_MINB
 #define AMBER_YPASS_MINB 2
 #endif
-template <typename T, int N, int MODE, int V = 0, bool OOP = false, bool MULTI = false>
+// OP (FP32, z pass only): a spectral operator fused into the pass.  kLoad: the
+// tile is not read from H but formed by op from its own spectra, with a table
+// it first fills in shared memory after the tile; kFilter: the
+// multiply of PASS_CONV is op's window instead of the radiation kernel.
+struct NoOp {
+  static constexpr bool kLoad = false, kFilter = false;
+};
+template <typename T, int N, int MODE, int V = 0, bool OOP = false, bool MULTI = false, class OP = NoOp>
 __global__ void __launch_bounds__(strided_threads<N, V>(), MODE == PASS_CONV ? AMBER_ZPASS_MINB : AMBER_YPASS_MINB)
 k_fft_strided(cpx<T>* __restrict__ H, int64_t elem_stride, int64_t outer_stride, int ncol,
               int ntx, const cpx<T>* __restrict__ tw, T kf, T l_mfp, T norm,
               const cpx<T>* __restrict__ Hin = nullptr, int64_t item_stride = 0,
-              const T* __restrict__ kp = nullptr) {
+              const T* __restrict__ kp = nullptr, const OP op = OP()) {
   using C = FftCfg<N, V>;
   using L = StridedSmem<T, N, V>;
   constexpr int R0 = C::R0, R1 = C::R1, E = C::E, SB = C::SB, NT = strided_threads<N, V>();
@@ -150,23 +159,42 @@ k_fft_strided(cpx<T>* __restrict__ H, int64_t elem_stride, int64_t outer_stride,
   const cpx<T>* ibase = OOP ? Hin + (int64_t)outer * outer_stride + kx0 : base;
 
   cpx<T> v[E];
+  if constexpr (OP::kLoad) {
+    op.template fill<N, SB, NT>(sm + L::elems, tid, kx0, outer);
+    __syncthreads();
+  }
   // ---- forward stage A: radix R0 over n = j + r N/R0, read from global
 #pragma unroll
   for (int q = 0; q < QA; ++q) {
     const int id = tid + q * NT;
     const int b = id % SB, j = id / SB;
     const bool ok = kx0 + b < ncol;
+    if constexpr (OP::kLoad) {
+      op.template load<N, SB, R0>(v + q * R0, sm + L::elems, ok, kx0 + b, b, outer,
+                                  (int64_t)outer * outer_stride + kx0 + b, elem_stride, j);
+    } else {
 #pragma unroll
-    for (int r = 0; r < R0; ++r) {
-      const int n = j + r * (N / R0);
-      v[q * R0 + r] = ok ? ibase[(int64_t)n * elem_stride + b] : mk<T>(0, 0);
+      for (int r = 0; r < R0; ++r) {
+        const int n = j + r * (N / R0);
+        v[q * R0 + r] = ok ? ibase[(int64_t)n * elem_stride + b] : mk<T>(0, 0);
+      }
     }
   }
   if constexpr (MODE == PASS_CONV) {
     // K(|k|)/n^3 of this tile's columns for |kz| = 0..N/2, into shared memory
     // after the tile, while the loads are in flight
-    tile_kernel<T, N, SB, NT>(reinterpret_cast<T*>(sm + L::elems), kx0, signed_freq(outer, N), tid, kf, l_mfp,
-                              norm);
+    if constexpr (OP::kFilter) {
+      T* Kt = reinterpret_cast<T*>(sm + L::elems);
+      const int my = signed_freq(outer, N);
+#pragma unroll 1
+      for (int i = tid; i < (N / 2 + 1) * SB; i += NT) {
+        const int kza = i / SB, kx = kx0 + (i - kza * SB);
+        Kt[i] = op.window(kx * kx + my * my + kza * kza) * norm;
+      }
+    } else {
+      tile_kernel<T, N, SB, NT>(reinterpret_cast<T*>(sm + L::elems), kx0, signed_freq(outer, N), tid, kf, l_mfp,
+                                norm);
+    }
     if constexpr (R1 == 1) __syncthreads();
   }
 #pragma unroll
@@ -585,11 +613,16 @@ k_fft_r2c_x(const T* __restrict__ src, cpx<T>* __restrict__ H, int64_t nrows, in
 // HIST (FP32): the intensities' raw 32-bit sort keys are also counted into
 // krange's histogram, four 8-bit digit positions, so a sort of raw keys with
 // 8-bit digits needs no histogram pass of its own.
-template <typename T, int N, int V = 0, bool MULTI = false, bool HIST = false>
+// EPI: what becomes of a value (store it and fold its key range in, or an
+// operation fused into the pass, see fft_ops.cuh; J may then be read too).
+struct EpiKeys {
+  static constexpr bool kKeys = true;
+};
+template <typename T, int N, int V = 0, bool MULTI = false, bool HIST = false, class EPI = EpiKeys>
 __global__ void __launch_bounds__(xpass_threads<N, V>())
 k_fft_c2r_x(const cpx<T>* __restrict__ H, T* __restrict__ J, int64_t nrows, int RS,
             const cpx<T>* __restrict__ tw, unsigned int* __restrict__ status, SortCtrl* __restrict__ krange,
-            int64_t rpi = 0) {
+            int64_t rpi = 0, const EPI epi = EPI()) {
   using C = FftCfg<N, V>;
   using L = XSmem<T, N, V>;
   using K = typename KeyOf<T>::K;
@@ -680,21 +713,46 @@ k_fft_c2r_x(const cpx<T>* __restrict__ H, T* __restrict__ J, int64_t nrows, int 
       }
     }
   };
+  // outputs of one butterfly: v[i] goes to element n0 + i step of rows ra, ra + 1
+  auto emit = [&](const cpx<T>* w, int64_t ra, int n0, auto count, int step) {
+    constexpr int R = decltype(count)::value;
+    if constexpr (EPI::kKeys) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int n = n0 + r * step;
+        J[ra * N + n] = w[r].x;
+        J[(ra + 1) * N + n] = w[r].y;
+        track(w[r].x);
+        track(w[r].y);
+      }
+    } else {
+      // four elements of both rows at a time: the operation's loads, then its stores
+      constexpr int G = R < 4 ? R : 4;
+#pragma unroll
+      for (int r0 = 0; r0 < R; r0 += G) {
+        typename EPI::Aux aux[2 * G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          aux[2 * g] = epi.fetch(J, ra * N + n0 + (r0 + g) * step);
+          aux[2 * g + 1] = epi.fetch(J, (ra + 1) * N + n0 + (r0 + g) * step);
+        }
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          const int n = n0 + (r0 + g) * step;
+          bad |= !isfinite(w[r0 + g].x) || !isfinite(w[r0 + g].y);
+          J[ra * N + n] = epi.value(aux[2 * g], w[r0 + g].x);
+          J[(ra + 1) * N + n] = epi.value(aux[2 * g + 1], w[r0 + g].y);
+        }
+      }
+    }
+  };
   if constexpr (R1 == 1) {
 #pragma unroll
     for (int q = 0; q < QA; ++q) {
       const int id = tid + q * NT;
       const int p = id / (N / R0);
       const int64_t ra = row0 + 2 * p;
-      if (ra + 1 < nrows) {
-#pragma unroll
-        for (int r = 0; r < R0; ++r) {
-          J[ra * N + r] = v[q * R0 + r].x;
-          J[(ra + 1) * N + r] = v[q * R0 + r].y;
-          track(v[q * R0 + r].x);
-          track(v[q * R0 + r].y);
-        }
-      }
+      if (ra + 1 < nrows) emit(v + q * R0, ra, 0, std::integral_constant<int, R0>{}, 1);
     }
   } else {
     __syncthreads();
@@ -718,21 +776,13 @@ k_fft_c2r_x(const cpx<T>* __restrict__ H, T* __restrict__ J, int64_t nrows, int 
       }
       dft<R1, true>(v + q * R1);
       const int64_t ra = row0 + 2 * p;
-      if (ra + 1 < nrows) {
-#pragma unroll
-        for (int r = 0; r < R1; ++r) {
-          const int n = j + r * R0;
-          J[ra * N + n] = v[q * R1 + r].x;
-          J[(ra + 1) * N + n] = v[q * R1 + r].y;
-          track(v[q * R1 + r].x);
-          track(v[q * R1 + r].y);
-        }
-      }
+      if (ra + 1 < nrows) emit(v + q * R1, ra, j, std::integral_constant<int, R1>{}, R0);
     }
   }
   if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) raise_status(status, AMBER_ERR_NONFINITE);
   // fold the intensities' key range into the sort's control block
-  if constexpr (MULTI) key_range_commit(klo, khi, krange + row0 / rpi);
+  if constexpr (!EPI::kKeys) return;
+  else if constexpr (MULTI) key_range_commit(klo, khi, krange + row0 / rpi);
   else if (krange) key_range_commit(klo, khi, krange);
   if constexpr (HIST) {
     __syncthreads();
@@ -945,34 +995,6 @@ cudaError_t source_spectrum_n(const T* src, cpx<T>* H, const cpx<T>* tw, cudaStr
   k_fft_strided<T, N, PASS_FWD, V><<<sgrid, strided_threads<N, V>(), ss, s>>>(H, RS, (int64_t)N * RS, ncol, ntx, tw,
                                                                            zero, zero, zero);
   prof_end(prof, PK_FFT_Y_FWD, s);
-  return cudaGetLastError();
-}
-
-// Inverse transform only: out = unnormalised inverse DFT of the half spectrum
-// H (z and y passes in place, then the C2R x-pass into out); the caller folds
-// 1/n^3 into the spectrum.  A non-finite output latches AMBER_ERR_NONFINITE.
-template <typename T, int N>
-cudaError_t inverse_spectrum_n(cpx<T>* H, T* out, const cpx<T>* tw, unsigned int* status, cudaStream_t s) {
-  using C = FftCfg<N>;
-  const int RS = N / 2 + 2;
-  const int ncol = N / 2 + 1;
-  const int64_t nrows = (int64_t)N * N;
-  const size_t xs = XSmem<T, N>::elems * sizeof(cpx<T>);
-  const size_t ss = StridedSmem<T, N>::elems * sizeof(cpx<T>);
-  static std::atomic<unsigned long long> attr_done{0};  // per instantiation and device
-  if (first_use_on_device(attr_done)) {
-    cudaFuncSetAttribute(k_fft_c2r_x<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xs);
-    cudaFuncSetAttribute(k_fft_strided<T, N, PASS_INV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
-  }
-  const int xgrid = (int)((nrows / 2 + C::XP - 1) / C::XP);
-  const int ntx = (ncol + C::SB - 1) / C::SB;
-  const int sgrid = N * ntx;
-  const T zero = (T)0;
-  k_fft_strided<T, N, PASS_INV><<<sgrid, strided_threads<N>(), ss, s>>>(H, (int64_t)N * RS, RS, ncol, ntx, tw,
-                                                                       zero, zero, zero);
-  k_fft_strided<T, N, PASS_INV><<<sgrid, strided_threads<N>(), ss, s>>>(H, RS, (int64_t)N * RS, ncol, ntx, tw,
-                                                                       zero, zero, zero);
-  k_fft_c2r_x<T, N><<<xgrid, xpass_threads<N>(), xs, s>>>(H, out, nrows, RS, tw, status, nullptr);
   return cudaGetLastError();
 }
 

@@ -8,20 +8,18 @@
 namespace amber {
 
 // Buffers a call may use: three half spectra (H0..H2, each n^2 (n/2 + 2)
-// complex floats) and two real n^3 float fields (F0, F1), plus one double.
+// complex floats) and a real n^3 float field (F0), plus one double.
 struct LptWork {
   void* H0;
   void* H1;
   void* H2;
   float* F0;
-  float* F1;
   double* acc;
   const void* tw;  // FP32 twiddles of this n
   unsigned int* status;
   int num_sms;
 };
 
-cudaError_t inverse_spectrum_f32(int n, void* H, float* out, const void* tw, unsigned int* status, cudaStream_t s);
 cudaError_t forward_spectrum_f32(int n, const float* src, void* H, const void* tw, cudaStream_t s);
 cudaError_t sum_f64_impl(const float* x, int64_t n, double* acc, int num_sms, cudaStream_t s);
 
