@@ -2,7 +2,7 @@
 // interlace and Wofk; Sec. 3.3, Eq. fcoll).
 //
 //   k_assign<P>   : NGP / CIC / TSC assignment of one particle per lattice
-//                   point (FP32 atomics on the mesh)
+//                   point (FP32 sums, in any order)
 //   k_scale_mesh  : plain assignment's normalisation
 //
 // The operators on spectra (second derivatives, inverse gradients, filters,
@@ -11,65 +11,258 @@
 #include <cmath>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "fft_ops.cuh"
 #include "lpt.cuh"
 
 namespace amber {
 
-__device__ __forceinline__ int wrap(int v, int n) {
-  v %= n;
-  return v < 0 ? v + n : v;
+// Window of order P of a particle at pos (cells) on one axis: the first mesh
+// point it reaches and its P weights.  The nearest mesh point is
+// floor(pos + 1/2), d = pos - that point in [-1/2, 1/2).
+template <int P> __device__ __forceinline__ int window(float pos, float w[P]) {
+  const float b = floorf(pos + 0.5f);
+  const float d = pos - b;
+  if constexpr (P == 1) {
+    w[0] = 1.f;
+    return (int)b;
+  } else if constexpr (P == 2) {
+    const float ad = fabsf(d);
+    w[0] = d < 0.f ? ad : 1.f - ad;
+    w[1] = d < 0.f ? 1.f - ad : ad;
+    return d < 0.f ? (int)b - 1 : (int)b;
+  } else {
+    w[0] = 0.5f * (0.5f - d) * (0.5f - d);
+    w[1] = 0.75f - d * d;
+    w[2] = 0.5f * (0.5f + d) * (0.5f + d);
+    return (int)b - 1;
+  }
 }
 
-// One particle per thread: lattice point (ix, iy, iz) displaced by psi
-// (box units, inv_dx cells per unit) plus `shift` cells on every axis; the
-// nearest mesh point is floor(pos + 1/2), d = pos - that point in [-1/2, 1/2).
+// Straight to the mesh: one global atomic per mesh point the particle reaches
+// (n is a power of two, so a coordinate wraps by its low bits).
 template <int P>
-__global__ void __launch_bounds__(256) k_assign(const float* __restrict__ px, const float* __restrict__ py,
-                                                const float* __restrict__ pz, const float* __restrict__ mass, int n,
-                                                float inv_dx, float shift, float* __restrict__ mesh) {
-  const int64_t np = (int64_t)n * n * n;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x) {
-    const int ix = (int)(i % n), iy = (int)((i / n) % n), iz = (int)(i / ((int64_t)n * n));
+__device__ __forceinline__ void deposit_global(float* __restrict__ mesh, const float pos[3], float m, int n) {
+  float w[3][P];
+  int b[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) b[a] = window<P>(pos[a], w[a]);
+  const unsigned mask = (unsigned)n - 1u;
+#pragma unroll
+  for (int oz = 0; oz < P; ++oz) {
+    const int64_t zo = (int64_t)(((unsigned)b[2] + oz) & mask) * n;
+#pragma unroll
+    for (int oy = 0; oy < P; ++oy) {
+      float* row = mesh + (zo + (((unsigned)b[1] + oy) & mask)) * n;
+      const float wzy = m * w[2][oz] * w[1][oy];
+#pragma unroll
+      for (int ox = 0; ox < P; ++ox) atomicAdd(&row[((unsigned)b[0] + ox) & mask], wzy * w[0][ox]);
+    }
+  }
+}
+
+// Grids below one block: one particle per thread; lattice point (ix, iy, iz)
+// displaced by psi (box units, inv_dx cells per unit) plus `shift` cells on
+// every axis.
+template <int P>
+__global__ void __launch_bounds__(256) k_assign_small(const float* __restrict__ px, const float* __restrict__ py,
+                                                      const float* __restrict__ pz, const float* __restrict__ mass,
+                                                      int n, int lg, float inv_dx, float shift,
+                                                      float* __restrict__ mesh) {
+  const int np = n * n * n;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < np; i += gridDim.x * blockDim.x) {
+    const int ix = i & (n - 1), iy = (i >> lg) & (n - 1), iz = i >> (2 * lg);
     const float pos[3] = {ix + px[i] * inv_dx + shift, iy + py[i] * inv_dx + shift, iz + pz[i] * inv_dx + shift};
-    int base[3];
-    float w[3][3];  // offsets -1, 0, +1
+    deposit_global<P>(mesh, pos, mass ? mass[i] : 1.0f, n);
+  }
+}
+
+// A CTA takes a block of 32 x 8 x 8 lattice points (lanes along x, 8 y and two
+// halves of z over the warps, four z per thread).  Neighbouring particles stay
+// neighbours, so the mesh points the block reaches fit a box of 2-4 points per
+// particle: its sums are formed there, in shared memory, and each box point
+// goes to the mesh with one coalesced global atomic.  Global atomics for every
+// window point, 27 per particle for TSC, were bound by the packets they send to
+// L2 (two 512^3 TSC meshes 9.84 ms); float atomics in shared memory are a
+// compare-and-swap loop here (9.7 wavefronts per warp, 9.28 ms).  Integer ones
+// take 2, so the box holds two 32-bit fixed-point words per point: with S the
+// power of two that brings the block's mass total M below 2^30, a contribution
+// c adds round(c S) to the first and the rest, in units of 2^-20 / S, to the
+// second.  No sum can overflow (|c| adds up to at most M; 2048 rests of at most
+// 1/2), and the resolution, 2^-50 M, is below float's 2^-24 of any point above
+// 2^-26 M.  Particles of equal mass need one word where no mesh point is the
+// nearest of more than 8 of them (counted first): a point then sums to at most
+// 8 (CIC; 5.4 for TSC) times that count, so a resolution of 2^-25 or finer
+// fits, under float's own rounding of a mean density of 1.  A block whose box does not fit, or whose total is 0, not finite or
+// out of the scale's range, deposits straight to the mesh.  Both meshes of an
+// interlaced density (the second's particles half a cell on) come from one
+// read of psi.  Two 512^3 TSC meshes now take 4.00 ms (5.40 with two words),
+// two weighted 256^3 CIC ones 0.2 instead of 1.2; bound by the shared-memory
+// pipe (69 % busy; 83 % with two words).
+constexpr int kAsgX = 32, kAsgY = 8, kAsgZ = 8, kAsgPer = 4;
+constexpr int kAsgThreads = kAsgX * kAsgY * kAsgZ / kAsgPer;
+constexpr int kAsgBox = 14000;  // mesh points a block's box may hold (two CTAs per SM)
+
+template <int P>
+__global__ void __launch_bounds__(kAsgThreads, 2)
+    k_assign(const float* __restrict__ px, const float* __restrict__ py, const float* __restrict__ pz,
+             const float* __restrict__ mass, int n, float inv_dx, float* __restrict__ mesh0,
+             float* __restrict__ mesh1) {
+  constexpr int NW = kAsgThreads / 32;
+  extern __shared__ __align__(16) int box_hi[];  // [kAsgBox], then the second words
+  int* box_lo = box_hi + kAsgBox;
+  __shared__ int s_lo[3][NW], s_hi[3][NW];
+  __shared__ float s_mass[NW];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nx = n / kAsgX, ny = n / kAsgY;
+  const int bx = blockIdx.x % nx, by = (blockIdx.x / nx) % ny, bz = blockIdx.x / (nx * ny);
+  const int ix = bx * kAsgX + lane, iy = by * kAsgY + (warp & 7), iz0 = bz * kAsgZ + (warp >> 3) * kAsgPer;
+  float pos[kAsgPer][3], m[kAsgPer];
+#pragma unroll
+  for (int q = 0; q < kAsgPer; ++q) {
+    const int64_t i = ((int64_t)(iz0 + q) * n + iy) * n + ix;
+    pos[q][0] = px[i];
+    pos[q][1] = py[i];
+    pos[q][2] = pz[i];
+    m[q] = mass ? mass[i] : 1.0f;
+  }
+  float msum = 0.f;
+#pragma unroll
+  for (int q = 0; q < kAsgPer; ++q) {
+    pos[q][0] = ix + pos[q][0] * inv_dx;
+    pos[q][1] = iy + pos[q][1] * inv_dx;
+    pos[q][2] = iz0 + q + pos[q][2] * inv_dx;
+    // a position that is not finite makes the sum NaN (straight to the mesh)
+    msum += fabsf(m[q]) + 0.f * (pos[q][0] + pos[q][1] + pos[q][2]);
+  }
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) msum += __shfl_xor_sync(0xffffffffu, msum, o);
+  if (lane == 0) s_mass[warp] = msum;
+  float scale = 0.f, unscale = 0.f;
+  for (int pass = 0; pass < 2; ++pass) {
+    float* __restrict__ mesh = pass ? mesh1 : mesh0;
+    if (!mesh) break;
+    const float shift = pass ? 0.5f : 0.f;
+    // the box of mesh points the block's windows reach
+    int ext[3], org[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const float b = floorf(pos[a] + 0.5f);
-      const float d = pos[a] - b;
-      base[a] = (int)b;
-      if (P == 1) {
-        w[a][0] = 0.f; w[a][1] = 1.f; w[a][2] = 0.f;
-      } else if (P == 2) {
-        const float ad = fabsf(d);
-        w[a][1] = 1.f - ad;
-        w[a][0] = d < 0.f ? ad : 0.f;
-        w[a][2] = d >= 0.f ? ad : 0.f;
-      } else {
-        w[a][0] = 0.5f * (0.5f - d) * (0.5f - d);
-        w[a][1] = 0.75f - d * d;
-        w[a][2] = 0.5f * (0.5f + d) * (0.5f + d);
+      int lo = 0x7fffffff, hi = -0x7fffffff;
+#pragma unroll
+      for (int q = 0; q < kAsgPer; ++q) {
+        float w[P];
+        const int b = window<P>(pos[q][a] + shift, w);
+        lo = min(lo, b);
+        hi = max(hi, b);
+      }
+      lo = __reduce_min_sync(0xffffffffu, lo);
+      hi = __reduce_max_sync(0xffffffffu, hi);
+      if (lane == 0) {
+        s_lo[a][warp] = lo;
+        s_hi[a][warp] = hi;
       }
     }
-    const float m = mass ? mass[i] : 1.0f;
+    __syncthreads();
+    if (pass == 0) {
+      float t = s_mass[lane % NW];  // NW = 16: every sum twice
 #pragma unroll
-    for (int oz = 0; oz < 3; ++oz) {
-      if (w[2][oz] == 0.f) continue;
-      const int64_t zo = (int64_t)wrap(base[2] + oz - 1, n) * n * n;
+      for (int o = NW / 2; o >= 1; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      // t < 2^(e - 126) (one more bit for the rounding of this sum)
+      const int e = (__float_as_int(t) >> 23) + 1;
+      if (t > 0.f && e > 40 && e < 250 && 30 - (e - 126) < 120) {
+        scale = __int_as_float((127 + 30 - (e - 126)) << 23);
+        unscale = __int_as_float((127 - 30 + (e - 126)) << 23);
+      }
+    }
+    bool fits = scale != 0.f;
 #pragma unroll
-      for (int oy = 0; oy < 3; ++oy) {
-        if (w[1][oy] == 0.f) continue;
-        const int64_t yo = zo + (int64_t)wrap(base[1] + oy - 1, n) * n;
-        const float wzy = m * w[2][oz] * w[1][oy];
+    for (int a = 0; a < 3; ++a) {
+      org[a] = __reduce_min_sync(0xffffffffu, s_lo[a][lane % NW]);
+      const int hi = __reduce_max_sync(0xffffffffu, s_hi[a][lane % NW]);
+      // (float: the spread of far-flung particles can exceed an int)
+      fits = fits && (float)hi - (float)org[a] < 256.f;
+      ext[a] = fits ? hi - org[a] + P : 0;
+    }
+    const int plane = ext[0] * ext[1], cells = plane * ext[2];
+    if (!fits || cells > kAsgBox) {  // the same on every thread
+#pragma unroll 1
+      for (int q = 0; q < kAsgPer; ++q) {
+        const float at[3] = {pos[q][0] + shift, pos[q][1] + shift, pos[q][2] + shift};
+        deposit_global<P>(mesh, at, m[q], n);
+      }
+      __syncthreads();  // s_lo, s_hi are read
+      continue;
+    }
+    for (int c = tid * 4; c < cells; c += kAsgThreads * 4) {
+      *reinterpret_cast<int4*>(box_hi + c) = make_int4(0, 0, 0, 0);
+      *reinterpret_cast<int4*>(box_lo + c) = make_int4(0, 0, 0, 0);
+    }
+    __syncthreads();
+    float one = 0.f;  // the scale of a single word, or 0: two words
+    if (!mass) {
 #pragma unroll
-        for (int ox = 0; ox < 3; ++ox) {
-          if (w[0][ox] == 0.f) continue;
-          atomicAdd(&mesh[yo + wrap(base[0] + ox - 1, n)], wzy * w[0][ox]);
+      for (int q = 0; q < kAsgPer; ++q) {
+        int b[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) b[a] = (int)floorf(pos[q][a] + shift + 0.5f) - org[a];
+        atomicAdd(box_lo + b[2] * plane + b[1] * ext[0] + b[0], 1);
+      }
+      __syncthreads();
+      int most = 0;
+      for (int c = tid * 4; c < cells; c += kAsgThreads * 4) {
+        int4* at = reinterpret_cast<int4*>(box_lo + c);
+        const int4 v = *at;
+        most = max(most, max(max(v.x, v.y), max(v.z, v.w)));
+        *at = make_int4(0, 0, 0, 0);
+      }
+      if (!__syncthreads_or(most > 8)) one = __syncthreads_or(most > 4) ? 33554432.f : 67108864.f;  // 2^25, 2^26
+    }
+    auto deposit = [&](auto words) {
+#pragma unroll
+      for (int q = 0; q < kAsgPer; ++q) {
+        float w[3][P];
+        int b[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) b[a] = window<P>(pos[q][a] + shift, w[a]) - org[a];
+        const float ms = decltype(words)::value == 1 ? one : m[q] * scale;
+        int* at = box_hi + b[2] * plane + b[1] * ext[0] + b[0];
+#pragma unroll
+        for (int oz = 0; oz < P; ++oz) {
+#pragma unroll
+          for (int oy = 0; oy < P; ++oy) {
+            const float wzy = ms * w[2][oz] * w[1][oy];
+            int* row = at + oz * plane + oy * ext[0];
+#pragma unroll
+            for (int ox = 0; ox < P; ++ox) {
+              const float c = wzy * w[0][ox];
+              const int h = __float2int_rn(c);
+              atomicAdd(row + ox, h);
+              if (decltype(words)::value == 2)
+                atomicAdd(row + ox + kAsgBox, __float2int_rn((c - (float)h) * 1048576.f));
+            }
+          }
         }
       }
+    };
+    if (one != 0.f) deposit(std::integral_constant<int, 1>{});
+    else deposit(std::integral_constant<int, 2>{});
+    __syncthreads();
+    const float back = one != 0.f ? 1.f / one : unscale;
+    const unsigned mask = (unsigned)n - 1u;
+    const unsigned mx = 0xffffffffu / (unsigned)ext[0] + 1u, my = 0xffffffffu / (unsigned)ext[1] + 1u;
+    for (int c = tid; c < cells; c += kAsgThreads) {
+      const int l = box_lo[c], h = box_hi[c] + (l >> 20);
+      const float v = ((float)h + (float)(l & 0xfffff) * 9.5367431640625e-7f) * back;
+      if (v != 0.f) {
+        // c = (z ext1 + y) ext0 + x; the reciprocals are exact for c < 2^16
+        const unsigned yz = ext[0] == 1 ? (unsigned)c : __umulhi((unsigned)c, mx), x = c - yz * ext[0];
+        const unsigned z = ext[1] == 1 ? yz : __umulhi(yz, my), y = yz - z * ext[1];
+        const unsigned gx = (org[0] + x) & mask, gy = (org[1] + y) & mask, gz = (org[2] + z) & mask;
+        atomicAdd(&mesh[((int64_t)gz * n + gy) * n + gx], v);
+      }
     }
+    __syncthreads();  // the box is read: the next mesh may use it
   }
 }
 
@@ -118,17 +311,38 @@ cudaError_t lpt_impl(const LptWork& w, int n, double box, double D1, double D2, 
   return e;
 }
 
-static cudaError_t assign(int order, int n, double box, float shift, const float* px, const float* py,
-                          const float* pz, const float* mass, float* mesh, int num_sms, cudaStream_t s) {
+template <int P>
+static cudaError_t assign_p(int n, float inv_dx, const float* px, const float* py, const float* pz, const float* mass,
+                            float* mesh0, float* mesh1, int num_sms, cudaStream_t s) {
   const int64_t n3 = (int64_t)n * n * n;
-  cudaError_t e = cudaMemsetAsync(mesh, 0, (size_t)n3 * sizeof(float), s);
+  if (n >= kAsgX) {
+    constexpr size_t smem = 2 * kAsgBox * sizeof(int);
+    static std::atomic<unsigned long long> attr{0};  // per instantiation and device
+    if (first_use_on_device(attr))
+      cudaFuncSetAttribute(k_assign<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k_assign<P><<<(unsigned)(n3 / (kAsgX * kAsgY * kAsgZ)), kAsgThreads, smem, s>>>(px, py, pz, mass, n, inv_dx, mesh0, mesh1);
+  } else {
+    int lg = 0;
+    while ((1 << lg) < n) ++lg;
+    for (int pass = 0; pass < 2; ++pass)
+      if (pass ? mesh1 : mesh0)
+        k_assign_small<P><<<grid_of(n3, num_sms), 256, 0, s>>>(px, py, pz, mass, n, lg, inv_dx, pass ? 0.5f : 0.f,
+                                                               pass ? mesh1 : mesh0);
+  }
+  return cudaGetLastError();
+}
+
+// mesh0 (and mesh1, shifted by half a cell, unless null) = sums of the masses
+static cudaError_t assign(int order, int n, double box, const float* px, const float* py, const float* pz,
+                          const float* mass, float* mesh0, float* mesh1, int num_sms, cudaStream_t s) {
+  const size_t bytes = (size_t)n * n * n * sizeof(float);
+  cudaError_t e = cudaMemsetAsync(mesh0, 0, bytes, s);
+  if (e == cudaSuccess && mesh1) e = cudaMemsetAsync(mesh1, 0, bytes, s);
   if (e != cudaSuccess) return e;
   const float inv_dx = (float)(n / box);
-  const int g = grid_of(n3, num_sms);
-  if (order == 1) k_assign<1><<<g, 256, 0, s>>>(px, py, pz, mass, n, inv_dx, shift, mesh);
-  else if (order == 2) k_assign<2><<<g, 256, 0, s>>>(px, py, pz, mass, n, inv_dx, shift, mesh);
-  else k_assign<3><<<g, 256, 0, s>>>(px, py, pz, mass, n, inv_dx, shift, mesh);
-  return cudaGetLastError();
+  if (order == 1) return assign_p<1>(n, inv_dx, px, py, pz, mass, mesh0, mesh1, num_sms, s);
+  if (order == 2) return assign_p<2>(n, inv_dx, px, py, pz, mass, mesh0, mesh1, num_sms, s);
+  return assign_p<3>(n, inv_dx, px, py, pz, mass, mesh0, mesh1, num_sms, s);
 }
 
 cudaError_t mesh_impl(const LptWork& w, int n, double box, int order, bool interlace, const float* psi_x,
@@ -141,14 +355,14 @@ cudaError_t mesh_impl(const LptWork& w, int n, double box, int order, bool inter
     k_set_total<<<1, 1, 0, s>>>(w.acc, (double)n3);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = assign(order, n, box, 0.f, psi_x, psi_y, psi_z, mass, rho, w.num_sms, s);
+  if (e == cudaSuccess)
+    e = assign(order, n, box, psi_x, psi_y, psi_z, mass, rho, interlace ? w.F0 : nullptr, w.num_sms, s);
   if (e != cudaSuccess) return e;
   if (!interlace) {
     k_scale_mesh<<<grid_of(n3, w.num_sms), 256, 0, s>>>(rho, n3, w.acc);
     return cudaGetLastError();
   }
-  e = assign(order, n, box, 0.5f, psi_x, psi_y, psi_z, mass, w.F0, w.num_sms, s);
-  if (e == cudaSuccess) e = forward_spectrum_f32(n, rho, w.H0, w.tw, s);
+  e = forward_spectrum_f32(n, rho, w.H0, w.tw, s);
   if (e == cudaSuccess) e = forward_spectrum_f32(n, w.F0, w.H1, w.tw, s);
   if (e == cudaSuccess) {
     // 1/total: mean 1 and the inverse transform's 1/n^3 together

@@ -65,3 +65,36 @@ def test_interlaced_density_vs_oracle(B, n, order):
     ref = O.interlace_deconvolve(O.mesh_assign(p64, m64, box, order), O.mesh_assign(p64, m64, box, order, 0.5), box,
                                  order)
     _close(got, ref)
+
+
+@pytest.mark.parametrize("order", [1, 2, 3])
+@pytest.mark.parametrize("kind", ["smooth", "clump", "far", "light"])
+def test_density_block_forms_vs_oracle(B, order, kind):
+    # a block's sums in one fixed-point word (equal masses, few particles per
+    # point), in two (a clump; masses over nine decades), or straight to the
+    # mesh (particles flung so far that the block's box does not fit)
+    n = 32
+    g = np.random.default_rng(7 * order + len(kind))
+    box = 1.0 * n
+    lo, hi = (0.05, 0.45) if order == 1 else (-1.4, 1.4)
+    psi = g.uniform(lo, hi, (3, n, n, n))
+    mass = None
+    if kind == "clump":  # every particle of an 8^3 region onto one cell
+        q = np.stack(np.meshgrid(*(np.arange(n),) * 3, indexing="ij")[::-1])
+        inside = np.all((q >= 8) & (q < 16), axis=0)
+        psi = np.where(inside, 11.2 - q, psi)
+    elif kind == "far":
+        psi = psi + g.integers(-n // 2, n // 2, (3, n, n, n))
+    elif kind == "light":
+        mass = (10.0 ** g.uniform(-9, 0, (n, n, n))).astype(np.float32)
+    psi = psi.astype(np.float32)
+    with B.Context(n ** 3) as ctx:
+        got = ctx.mesh_density(tuple(_t(p) for p in psi), box, order, False, mass=None if mass is None else _t(mass))
+        assert ctx.sync_status() == 0
+    ref = O.mesh_assign(list(psi.astype(np.float64)), None if mass is None else mass.astype(np.float64), box, order)
+    # FP32 positions up to 2 n cells: windows good to a few 1e-6 of a particle
+    _close(got, ref, 2e-5)
+    if kind == "light":  # every mesh point to FP32 accuracy, not only the heavy ones
+        r = got.double().cpu().numpy()
+        live = ref > 1e-7 * ref.max()
+        assert np.max(np.abs(r - ref)[live] / ref[live]) < 1e-3
