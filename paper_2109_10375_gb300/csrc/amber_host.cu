@@ -35,7 +35,7 @@ cudaError_t radiation_field_multi_f32(int n, int variant, const float* const* sr
                                       SortCtrl* kranges);
 cudaError_t radiation_field_f64(int n, const double* src, double* J, void* H, const void* tw, double box,
                                double l_mfp, unsigned int* status, cudaStream_t s, FftProfile* prof,
-                               SortCtrl* krange);
+                               SortCtrl* krange, double* ktable);  // ktable: kernel_table_size(n) values of scratch
 
 // ---------------------------------------------------------------------------
 // Per-kernel timing: a pool of events recorded around launches.
@@ -177,7 +177,7 @@ struct Plan {
   int n32 = 0, n64 = 0;
   int64_t cells64 = 0;
   size_t off_spec, off_keysA, off_keysB, off_idxA, off_idxB, off_massA, off_massB, off_lb, off_sctrl, off_actrl, off_X, off_invdx, off_lin,
-      off_state, off_btab, off_tilemass, off_status, off_srcsum, off_pow, off_tw32, off_tw64, total;
+      off_state, off_btab, off_tilemass, off_status, off_srcsum, off_pow, off_ktab, off_tw32, off_tw64, total;
   size_t tw32_off[11] = {}, tw64_off[11] = {};
 };
 
@@ -215,6 +215,7 @@ static Plan make_plan(int64_t max_cells) {
   p.off_status = take(256);
   p.off_srcsum = take(256);
   p.off_pow = take((size_t)kPowerAcc * kMaxPowerBins * sizeof(double));
+  p.off_ktab = take(p.n64 ? (size_t)kernel_table_size(p.n64) * sizeof(double) : 0);
   size_t tw32 = 0, tw64 = 0;
   for (int l = 2, n = 4; n <= 1024; ++l, n *= 2) {
     if (n <= p.n32) { p.tw32_off[l] = tw32; tw32 += align256((size_t)n * 8); }
@@ -496,7 +497,8 @@ int amber_radiation_field_f64(amber_ctx* c, const double* d_src, int n, double b
   const Plan& p = c->plan;
   const int l = ilog2i(n);
   return cuda_status(radiation_field_f64(n, d_src, d_J, c->ws + p.off_spec, c->ws + p.off_tw64 + p.tw64_off[l], box,
-                                         l_mfp, c->status, s, &c->prof, nullptr));
+                                         l_mfp, c->status, s, &c->prof, nullptr,
+                                         reinterpret_cast<double*>(c->ws + p.off_ktab)));
 }
 
 int amber_power_bins(int n, int* nbins) {
@@ -1392,7 +1394,8 @@ int amber_solve_f64(amber_ctx* c, const double* d_src, const float* d_mass, cons
   cudaError_t e = sort_ctrl_reset(c->sortw.ctrl, s);
   if (e == cudaSuccess)
     e = radiation_field_f64(n, d_src, J, c->ws + pl.off_spec, c->ws + pl.off_tw64 + pl.tw64_off[ilog2i(n)], p->box,
-                           p->l_mfp, c->status, s, &c->prof, c->sortw.ctrl);
+                           p->l_mfp, c->status, s, &c->prof, c->sortw.ctrl,
+                           reinterpret_cast<double*>(c->ws + pl.off_ktab));
   unsigned long long* tile_mass = reinterpret_cast<unsigned long long*>(c->ws + pl.off_tilemass);
   if (e == cudaSuccess)
     e = rank_impl<double>(c->sortw, J, C, nullptr, d_mass, nullptr, tile_mass, true, c->status, s, &c->prof,

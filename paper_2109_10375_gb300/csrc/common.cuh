@@ -113,6 +113,10 @@ __device__ __forceinline__ void dft(cpx<T>* v) {
   }
 }
 
+// NaN or infinite, by the exponent bits (no FP64 comparison)
+__device__ __forceinline__ bool not_finite(float x) { return (__float_as_uint(x) & 0x7f800000u) == 0x7f800000u; }
+__device__ __forceinline__ bool not_finite(double x) { return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000; }
+
 // True the first time it is called with a given device current (per flag):
 // kernel attributes such as the dynamic shared-memory limit are set per device.
 inline bool first_use_on_device(std::atomic<unsigned long long>& mask) {

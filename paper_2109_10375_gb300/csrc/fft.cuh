@@ -93,15 +93,28 @@ __device__ __forceinline__ int sm_count() {
 __device__ __forceinline__ int signed_freq(int m, int n) { return m < n / 2 ? m : m - n; }
 
 // K(|k|)/n^3 of one tile's columns kx0 .. kx0 + SB - 1 at ky for |kz| = 0..n/2
-// into Kt (row |kz|, column b).  Evaluated per tile while the tile's loads
-// are in flight: a table over |k|^2 read from L2 was measured slower.
+// into Kt (row |kz|, column b).  FP32: evaluated per tile while the tile's
+// loads are in flight (a table over |k|^2 read from L2 was measured slower).
+// FP64: read from such a table (k_kernel_table): the arctangent, division and
+// square root of half a value per element kept the narrow FP64 pipe busier than
+// the transforms (z pass at 256^3 1.36 ms, 0.94 with the table).
 template <typename T, int N, int SB, int NT>
-__device__ __forceinline__ void tile_kernel(T* Kt, int kx0, int ky, int tid, T kf, T l_mfp, T norm) {
+__device__ __forceinline__ void tile_kernel(T* Kt, int kx0, int ky, int tid, T kf, T l_mfp, T norm,
+                                            const T* __restrict__ table = nullptr) {
 #pragma unroll 1
   for (int i = tid; i < (N / 2 + 1) * SB; i += NT) {
-    const int kza = i / SB, kx = kx0 + (i - kza * SB);
-    Kt[i] = kernel_K<T>((T)(kx * kx + ky * ky + kza * kza), l_mfp, kf, norm);
+    const int kza = i / SB, kx = kx0 + (i - kza * SB), k2 = kx * kx + ky * ky + kza * kza;
+    if constexpr (sizeof(T) == 8) Kt[i] = kx <= N / 2 ? table[k2] : (T)0;
+    else Kt[i] = kernel_K<T>((T)k2, l_mfp, kf, norm);
   }
+}
+
+// K(|k|) norm for |k|^2 = 0 .. 3 (n/2)^2 in lattice units
+constexpr int kernel_table_size(int n) { return 3 * (n / 2) * (n / 2) + 1; }
+template <typename T>
+__global__ void __launch_bounds__(64) k_kernel_table(T* __restrict__ table, int count, T kf, T l_mfp, T norm) {
+  const int i = blockIdx.x * 64 + threadIdx.x;
+  if (i < count) table[i] = kernel_K<T>((T)i, l_mfp, kf, norm);
 }
 
 // ---------------------------------------------------------------------------
@@ -116,6 +129,7 @@ enum { PASS_FWD = 0, PASS_INV = 1, PASS_CONV = 2 };
 // MULTI (z-pass only): several transforms of size N back to back, item_stride
 // elements apart; line family `outer` of the launch is line y = outer % N of
 // item outer / N, whose box and l_mfp give kp[2 item] = kf, kp[2 item + 1] = l.
+// FP64: kp is the table of the kernel over |k|^2 (k_kernel_table).
 // CTAs per SM the strided passes are compiled for (build-time tunables): two
 // keep 128 registers per thread at 256 threads.
 #ifndef AMBER_ZPASS_MINB
@@ -193,7 +207,7 @@ k_fft_strided(cpx<T>* __restrict__ H, int64_t elem_stride, int64_t outer_stride,
       }
     } else {
       tile_kernel<T, N, SB, NT>(reinterpret_cast<T*>(sm + L::elems), kx0, signed_freq(outer, N), tid, kf, l_mfp,
-                                norm);
+                                norm, kp);
     }
     if constexpr (R1 == 1) __syncthreads();
   }
@@ -595,7 +609,8 @@ k_fft_r2c_x(const T* __restrict__ src, cpx<T>* __restrict__ H, int64_t nrows, in
     if (ra + 1 >= nrows) continue;
     const cpx<T> zk = sm[L::pos(p, k)];
     const cpx<T> zn = sm[L::pos(p, (N - k) & (N - 1))];
-    const T h = (T)0.5;
+    // FP64: the halves are left to the z pass's normalisation (exact powers of two)
+    const T h = sizeof(T) == 8 ? (T)1 : (T)0.5;
     const cpx<T> A = mk<T>(h * (zk.x + zn.x), h * (zk.y - zn.y));
     const cpx<T> B = mk<T>(h * (zk.y + zn.y), h * (zn.x - zk.x));
     H[ra * RS + k] = A;
@@ -689,7 +704,7 @@ k_fft_c2r_x(const cpx<T>* __restrict__ H, T* __restrict__ J, int64_t nrows, int 
     __syncthreads();
   }
   auto track = [&](T x) {
-    bad |= !isfinite(x);
+    bad |= not_finite(x);
     const K kk = enc_desc(x, nan);
     klo = kk < klo ? kk : klo;
     khi = kk > khi ? kk : khi;
@@ -739,7 +754,7 @@ k_fft_c2r_x(const cpx<T>* __restrict__ H, T* __restrict__ J, int64_t nrows, int 
 #pragma unroll
         for (int g = 0; g < G; ++g) {
           const int n = n0 + (r0 + g) * step;
-          bad |= !isfinite(w[r0 + g].x) || !isfinite(w[r0 + g].y);
+          bad |= not_finite(w[r0 + g].x) || not_finite(w[r0 + g].y);
           J[ra * N + n] = epi.value(aux[2 * g], w[r0 + g].x);
           J[(ra + 1) * N + n] = epi.value(aux[2 * g + 1], w[r0 + g].y);
         }
@@ -810,16 +825,19 @@ enum ProfKind {
 // pass reads it, leaving it unchanged.
 // hist8 (FP32, krange given): the inverse x pass also counts the raw keys'
 // four 8-bit digits into krange's histogram.
+// ktable (FP64): kernel_table_size(N) values of scratch.
 template <typename T, int N, int V = 0>
 cudaError_t radiation_field_n(const T* src, T* J, cpx<T>* H, const cpx<T>* tw, double box, double l_mfp,
                               unsigned int* status, cudaStream_t s, FftProfile* prof, SortCtrl* krange,
-                              const cpx<T>* spec_in = nullptr, bool hist8 = false, bool tma = false) {
+                              const cpx<T>* spec_in = nullptr, bool hist8 = false, bool tma = false,
+                              T* ktable = nullptr) {
   using C = FftCfg<N, V>;
   const int RS = N / 2 + 2;
   const int ncol = N / 2 + 1;
   const int64_t nrows = (int64_t)N * N;
   const T kf = (T)(2.0 * 3.14159265358979323846 / box);
-  const T norm = (T)(1.0 / ((double)N * N * N));
+  // FP64: with the factor 1/2 of the real-to-complex split (k_fft_r2c_x)
+  const T norm = (T)((sizeof(T) == 8 ? 0.5 : 1.0) / ((double)N * N * N));
   const size_t xs = XSmem<T, N, V>::elems * sizeof(cpx<T>);
   const size_t ss = StridedSmem<T, N, V>::elems * sizeof(cpx<T>);
   // the z pass adds its table of K over |kz| = 0..N/2 for the tile's columns
@@ -852,6 +870,8 @@ cudaError_t radiation_field_n(const T* src, T* J, cpx<T>* H, const cpx<T>* tw, d
   }
   // z-pass: lines (y, kx); element stride N*RS; outer (y) stride RS
   prof_begin(prof, PK_FFT_Z_CONV, s);
+  if constexpr (sizeof(T) == 8)
+    k_kernel_table<T><<<(kernel_table_size(N) + 63) / 64, 64, 0, s>>>(ktable, kernel_table_size(N), kf, (T)l_mfp, norm);
   bool z_done = false;
   if constexpr (sizeof(T) == 4 && C::R1 > 1) {
     CUtensorMap map;
@@ -875,7 +895,7 @@ cudaError_t radiation_field_n(const T* src, T* J, cpx<T>* H, const cpx<T>* tw, d
         H, (int64_t)N * RS, RS, ncol, ntx, tw, kf, (T)l_mfp, norm, spec_in);
   else
     k_fft_strided<T, N, PASS_CONV, V><<<sgrid, strided_threads<N, V>(), sc, s>>>(
-        H, (int64_t)N * RS, RS, ncol, ntx, tw, kf, (T)l_mfp, norm);
+        H, (int64_t)N * RS, RS, ncol, ntx, tw, kf, (T)l_mfp, norm, nullptr, 0, ktable);
   prof_end(prof, PK_FFT_Z_CONV, s);
   prof_begin(prof, PK_FFT_Y_INV, s);
   k_fft_strided<T, N, PASS_INV, V><<<sgrid, strided_threads<N, V>(), ss, s>>>(H, RS, (int64_t)N * RS, ncol, ntx, tw,

@@ -23,10 +23,12 @@ __device__ __forceinline__ uint32_t enc_desc(float v, bool& bad) {
   const uint32_t u = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
   return ~u;
 }
+// (integer tests: each comparison or addition of doubles would take 16 cycles
+// of the narrow FP64 pipe per warp)
 __device__ __forceinline__ uint64_t enc_desc(double v, bool& bad) {
-  bad |= isnan(v);
-  v = v + 0.0;
-  const uint64_t b = (uint64_t)__double_as_longlong(v);
+  uint64_t b = (uint64_t)__double_as_longlong(v);
+  bad |= (b << 1) > 0xffe0000000000000ull;  // NaN
+  if ((b << 1) == 0) b = 0;                 // -0 -> +0
   const uint64_t u = (b & 0x8000000000000000ull) ? ~b : (b | 0x8000000000000000ull);
   return ~u;
 }

@@ -94,12 +94,12 @@ __global__ void __launch_bounds__(256) k_assign_small(const float* __restrict__ 
 // 2^-26 M.  Particles of equal mass need one word where no mesh point is the
 // nearest of more than 8 of them (counted first): a point then sums to at most
 // 8 (CIC; 5.4 for TSC) times that count, so a resolution of 2^-25 or finer
-// fits, under float's own rounding of a mean density of 1.  A block whose box does not fit, or whose total is 0, not finite or
-// out of the scale's range, deposits straight to the mesh.  Both meshes of an
-// interlaced density (the second's particles half a cell on) come from one
-// read of psi.  Two 512^3 TSC meshes now take 4.00 ms (5.40 with two words),
-// two weighted 256^3 CIC ones 0.2 instead of 1.2; bound by the shared-memory
-// pipe (69 % busy; 83 % with two words).
+// fits, under float's own rounding of a mean density of 1.  A block whose box
+// does not fit, or whose total is 0, not finite or out of the scale's range, or
+// that has a position that is not finite, deposits straight to the mesh.  Both
+// meshes of an interlaced density (the second's particles half a cell on) come
+// from one read of psi.  Two 512^3 TSC meshes now take 4.00 ms (5.40 with two
+// words), bound by the shared-memory pipe (69 % busy; 83 % with two words).
 constexpr int kAsgX = 32, kAsgY = 8, kAsgZ = 8, kAsgPer = 4;
 constexpr int kAsgThreads = kAsgX * kAsgY * kAsgZ / kAsgPer;
 constexpr int kAsgBox = 14000;  // mesh points a block's box may hold (two CTAs per SM)
