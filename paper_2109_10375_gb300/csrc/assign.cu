@@ -21,9 +21,11 @@
 // 2^-s, so F_n is off by at most n 2^-60 (1e-9 at 2^30 cells), and no sum
 // depends on the order of addition.  Only the interpolation weight is FP32.
 #include <cstdlib>
+#include <type_traits>
 
 #include "assign.cuh"
 #include "fixed128.cuh"
+#include "scan.cuh"
 #include "sort.cuh"
 
 namespace amber {
@@ -230,87 +232,16 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresholds_multi(const Thres
 }
 
 // ---------------------------------------------------------------------------
-// Cell mass in the scan's 64-bit fixed point: floor(m 2^s), s chosen per call
-// by k_thresholds so the total stays below 2^62.  Each cell loses less than
-// 2^-s, so over n cells F_n is off by less than n 2^-s / T <= n 2^-62 (2e-10
-// relative at 2^30 cells) -- far inside an FP64 running sum's own error.
-// scale = 2^s: scaling by a power of two is exact, so this is floor_u64 of
-// m 2^s (below 2^62 for every valid mass, since m <= T); masses the total pass
-// flagged count as 0.
-__device__ __forceinline__ unsigned long long mass_fix(float m, float scale) {
-  return (m >= 0.0f && m < 1099511627776.0f) ? floor_u64(m * scale) : 0ull;
-}
-
-// u64 -> float from its two 32-bit halves (within two roundings; only the
-// interpolation weight uses it)
-__device__ __forceinline__ float u64_to_float(unsigned long long x) {
-  return fmaf(__uint2float_rn((uint32_t)(x >> 32)), 4294967296.0f, __uint2float_rn((uint32_t)x));
-}
-
-// Look-back word of a scan tile: 2 flag bits over a 62-bit prefix.
-constexpr unsigned long long kScanAgg = 1ull << 62;
-constexpr unsigned long long kScanInc = 2ull << 62;
-constexpr unsigned long long kScanMask = 3ull << 62;
-constexpr unsigned long long kScanValue = (1ull << 62) - 1ull;
-
-__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-// One round of a warp-wide 32-ary search for c = #{j : X_j >= v} (X
-// non-increasing), c known to lie in [lo, hi]: lane k probes lo + k step; the
-// probes that hold form a prefix, and the range shrinks below step.
-__device__ __forceinline__ void count_ge_round(const unsigned long long* __restrict__ X, unsigned long long v,
-                                               int& lo, int& hi, int lane) {
-  if (lo >= hi) return;  // warp-uniform
-  const int step = (hi - lo + 31) >> 5;
-  const int q = lo + lane * step;
-  const bool t = q < hi && X[q] >= v;
-  const int c = __popc(__ballot_sync(0xffffffffu, t));
-  const int nlo = c ? lo + (c - 1) * step + 1 : lo;
-  const int nhi = min(hi, lo + c * step);
-  lo = nlo;
-  hi = nhi;
-}
-
-constexpr int kScanWin = 64;  // thresholds one tile may span, staged in shared memory
-
-// LIN: a linear weighting (growth or volume).  The exact-integer threshold
-// test of the mass weighting is replaced by the margins h_j(n) in FP32: a
-// cell takes the largest table point j with h_j >= 0.  A margin is linear in
-// (n, M_n), so its extremes over the box that a run of ranks spans lie at the
-// corners.  Per tile every point is classified: jall is the largest one that
-// ionizes all of its cells, jtop the largest one that can ionize any.  From
-// jtop each warp walks down 32 points at a time to the first one its own box
-// allows, each thread from there to the first one its 16 ranks allow, and only
-// then each cell tests margins.  (The first tile of 128^3 spans over 1000 of
-// 2000 points; with every cell testing all of the tile's points it took 1.06 ms.)
-template <bool GATHER, bool WANT_F, bool LIN>
+template <bool GATHER, bool WANT_F, bool LIN, bool DIRECT>
 __device__ __forceinline__ void scan_assign_body(const ScanArgs& a) {
   constexpr int NT = kScanThreads, IT = kScanItems, TILE = kScanTile;
-  __shared__ int s_jall, s_jtop;
   __shared__ uint32_t sord[TILE + TILE / 32];
   __shared__ float smass[TILE + TILE / 32];
-  __shared__ unsigned long long wtot[NT / 32];
-  __shared__ unsigned long long s_excl;
   __shared__ uint32_t s_tile;
-  __shared__ int s_cx[3];  // c(M_last), c(M_first), first staged threshold (-1: none)
-  __shared__ unsigned long long sX[kScanWin];
-  __shared__ float sInv[kScanWin];
-  __shared__ uint32_t scnt[kMaxBuckets];
-  __shared__ uint32_t soff[kMaxBuckets + 1];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) {
-    s_tile = atomicAdd(a.ticket, 1u);
-    s_jall = -1;
-    s_jtop = -1;
-  }
-  for (int b = tid; b < a.nbuckets; b += NT) scnt[b] = 0;
+  __shared__ ScanShared S;
+  const int tid = threadIdx.x;
+  if (tid == 0) s_tile = atomicAdd(a.ticket, 1u);
+  scan_clear<NT>(S, a.nbuckets);
   __syncthreads();
   const uint32_t tile = s_tile;
   // n <= 2^30: positions fit 32 bits
@@ -330,7 +261,6 @@ __device__ __forceinline__ void scan_assign_body(const ScanArgs& a) {
     }
   }
   const float qs = __int_as_float((127 + *a.qshift) << 23);  // 2^s, s in [-2, 64]
-  const int M = a.n_table;
 
   // order (and rank-order masses): coalesced striped loads -> padded shared
   // memory -> a blocked run of IT consecutive ranks per thread
@@ -352,360 +282,14 @@ __device__ __forceinline__ void scan_assign_body(const ScanArgs& a) {
     if (p < cnt) mv[i] = GATHER ? mass[cell[i]] : smass[p + (p >> 5)];
     run += mass_fix(mv[i], qs);
   }
-  // block exclusive scan of the thread totals
-  unsigned long long x = run;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) wtot[warp] = x;
-  __syncthreads();
-  unsigned long long wpre = 0, tile_sum = 0;
-#pragma unroll
-  for (int w = 0; w < NT / 32; ++w) {
-    if (w < warp) wpre += wtot[w];
-    tile_sum += wtot[w];
-  }
-  const unsigned long long thr_excl = wpre + x - run;
-
-  // warp 0 publishes the tile's aggregate and starts its look-back load; the
-  // bucket slots of every cell (which need no prefix) are taken meanwhile
-  unsigned long long lbw = 0;
-  int64_t lbt = (int64_t)tile - 1;
-  if (warp == 0) {
-    if (lane == 0) st_relaxed_u64(a.state + tile, (tile == 0 ? kScanInc : kScanAgg) | tile_sum);
-    lbw = (lbt - lane >= 0) ? ld_relaxed_u64(a.state + lbt - lane) : kScanInc;
-  }
-  uint32_t slot[IT];
-  if (a.nbuckets <= 16) {
-    // few buckets (small grids: one below 2^23 cells): most lanes share one,
-    // and one shared add per lane would serialise on its counter; the lanes
-    // of a bucket take their slots with one add for the warp
-    const unsigned lt = (1u << lane) - 1u;
-#pragma unroll
-    for (int i = 0; i < IT; ++i) {
-      const bool ok = tid * IT + i < cnt;
-      const unsigned bk = ok ? cell[i] >> a.bucket_shift : 0xffffu;
-      const unsigned peers = __match_any_sync(0xffffffffu, bk);
-      const int leader = __ffs(peers) - 1;
-      uint32_t base = 0;
-      if (ok && lane == leader) base = atomicAdd(&scnt[bk], (uint32_t)__popc(peers));
-      base = __shfl_sync(0xffffffffu, base, leader);
-      slot[i] = ok ? base + (uint32_t)__popc(peers & lt) : 0xffffffffu;
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < IT; ++i)
-      slot[i] = (tid * IT + i < cnt) ? atomicAdd(&scnt[cell[i] >> a.bucket_shift], 1u) : 0xffffffffu;
-  }
-  __syncthreads();
-
-  if (warp == 0) {
-    // decoupled look-back: each lane holds one predecessor's word, so a round
-    // trip covers 32 tiles; aggregates are summed back to the nearest
-    // inclusive prefix
-    unsigned long long excl = 0;
-    unsigned spins = 0;
-    while (true) {
-      const unsigned long long f = lbw & kScanMask;
-      const unsigned inc_mask = __ballot_sync(0xffffffffu, f == kScanInc);
-      const unsigned stop_mask = inc_mask | __ballot_sync(0xffffffffu, f == 0ull);
-      const int first = stop_mask ? __ffs(stop_mask) - 1 : 32;
-      const bool found = first < 32 && ((inc_mask >> first) & 1u);
-      unsigned long long part = (lane < first || (found && lane == first)) ? (lbw & kScanValue) : 0ull;
-#pragma unroll
-      for (int o = 16; o >= 1; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
-      excl += __shfl_sync(0xffffffffu, part, 0);
-      if (found) break;
-      lbt -= first;
-      if (first < 32) {
-        if (++spins >= a.spin_limit) {
-          if (lane == 0) raise_status(a.status, AMBER_ERR_DEVICE_TIMEOUT);
-          break;
-        }
-        __nanosleep(20);
-      }
-      lbw = (lbt - lane >= 0) ? ld_relaxed_u64(a.state + lbt - lane) : kScanInc;
-    }
-    if (lane == 0) {
-      if (tile != 0) st_relaxed_u64(a.state + tile, kScanInc | ((excl + tile_sum) & kScanValue));
-      s_excl = excl;
-    }
-    // bracket the whole tile: c(M) = #{j : X_j >= M} at its first and last
-    // prefix, both searched at once (three round trips for 2000 thresholds)
-    int lo0 = 0, hi0 = LIN ? 0 : M, lo1 = 0, hi1 = LIN ? 0 : M;
-    while (lo0 < hi0 || lo1 < hi1) {
-      count_ge_round(a.Xq, excl, lo0, hi0, lane);
-      count_ge_round(a.Xq, excl + tile_sum, lo1, hi1, lane);
-    }
-    // thresholds the tile's cells can touch: X_j for j in [c_last - 1, c_first]
-    const int base = max(lo1 - 1, 0), L = min(lo0, M - 1) - base + 1;
-    const bool stage = !LIN && L <= kScanWin;
-    if (stage) {
-      for (int i = lane; i < L; i += 32) {
-        sX[i] = a.Xq[base + i];
-        sInv[i] = (base + i < M - 1) ? a.inv_dx[base + i] : 0.0f;
-      }
-    }
-    if (lane == 0) {
-      s_cx[0] = lo1;
-      s_cx[1] = lo0;
-      s_cx[2] = stage ? base : -1;
-    }
-  } else if (warp == 1) {
-    // tile-local bucket starts (exclusive scan over the buckets) and this
-    // tile's row of the offset table
-    uint32_t carry = 0;
-    uint16_t* row = a.btab + (int64_t)tile * (a.nbuckets + 1);
-    for (int b0 = 0; b0 < a.nbuckets; b0 += 32) {
-      const int b = b0 + lane;
-      const uint32_t c = b < a.nbuckets ? scnt[b] : 0u;
-      uint32_t y = c;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t z = __shfl_up_sync(0xffffffffu, y, o);
-        if (lane >= o) y += z;
-      }
-      if (b < a.nbuckets) {
-        soff[b] = carry + y - c;
-        row[b] = (uint16_t)(carry + y - c);
-      }
-      carry += __shfl_sync(0xffffffffu, y, 31);
-    }
-    if (lane == 0) {
-      soff[a.nbuckets] = carry;
-      row[a.nbuckets] = (uint16_t)carry;
-    }
-  }
-  __syncthreads();
-  unsigned long long Mn = s_excl + thr_excl;
-  const double invT = WANT_F ? 1.0 / (double)*a.qtotal : 0.0;
-  const float qinv = __int_as_float((127 - *a.qshift) << 23);  // 2^-s: fixed point -> mass units
-  const unsigned long long qT = LIN ? *a.qtotal : 0ull;  // total in the prefix's fixed point (>= every M_n)
-  // head form (ranks in the first half) or tail form, for the tile's box:
-  // h = C_j + sa alpha_j u + sa beta_j v with (C, u, v, sa) = (x W_N, n, M_n, -1)
-  // or ((x - 1) W_N, N - n, T - M_n, +1)
-  const bool head = start + (uint32_t)cnt / 2u <= n / 2u;
-  const float* linC = head ? a.linP : a.linQ;
-  const float sa = head ? -1.0f : 1.0f;
-  // table point j over the box of ranks (r0, r1] (from 0) with prefix masses
-  // in [m0, m1]: bounds of its margin and the rounding they are good to
-  struct Box { float u0, u1, v0, v1; };
-  auto box_of = [&](uint32_t r0, uint32_t r1, unsigned long long m0, unsigned long long m1) -> Box {
-    if (head) return {(float)(r0 + 1u), (float)r1, u64_to_float(m0) * qinv, u64_to_float(m1) * qinv};
-    return {(float)(n - r1), (float)(n - (r0 + 1u)), u64_to_float(qT - m1) * qinv, u64_to_float(qT - m0) * qinv};
-  };
-  auto classify = [&](const Box& x, int j, float& hmin, float& hmax, float& tol) {
-    const float Cj = linC[j], al = sa * a.lina[j], be = sa * a.linb[j];
-    const float au0 = al * x.u0, au1 = al * x.u1, bv0 = be * x.v0, bv1 = be * x.v1;
-    hmin = Cj + fminf(au0, au1) + fminf(bv0, bv1);
-    hmax = Cj + fmaxf(au0, au1) + fmaxf(bv0, bv1);
-    tol = 4e-7f * (fabsf(Cj) + fmaxf(fabsf(au0), fabsf(au1)) + fmaxf(fabsf(bv0), fabsf(bv1)));
-  };
-  if constexpr (LIN) {
-    const Box tb = box_of(start, start + (uint32_t)cnt, s_excl, s_excl + tile_sum);
-    int ja = -1, jt = -1;
-    for (int j = tid; j < M; j += NT) {
-      float hmin, hmax, tol;
-      classify(tb, j, hmin, hmax, tol);
-      if (hmin >= tol) ja = j;
-      if (hmax >= -tol) jt = j;
-    }
-    ja = __reduce_max_sync(0xffffffffu, ja);
-    jt = __reduce_max_sync(0xffffffffu, jt);
-    if (lane == 0) {
-      if (ja >= 0) atomicMax(&s_jall, ja);
-      if (jt >= 0) atomicMax(&s_jtop, jt);
-    }
-    __syncthreads();
-  }
-  const int cx_lo = s_cx[0], cx_hi = s_cx[1], wb = s_cx[2];
-  // threshold j from the staged window when the tile fits it
-  auto Xj = [&](int j) -> unsigned long long { return wb >= 0 ? sX[j - wb] : a.Xq[j]; };
-  auto Ij = [&](int j) -> float { return wb >= 0 ? sInv[j - wb] : a.inv_dx[j]; };
-
-  // bracket: cx = #{j : X_j >= M_n}; X is non-increasing in j and M_n grows
-  // with rank, so each thread searches the tile's range once, then walks
-  // down.  Each (cell, z) goes straight to its bucket-ordered staging slot
-  // (order and masses were consumed above, so their shared arrays are free).
-  uint32_t* scell = sord;
-  float* sz = smass;
-  if (LIN && s_jtop <= s_jall) {
-    // no table point above max{j : all ionized} can ionize any cell of the
-    // tile: every cell takes j* = jall, whose two margin rows are held in
-    // registers
-    const int js = s_jall;
-    const bool mid = js >= 0 && js < M - 1;
-    float la0 = 0.f, lb0 = 0.f, P0 = 0.f, Q0 = 0.f, la1 = 0.f, lb1 = 0.f, P1 = 0.f, Q1 = 0.f;
-    if (mid) {
-      la0 = a.lina[js], lb0 = a.linb[js], P0 = a.linP[js], Q0 = a.linQ[js];
-      la1 = a.lina[js + 1], lb1 = a.linb[js + 1], P1 = a.linP[js + 1], Q1 = a.linQ[js + 1];
-    }
-    const float zc = js < 0 ? a.z_lo : a.z_hi;
-#pragma unroll
-    for (int i = 0; i < IT; ++i) {
-      const int p = tid * IT + i;
-      if (p >= cnt) continue;
-      Mn += mass_fix(mv[i], qs);
-      float z = zc;
-      if (mid) {
-        const uint32_t rank1 = start + (uint32_t)p + 1u;
-        const bool chead = rank1 <= n / 2u;
-        const float cs = chead ? -1.0f : 1.0f;
-        const float uu = cs * (chead ? (float)rank1 : (float)(n - rank1));
-        const float vv = cs * (chead ? u64_to_float(Mn) * qinv : u64_to_float(qT - Mn) * qinv);
-        const float h0 = fmaf(lb0, vv, fmaf(la0, uu, chead ? P0 : Q0));
-        const float h1 = fmaf(lb1, vv, fmaf(la1, uu, chead ? P1 : Q1));
-        float t = h0 / (h0 - h1);
-        t = fminf(fmaxf(t, 0.0f), 0.99999994f);
-        z = a.z_lo + ((float)js + t) * a.dzt;
-      }
-      if (WANT_F) a.F[start + p] = (double)Mn * invT;
-      const uint32_t q = soff[cell[i] >> a.bucket_shift] + slot[i];
-      scell[q + (q >> 5)] = cell[i];
-      sz[q + (q >> 5)] = z;
-    }
-  } else if (!LIN && cx_lo == cx_hi) {
-    // the whole tile between two thresholds (all but a few tiles): one
-    // interval, its threshold and slope held in registers
-    const int j = cx_lo - 1;
-    const bool mid = j >= 0 && j < M - 1;
-    const unsigned long long Xu = mid ? Xj(j) : 0ull;
-    const float Iu = mid ? Ij(j) : 0.0f;
-    const float zc = j < 0 ? a.z_lo : a.z_hi;
-#pragma unroll
-    for (int i = 0; i < IT; ++i) {
-      const int p = tid * IT + i;
-      if (p >= cnt) continue;
-      Mn += mass_fix(mv[i], qs);
-      float z = zc;
-      if (mid) {
-        float t = u64_to_float(Xu - Mn) * Iu;
-        t = fminf(fmaxf(t, 0.0f), 0.99999994f);
-        z = a.z_lo + ((float)j + t) * a.dzt;
-      }
-      if (WANT_F) a.F[start + p] = (double)Mn * invT;
-      const uint32_t q = soff[cell[i] >> a.bucket_shift] + slot[i];
-      scell[q + (q >> 5)] = cell[i];
-      sz[q + (q >> 5)] = z;
-    }
-  } else if constexpr (LIN) {
-    const int jall = s_jall;
-    int jt = s_jtop;
-    {
-      // the warp's ranks: 32 points per round from the top down
-      const uint32_t w0 = start + (uint32_t)min(warp * 32 * IT, cnt), w1 = start + (uint32_t)min((warp + 1) * 32 * IT, cnt);
-      const Box wbx = box_of(w0, w1, s_excl + wpre, s_excl + wpre + wtot[warp]);
-      unsigned hit = 0;
-      if (w1 > w0) {
-        for (; jt > jall; jt -= 32) {
-          const int j = jt - lane;
-          float hmin, hmax = -1.f, tol = 0.f;
-          if (j > jall) classify(wbx, j, hmin, hmax, tol);
-          hit = __ballot_sync(0xffffffffu, j > jall && hmax >= -tol);
-          if (hit) break;
-        }
-      }
-      jt = hit ? jt - (__ffs(hit) - 1) : jall;
-    }
-    if (tid * IT < cnt) {
-      const Box cb = box_of(start + (uint32_t)(tid * IT), start + (uint32_t)min((tid + 1) * IT, cnt), Mn, Mn + run);
-      for (; jt > jall; --jt) {
-        float hmin, hmax, tol;
-        classify(cb, jt, hmin, hmax, tol);
-        if (hmax >= -tol) break;
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < IT; ++i) {
-      const int p = tid * IT + i;
-      if (p >= cnt) continue;
-      Mn += mass_fix(mv[i], qs);
-      // the cell's own form (a tile can straddle the middle rank; the boxes'
-      // classification above carries a tolerance for either form)
-      const uint32_t rank1 = start + (uint32_t)p + 1u;
-      const bool chead = rank1 <= n / 2u;
-      const float cs = chead ? -1.0f : 1.0f;
-      const float* cC = chead ? a.linP : a.linQ;
-      const float uu = cs * (chead ? (float)rank1 : (float)(n - rank1));
-      const float vv = cs * (chead ? u64_to_float(Mn) * qinv : u64_to_float(qT - Mn) * qinv);
-      auto h = [&](int j) { return fmaf(a.linb[j], vv, fmaf(a.lina[j], uu, cC[j])); };
-      int js = jt;
-      while (js > jall && !(h(js) >= 0.0f)) --js;
-      float z;
-      if (js < 0) z = a.z_lo;
-      else if (js == M - 1) z = a.z_hi;
-      else {
-        const float h0 = h(js), h1 = h(js + 1);
-        float t = h0 / (h0 - h1);
-        t = fminf(fmaxf(t, 0.0f), 0.99999994f);
-        z = a.z_lo + ((float)js + t) * a.dzt;
-      }
-      if (WANT_F) a.F[start + p] = (double)Mn * invT;
-      const uint32_t q = soff[cell[i] >> a.bucket_shift] + slot[i];
-      scell[q + (q >> 5)] = cell[i];
-      sz[q + (q >> 5)] = z;
-    }
-  } else {
-    int cx = -1;
-#pragma unroll
-    for (int i = 0; i < IT; ++i) {
-      const int p = tid * IT + i;
-      if (p >= cnt) continue;
-      Mn += mass_fix(mv[i], qs);
-      int lo = cx_lo, hi = cx_hi;
-      if (cx >= 0) {
-        // the prefix grew: gallop down from the last cell's bracket (in a
-        // small grid's first tile neighbours lie hundreds of points apart, and
-        // stepping through them one dependent load at a time took 63 us at 32^3)
-        hi = cx;
-        lo = cx;
-        for (int step = 1; lo > cx_lo; step *= 2) {
-          const int q = max(lo - step, cx_lo);
-          if (Xj(q) >= Mn) {
-            lo = q + 1;
-            break;
-          }
-          hi = lo = q;
-        }
-      }
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (Xj(mid) >= Mn) lo = mid + 1; else hi = mid;
-      }
-      cx = lo;
-      const int j = cx - 1;
-      float z;
-      if (j < 0) z = a.z_lo;
-      else if (j == M - 1) z = a.z_hi;
-      else {
-        float t = u64_to_float(Xj(j) - Mn) * Ij(j);
-        t = fminf(fmaxf(t, 0.0f), 0.99999994f);
-        z = a.z_lo + ((float)j + t) * a.dzt;
-      }
-      if (WANT_F) a.F[start + p] = (double)Mn * invT;
-      const uint32_t q = soff[cell[i] >> a.bucket_shift] + slot[i];
-      scell[q + (q >> 5)] = cell[i];
-      sz[q + (q >> 5)] = z;
-    }
-  }
-  __syncthreads();
-  // the pairs are read back only after the whole scan: keep them out of L2
-  const unsigned long long pol = l2_evict_first();
-#pragma unroll
-  for (int k = 0; k < IT; ++k) {
-    const int p = k * NT + tid;
-    if (p < cnt) {
-      st_hint(a.bcell + start + p, scell[p + (p >> 5)], pol);
-      st_hint(a.bz + start + p, sz[p + (p >> 5)], pol);
-    }
-  }
+  LookBack lb;
+  scan_tile<NT, IT, true, false, DIRECT, WANT_F, LIN>(a, S, lb, tile, start, cnt, cell, mv, run, qs, sord, smass, a.bcell,
+                                              a.bz);
 }
 
-template <bool GATHER, bool WANT_F, bool LIN>
+template <bool GATHER, bool WANT_F, bool LIN, bool DIRECT>
 __global__ void __launch_bounds__(kScanThreads, AMBER_SCAN_MINB) k_scan_assign(const ScanArgs a) {
-  scan_assign_body<GATHER, WANT_F, LIN>(a);
+  scan_assign_body<GATHER, WANT_F, LIN, DIRECT>(a);
 }
 
 // Several matchings at once: CTA b works on item find_item(prefix, M, b) (the
@@ -716,7 +300,7 @@ __global__ void __launch_bounds__(kScanThreads, AMBER_SCAN_MINB)
   __shared__ ScanArgs sa;
   if (threadIdx.x == 0) sa = args[find_item(prefix, M, blockIdx.x)];
   __syncthreads();
-  scan_assign_body<false, false, LIN>(sa);
+  scan_assign_body<false, false, LIN, false>(sa);
 }
 
 // z_re[cell] = z, bucket after bucket: CTA (bucket b, tile group g) copies
@@ -904,6 +488,7 @@ void assign_args(const AssignWork& w, const uint32_t* order, const float* mass, 
   a.state = w.state;
   a.ticket = ticket;
   bucket_plan(n, &a.nbuckets, &a.bucket_shift);
+  a.zre = nullptr;
   a.bcell = w.bcell;
   a.bz = w.bz;
   a.btab = w.btab;
@@ -928,6 +513,11 @@ void assign_args(const AssignWork& w, const uint32_t* order, const float* mass, 
   const int tiles_per_cta = kBackTilesPerCta / x.wpt;
   x.groups = (int)((tiles + tiles_per_cta - 1) / tiles_per_cta);
   x.zre = zre;
+}
+
+template <typename A, typename B> static bool disjoint(const A* a, int64_t na, const B* b, int64_t nb) {
+  return !b || reinterpret_cast<uintptr_t>(a + na) <= reinterpret_cast<uintptr_t>(b) ||
+         reinterpret_cast<uintptr_t>(b + nb) <= reinterpret_cast<uintptr_t>(a);
 }
 
 cudaError_t assign_impl(const AssignWork& w, const uint32_t* order, const float* mass, bool mass_in_rank_order,
@@ -964,18 +554,36 @@ cudaError_t assign_impl(const AssignWork& w, const uint32_t* order, const float*
   prof_begin(prof, PK_SCAN_ASSIGN, s);
   const unsigned g = (unsigned)tiles;
   const bool gather = !mass_in_rank_order, lin = hc.weighting != AMBER_WEIGHT_MASS;
-  const int v = (gather ? 4 : 0) | (F ? 2 : 0) | (lin ? 1 : 0);
-  switch (v) {
-    case 0: k_scan_assign<false, false, false><<<g, kScanThreads, 0, s>>>(a); break;
-    case 1: k_scan_assign<false, false, true><<<g, kScanThreads, 0, s>>>(a); break;
-    case 2: k_scan_assign<false, true, false><<<g, kScanThreads, 0, s>>>(a); break;
-    case 3: k_scan_assign<false, true, true><<<g, kScanThreads, 0, s>>>(a); break;
-    case 4: k_scan_assign<true, false, false><<<g, kScanThreads, 0, s>>>(a); break;
-    case 5: k_scan_assign<true, false, true><<<g, kScanThreads, 0, s>>>(a); break;
-    case 6: k_scan_assign<true, true, false><<<g, kScanThreads, 0, s>>>(a); break;
-    default: k_scan_assign<true, true, true><<<g, kScanThreads, 0, s>>>(a); break;
-  }
+  // Up to 2^24 cells the field (64 MB) stays in L2 while it is written, so the
+  // scan stores each redshift in its place (ranked matching: 256^3 301 -> 216
+  // us, 128^3 72 -> 56, 32^3 64 -> 52); above that the stores would reach HBM
+  // one sector per cell, so the pairs go through the buckets.  With the masses
+  // gathered as well the two kinds of scattered access share the pipe: ranking
+  // and matching 1.0e6 cells 154 -> 145 us, 3.0e6 274 -> 272, 1.0e7 610 -> 618.
+  // (Also when the result may overwrite what the scan reads.)
+  const bool direct = n <= (gather ? kDirectGatherMaxCells : kDirectMaxCells) && disjoint(zre, n, order, n) && disjoint(zre, n, mass, n) &&
+                      disjoint(zre, n, order_b, n) && disjoint(zre, n, mass_b, n) && disjoint(zre, n, F, n);
+  if (direct) a.zre = zre;
+  auto launch = [&](auto gt, auto ft, auto lt, auto dt) {
+    k_scan_assign<decltype(gt)::value, decltype(ft)::value, decltype(lt)::value, decltype(dt)::value>
+        <<<g, kScanThreads, 0, s>>>(a);
+  };
+  auto pick4 = [&](auto gt, auto ft, auto lt) {
+    if (direct) launch(gt, ft, lt, std::true_type{});
+    else launch(gt, ft, lt, std::false_type{});
+  };
+  auto pick3 = [&](auto gt, auto ft) {
+    if (lin) pick4(gt, ft, std::true_type{});
+    else pick4(gt, ft, std::false_type{});
+  };
+  auto pick2 = [&](auto gt) {
+    if (F) pick3(gt, std::true_type{});
+    else pick3(gt, std::false_type{});
+  };
+  if (gather) pick2(std::true_type{});
+  else pick2(std::false_type{});
   prof_end(prof, PK_SCAN_ASSIGN, s);
+  if (direct) return cudaGetLastError();
   prof_begin(prof, PK_SCATTER_BACK, s);
   k_scatter_back<<<(unsigned)(xa.groups * xa.nbuckets), 256, 0, s>>>(xa.bcell, xa.bz, xa.btab, xa.nbuckets, xa.tiles,
                                                                      xa.groups, xa.wpt, xa.zre);

@@ -23,8 +23,10 @@ constexpr int kScanThreads = AMBER_SCAN_THREADS;
 constexpr int kScanItems = AMBER_SCAN_ITEMS;
 constexpr int kScanTile = kScanThreads * kScanItems;
 constexpr int kMaxTable = 1 << 16;
-constexpr int kMaxBuckets = 1024;
+constexpr int kMaxBuckets = 128;  // 2^30 cells in buckets of 2^23
 
+// the scan writes z in place up to these sizes (masses in rank order; gathered)
+constexpr int64_t kDirectMaxCells = (int64_t)1 << 24, kDirectGatherMaxCells = (int64_t)1 << 22;
 constexpr int kBackTilesPerCta = 8;  // scan tiles one scatter-back CTA covers
 constexpr int kBucketShift = 23;  // 2^23 cells (32 MB of z_re) per bucket by default
 
@@ -71,6 +73,7 @@ struct ScanArgs {
   uint32_t* ticket;
   int nbuckets;
   int bucket_shift;  // bucket of a cell = cell >> bucket_shift
+  float* zre;        // DIRECT scans: the field itself (the buckets are not used)
   uint32_t* bcell;
   float* bz;
   uint16_t* btab;

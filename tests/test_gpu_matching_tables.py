@@ -46,3 +46,24 @@ def test_assign_table_edges_vs_oracle(B, weighting, n_table, n):
         d = np.abs(z.cpu().numpy().astype(np.float64) - zo)
         assert np.mean(d > 1e-3) <= (0.0 if n < 10_000 else 1e-4), (np.mean(d > 1e-3), d.max())
         assert np.quantile(d, 0.999) < 5e-5, np.quantile(d, 0.999)
+
+
+@pytest.mark.parametrize("weighting", [0, 1])
+@pytest.mark.parametrize("n", [8_193, (1 << 22) + 1])
+def test_assign_forms_agree(B, n, weighting):
+    # redshifts stored in place (masses in rank order, or gathered up to 2^22
+    # cells) and through the buckets (gathered above 2^22; a result that
+    # overwrites the rank-order masses): the same numbers, bit for bit
+    g = torch.Generator(device="cuda").manual_seed(n + weighting)
+    mass = torch.rand(n, generator=g, device="cuda") * 2.9 + 0.01
+    order = torch.randperm(n, generator=g, device="cuda").to(torch.int32)
+    ranked = mass[order.long()].contiguous()
+    h = B.history(8.0, 4.0, 3.0, weighting=weighting)
+    with B.Context(n) as ctx:
+        gathered = ctx.assign_zre(order, mass, h)
+        placed = ctx.assign_zre_ranked(order, ranked, h, torch.empty_like(mass))
+        F = torch.empty(n, dtype=torch.float64, device="cuda")
+        with_F = ctx.assign_zre_ranked(order, ranked, h, torch.empty_like(mass), F=F)
+        over = ctx.assign_zre_ranked(order, ranked, h, ranked)
+        assert ctx.sync_status() == 0
+    assert torch.equal(gathered, placed) and torch.equal(gathered, with_F) and torch.equal(gathered, over)
