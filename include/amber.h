@@ -255,6 +255,10 @@ int amber_solve_spectrum(amber_ctx *ctx, const void *d_spec, const float *d_mass
  *   fft_variant      0: the default tiles (every n); 1: an alternative radix
  *                    split or tile width (n >= 128: 1024 with 4-line tiles,
  *                    512 as 16 x 32, 256 as 32 x 8, 128 as 8 x 16);
+ *   (FP32 rankings split their cells into buckets of like intensity and sort
+ *   those on chip.  The three sort choices are those of the radix sort that
+ *   ranks with fuse_histogram 1, in a batch, in the later intervals of a
+ *   tomographic matching, and when AMBER_SORT_RANK is set.)
  *   sort_digit_bits  9 or 8: digit width of the radix sort (a few-octave
  *                    intensity field needs 27 bits: 3 passes of 9 bits, 4 of 8;
  *                    a 24-bit range takes 3 of either, the 8-bit ones cheaper);
@@ -379,10 +383,11 @@ int amber_profile_reset(amber_ctx *ctx);
 int amber_profile_kinds(void);
 int amber_profile_read(amber_ctx *ctx, int kind, const char **name, double *total_ms, int64_t *launches);
 
-/* Digit passes the last ranking needed (diagnostic; synchronises the
- * context's last stream).  The sort runs on key - min(key) with 9- or 8-bit
- * digits (amber_tuning_t), so an intensity field spanning few octaves (27
- * bits) needs 3 or 4 passes; at most 4 for FP32 keys. */
+/* Digit passes the last ranking's key range takes (diagnostic; synchronises
+ * the context's last stream): with 9- or 8-bit digits (amber_tuning_t) of
+ * key - min(key), an intensity field spanning few octaves (27 bits) takes 3
+ * or 4; at most 4 for FP32 keys.  (An FP32 ranking that splits its cells into
+ * balanced buckets instead reports the same number.) */
 int amber_sort_passes(amber_ctx *ctx, int *out_passes);
 
 /* Tomographic abundance matching (Sec. 3.4.2 names matching over several

@@ -15,6 +15,7 @@
 #include "source.cuh"
 #include "spectra.cuh"
 #include "lpt.cuh"
+#include "msd.cuh"
 
 namespace amber {
 // krange: if not null, the intensities' key range is folded into it (the
@@ -177,9 +178,17 @@ struct Plan {
   int n32 = 0, n64 = 0;
   int64_t cells64 = 0;
   size_t off_spec, off_keysA, off_keysB, off_idxA, off_idxB, off_massA, off_massB, off_lb, off_sctrl, off_actrl, off_X, off_invdx, off_lin,
-      off_state, off_btab, off_tilemass, off_status, off_srcsum, off_pow, off_ktab, off_tw32, off_tw64, total;
+      off_state, off_btab, off_tilemass, off_msd, off_msd_cnt2, off_msd_small, off_status, off_srcsum, off_pow, off_ktab, off_tw32, off_tw64, total;
   size_t tw32_off[11] = {}, tw64_off[11] = {};
 };
+
+// Rankings of fewer cells take their bucket regions here: what a region holds
+// beyond its bucket's average weighs more in small buckets (3 words per cell).
+constexpr int64_t kMsdSmallCells = 1 << 18;
+static size_t msd_small_words(int64_t max_cells) {
+  const int64_t n = std::min(max_cells, kMsdSmallCells);
+  return (size_t)(3 * (n + n / 5 + 96 * (n / kMsdMinAvg + 1)));
+}
 
 static size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
@@ -193,7 +202,10 @@ static Plan make_plan(int64_t max_cells) {
   const size_t keyb = std::max((size_t)max_cells * 4, (size_t)p.cells64 * 8);
   const size_t idxb = (size_t)max_cells * 4;
   const size_t lb = 2 * sort_lookback_words(max_cells) * 4;
-  const size_t stt = (size_t)((max_cells + kScanTile - 1) / kScanTile) * sizeof(unsigned long long);
+  // scan tiles of a given ranking, or final buckets of a ranking by splitting
+  const int64_t buckets = msd_most_buckets(max_cells);
+  const int64_t rows = std::max<int64_t>((max_cells + kScanTile - 1) / kScanTile, buckets);
+  const size_t stt = (size_t)rows * sizeof(unsigned long long);
   size_t o = 0;
   auto take = [&](size_t bytes) { const size_t at = o; o += align256(bytes); return at; };
   p.off_spec = take(spec);
@@ -210,8 +222,11 @@ static Plan make_plan(int64_t max_cells) {
   p.off_invdx = take((size_t)kMaxTable * sizeof(float));
   p.off_lin = take((size_t)4 * kMaxTable * sizeof(float));
   p.off_state = take(stt);
-  p.off_btab = take((size_t)((max_cells + kScanTile - 1) / kScanTile) * (kMaxBuckets + 1) * sizeof(uint16_t));
-  p.off_tilemass = take((size_t)sort_tiles(max_cells) * 16);
+  p.off_btab = take((size_t)rows * (kMaxBuckets + 1) * sizeof(uint16_t));
+  p.off_tilemass = take(std::max<size_t>((size_t)sort_tiles(max_cells) * 16, 4096 * 16));
+  p.off_msd = take(sizeof(MsdCtrl));
+  p.off_msd_cnt2 = take((size_t)buckets * 4);
+  p.off_msd_small = take(msd_small_words(max_cells) * 4);
   p.off_status = take(256);
   p.off_srcsum = take(256);
   p.off_pow = take((size_t)kPowerAcc * kMaxPowerBins * sizeof(double));
@@ -290,6 +305,123 @@ int cuda_status(cudaError_t e) {
 }  // namespace
 
 namespace {
+
+// Ranking by splitting (msd.cu) of n intensities J on this context's workspace:
+// fills its arguments, or returns false where the digit passes are asked for
+// (AMBER_SORT_RANK) or the workspace is too small for the buckets' regions.
+// The spectrum and the six sort arrays are one block.  The first split's regions
+// lie at its start, the second's after them; J (J_inside) is massB and the
+// masses (mass_inside) idxB, which only the second split may overwrite.  Their
+// values then come back from the first split's regions if it overflows.
+bool msd_setup(amber_ctx* c, const float* J, bool J_inside, const float* mass, bool mass_inside, int64_t n,
+               uint32_t* order, float* mass_out, int digit_bits, MsdArgs* out, FallbackArgs* fb) {
+  const Plan& pl = c->plan;
+  if (sort_rank_env() >= 0) return false;
+  const MsdPlan p = msd_plan(n, mass != nullptr, c->num_sms);
+  uint32_t* block = reinterpret_cast<uint32_t*>(c->ws + pl.off_spec);
+  const int64_t words = (int64_t)(pl.off_lb - pl.off_spec) / 4;
+  // the first split must leave the values it reads alone, and with one split the
+  // arrays its ranking may go to as well (idxB, massA)
+  const size_t first_end = mass_inside || (J_inside && p.nb2 == 1) ? pl.off_idxB : J_inside ? pl.off_massB : pl.off_lb;
+  const int64_t inside = (int64_t)(first_end - pl.off_spec) / 4;
+  const bool small = n < kMsdSmallCells;
+  if (small && p.kv1 + p.m1 > (int64_t)msd_small_words(c->max_cells)) return false;
+  if (!small && (p.kv1 + p.m1 > inside || p.kv1 + p.m1 + p.kv2 + p.m2 > words)) return false;
+  if (n > c->max_cells) return false;
+  uint32_t* at = small ? reinterpret_cast<uint32_t*>(c->ws + pl.off_msd_small) : block;
+  MsdArgs& a = *out;
+  a = MsdArgs{};
+  a.J = J;
+  a.mass = mass;
+  a.n = n;
+  a.kv1 = reinterpret_cast<uint2*>(at);
+  a.mass1 = reinterpret_cast<float*>(at + p.kv1);
+  a.kv2 = reinterpret_cast<uint2*>(at + p.kv1 + p.m1);
+  a.mass2 = reinterpret_cast<float*>(at + p.kv1 + p.m1 + p.kv2);
+  a.cap1 = p.cap1;
+  a.nb1 = p.nb1;
+  a.nb2 = p.nb2;
+  a.idx_shift = p.idx_shift;
+  a.digit_bits = digit_bits;
+  a.ctrl = c->sortw.ctrl;
+  a.mc = reinterpret_cast<MsdCtrl*>(c->ws + pl.off_msd);
+  a.cnt2 = reinterpret_cast<uint32_t*>(c->ws + pl.off_msd_cnt2);
+  a.cta_mass = reinterpret_cast<unsigned long long*>(c->ws + pl.off_tilemass);
+  a.order = order;
+  a.mass_out = mass_out;
+  a.status = c->status;
+  a.fb_order[0] = c->sortw.idxA;
+  a.fb_order[1] = c->sortw.idxB;
+  a.fb_mass[0] = c->sortw.massA;
+  a.fb_mass[1] = c->sortw.massB;
+  FallbackArgs& f = *fb;
+  f = FallbackArgs{};
+  f.mc = a.mc;
+  uint32_t blocks;
+  // with masses the fallback leaves its ranking in the workspace for the matching
+  rank_args<float>(c->sortw, J, n, mass ? nullptr : order, mass, nullptr, nullptr, c->status, kSpinLimit, 8, &f.hist,
+                   &blocks, f.pass);
+  f.tiles = sort_tiles(n);
+  if (p.nb2 > 1) {
+    f.J_restore = J_inside ? const_cast<float*>(J) : nullptr;
+    f.mass_restore = mass_inside ? const_cast<float*>(mass) : nullptr;
+  }
+  f.kv1 = a.kv1;
+  f.mass1 = a.mass1;
+  f.nb1 = p.nb1;
+  f.cap1 = p.cap1;
+  return true;
+}
+
+// Rank J (key range already in the control block) and match.  False (nothing
+// enqueued) as msd_setup.
+bool msd_match(amber_ctx* c, const float* J, bool J_inside, const float* mass, bool mass_inside, int64_t n,
+               const HistoryCoeffs& hc, float* zre, uint32_t* order_out, float* mass_rank_out, int digit_bits,
+               cudaStream_t s, cudaError_t* err) {
+  MsdArgs ma;
+  FallbackArgs fa;
+  if (!msd_setup(c, J, J_inside, mass, mass_inside, n, order_out, mass_rank_out, digit_bits, &ma, &fa)) return false;
+  const Plan& pl = c->plan;
+  const int nsums = msd_split_ctas(n, MsdPlan{ma.nb1, ma.nb2, ma.cap1}, c->num_sms);
+  const unsigned char* z = reinterpret_cast<const unsigned char*>(zre);
+  // Matched in the local sort where redshifts are stored in place (assign.cu;
+  // a result inside the workspace would lie among what the local sort reads).
+  // With pairs and buckets to form as well it is slower than the scan on its
+  // 8192-rank tiles (512^3: local sort with matching 2.31 ms, apart 1.13 + 0.92).
+  if (n <= kDirectMaxCells && (z < c->ws || z >= c->ws + pl.total)) {
+    ThreshArgs ta;
+    ScanArgs sa;
+    ScatterArgs xa;
+    assign_args(c->assw, nullptr, nullptr, nullptr, n, hc, zre, nullptr, c->status, kSpinLimit, nullptr, nullptr,
+                nullptr, &ta, &sa, &xa);
+    ta.tile_mass = ma.cta_mass;
+    ta.ntiles = nsums;
+    ma.actrl = c->assw.ctrl;
+    ma.state = c->assw.state;
+    sa.zre = zre;
+    *err = msd_run(ma, fa, c->num_sms, &ta, &sa, s, &c->prof);
+    return true;
+  }
+  // the ranking over the first split's regions (two splits: dead by then) or
+  // idxB and massA; the pairs in arrays that are free then
+  uint32_t* block = reinterpret_cast<uint32_t*>(c->ws + pl.off_spec);
+  AssignWork w = c->assw;
+  if (ma.nb2 > 1) {
+    w.bcell = c->sortw.idxB;
+    w.bz = c->sortw.massA;
+  }
+  if (!order_out) {
+    ma.order = ma.nb2 > 1 ? block : c->sortw.idxB;
+    ma.mass_out = ma.nb2 > 1 ? reinterpret_cast<float*>(block + (n + 63) / 64 * 64) : c->sortw.massA;
+  }
+  fa.order_to = ma.order;
+  fa.mass_to = ma.mass_out;
+  *err = msd_run(ma, fa, c->num_sms, nullptr, nullptr, s, &c->prof);
+  if (*err == cudaSuccess)
+    *err = assign_impl(w, ma.order, ma.mass_out, true, ma.cta_mass, n, hc, zre, nullptr, c->status, s, &c->prof,
+                       kSpinLimit, nullptr, nullptr, nullptr, nsums);
+  return true;
+}
 
 // Bump allocator over one device allocation (256-byte aligned pieces).
 struct Layout {
@@ -397,6 +529,7 @@ int amber_create(amber_ctx** out, int device, int64_t max_cells) {
   const Plan& p = c->plan;
   c->status = reinterpret_cast<unsigned int*>(c->ws + p.off_status);
   cudaMemset(c->ws + p.off_status, 0, 256);
+  cudaMemset(c->ws + p.off_msd, 0, sizeof(MsdCtrl));
   c->sortw.keysA = c->ws + p.off_keysA;
   c->sortw.keysB = c->ws + p.off_keysB;
   c->sortw.idxA = reinterpret_cast<uint32_t*>(c->ws + p.off_idxA);
@@ -658,6 +791,14 @@ int amber_rank(amber_ctx* c, const float* d_J, int64_t ncells, uint32_t* d_order
   DeviceGuard g(c->device);
   cudaStream_t s = (cudaStream_t)stream;
   c->last_stream = s;
+  MsdArgs ma;
+  FallbackArgs fa;
+  if (msd_setup(c, d_J, false, nullptr, false, ncells, d_order, nullptr, KeyOf<float>::RB, &ma, &fa)) {
+    cudaError_t e = sort_ctrl_reset(c->sortw.ctrl, s);
+    if (e == cudaSuccess) e = key_range_impl(d_J, ncells, c->sortw.ctrl, c->num_sms, c->status, s);
+    if (e == cudaSuccess) e = msd_run(ma, fa, c->num_sms, nullptr, nullptr, s, &c->prof);
+    return cuda_status(e);
+  }
   return cuda_status(rank_impl<float>(c->sortw, d_J, ncells, d_order, nullptr, nullptr, nullptr, false, c->status, s,
                                       &c->prof, kSpinLimit));
 }
@@ -710,7 +851,7 @@ static cudaError_t solve_f32_enqueue(amber_ctx* c, const float* d_src, const flo
   const Plan& pl = c->plan;
   const int n = p->n;
   const int64_t C = (int64_t)n * n * n;
-  float* J = d_J_opt ? d_J_opt : reinterpret_cast<float*>(c->sortw.keysB);
+  float* J = d_J_opt ? d_J_opt : c->sortw.massB;
   const amber_tuning_t& tu = c->tune[ilog2i(n)];
   // with 8-bit digits the inverse x pass can count the raw keys' digits
   const bool fuse = tu.fuse_histogram && tu.sort_digit_bits == 8;
@@ -719,6 +860,10 @@ static cudaError_t solve_f32_enqueue(amber_ctx* c, const float* d_src, const flo
     e = radiation_field_f32(n, d_src, J, c->ws + pl.off_spec, c->ws + pl.off_tw32 + pl.tw32_off[ilog2i(n)], p->box,
                            p->l_mfp, c->status, s, &c->prof, c->sortw.ctrl, tu.fft_variant, spec_in, fuse,
                            tu.zpass_tma != 0);
+  if (e != cudaSuccess) return e;
+  if (!fuse && msd_match(c, J, !d_J_opt, d_mass, d_mass == reinterpret_cast<const float*>(c->sortw.idxB), C, hc, d_zre,
+                         order_out, mass_rank_out, tu.sort_digit_bits, s, &e))
+    return e;
   // the first sort pass sums each tile's masses; the thresholds kernel adds them
   unsigned long long* tile_mass = reinterpret_cast<unsigned long long*>(c->ws + pl.off_tilemass);
   if (e == cudaSuccess)
@@ -843,12 +988,12 @@ int amber_solve_host(amber_ctx* c, const float* h_src, const float* h_mass, cons
   c->last_stream = s;
   const size_t bytes = (size_t)p->n * p->n * p->n * sizeof(float);
   // device copies in workspace that is free when they are live: the source in
-  // the second index array (read by the forward x pass, first written by the
-  // second digit pass), the masses in the second mass array (read by the
-  // first digit pass, first written by the second), z_re in the transform
-  // buffer (free once the inverse x pass has run)
-  float* dS = reinterpret_cast<float*>(c->sortw.idxB);
-  float* dM = c->sortw.massB;
+  // the first mass array (read by the forward x pass, not written before the
+  // ranking), the masses in the second index array (read by the ranking's first
+  // pass, first written by its second), z_re in the transform buffer (free once
+  // the inverse x pass has run, and written last)
+  float* dS = c->sortw.massA;
+  float* dM = reinterpret_cast<float*>(c->sortw.idxB);
   float* dZ = reinterpret_cast<float*>(c->ws + c->plan.off_spec);
   cudaError_t e = cudaMemcpyAsync(dS, h_src, bytes, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dM, h_mass, bytes, cudaMemcpyHostToDevice, s);
@@ -913,7 +1058,7 @@ int amber_solve_tomographic(amber_ctx* c, const float* const* d_src_list, int ni
   const Plan& pl = c->plan;
   const int n = p->n;
   const int64_t C = (int64_t)n * n * n;
-  float* J = reinterpret_cast<float*>(c->sortw.keysB);
+  float* J = c->sortw.massB;
   // the transform buffer is free once J is formed: it holds each interval's matching
   float* ztmp = reinterpret_cast<float*>(c->ws + pl.off_spec);
   unsigned long long* tile_mass = reinterpret_cast<unsigned long long*>(c->ws + pl.off_tilemass);
@@ -926,12 +1071,16 @@ int amber_solve_tomographic(amber_ctx* c, const float* const* d_src_list, int ni
                               p->box, p->l_mfp, c->status, s, &c->prof, c->sortw.ctrl,
                               c->tune[ilog2i(n)].fft_variant, nullptr, false, c->tune[ilog2i(n)].zpass_tma != 0);
     if (e == cudaSuccess && k > 0) e = tomo_mask(J, d_zre, C, c->sortw.ctrl, c->num_sms, s);
-    if (e == cudaSuccess)
+    // the cells ionized so far share one key and lie together: buckets of the
+    // splits would overflow, so later intervals take the digit passes at once
+    if (e == cudaSuccess && (k > 0 || !msd_match(c, J, true, d_mass, false, C, hc, ztmp, nullptr, nullptr,
+                                                 c->tune[ilog2i(n)].sort_digit_bits, s, &e))) {
       e = rank_impl<float>(c->sortw, J, C, nullptr, d_mass, nullptr, tile_mass, true, c->status, s, &c->prof,
                            kSpinLimit, c->tune[ilog2i(n)].sort_digit_bits, c->tune[ilog2i(n)].sort_match);
-    if (e == cudaSuccess)
-      e = assign_impl(c->assw, c->sortw.idxA, c->sortw.massA, true, tile_mass, C, hc, ztmp, nullptr, c->status, s,
-                      &c->prof, kSpinLimit, c->sortw.idxB, c->sortw.massB, &c->sortw.ctrl->npasses);
+      if (e == cudaSuccess)
+        e = assign_impl(c->assw, c->sortw.idxA, c->sortw.massA, true, tile_mass, C, hc, ztmp, nullptr, c->status, s,
+                        &c->prof, kSpinLimit, c->sortw.idxB, c->sortw.massB, &c->sortw.ctrl->npasses);
+    }
     if (e == cudaSuccess) e = tomo_merge(d_zre, ztmp, C, (float)z_bounds[k + 1], k == nint - 1, c->num_sms, s);
   }
   return cuda_status(e);

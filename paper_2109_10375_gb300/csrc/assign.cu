@@ -313,9 +313,13 @@ __global__ void __launch_bounds__(kScanThreads, AMBER_SCAN_MINB)
 // wpt (1, 2, 4 or 8) warps share one tile's run, each taking a contiguous
 // part: with few buckets (small grids) a run holds most of a tile's 8192
 // pairs, and one warp copying it alone would wait through dozens of rounds.
-__device__ __forceinline__ void scatter_back_body(const uint32_t* __restrict__ bcell, const float* __restrict__ bz,
-                                                  const uint16_t* __restrict__ btab, int nbuckets, int64_t tiles,
-                                                  int groups, int wpt, float* __restrict__ zre, uint32_t blk) {
+__device__ __forceinline__ void scatter_back_body(const ScatterArgs& x, uint32_t blk) {
+  const uint32_t* __restrict__ bcell = x.bcell;
+  const float* __restrict__ bz = x.bz;
+  const uint16_t* __restrict__ btab = x.btab;
+  float* __restrict__ zre = x.zre;
+  const int nbuckets = x.nbuckets, groups = x.groups, wpt = x.wpt;
+  const int64_t tiles = x.tiles;
   constexpr int TPW = 1;  // tiles per warp
   const int b = blk / groups;
   const int64_t g = blk - (int64_t)b * groups;
@@ -365,19 +369,13 @@ __device__ __forceinline__ void scatter_back_body(const uint32_t* __restrict__ b
   }
 }
 
-__global__ void __launch_bounds__(256) k_scatter_back(const uint32_t* __restrict__ bcell,
-                                                      const float* __restrict__ bz,
-                                                      const uint16_t* __restrict__ btab, int nbuckets,
-                                                      int64_t tiles, int groups, int wpt, float* __restrict__ zre) {
-  scatter_back_body(bcell, bz, btab, nbuckets, tiles, groups, wpt, zre, blockIdx.x);
-}
+__global__ void __launch_bounds__(256) k_scatter_back(const ScatterArgs x) { scatter_back_body(x, blockIdx.x); }
 
 // Several scatters at once: CTA b works on item find_item(prefix, M, b).
 __global__ void __launch_bounds__(256) k_scatter_back_multi(const ScatterArgs* __restrict__ args,
                                                             const uint32_t* __restrict__ prefix, int M) {
   const int it = find_item(prefix, M, blockIdx.x);
-  const ScatterArgs& a = args[it];
-  scatter_back_body(a.bcell, a.bz, a.btab, a.nbuckets, a.tiles, a.groups, a.wpt, a.zre, blockIdx.x - prefix[it]);
+  scatter_back_body(args[it], blockIdx.x - prefix[it]);
 }
 
 // ---------------------------------------------------------------------------
@@ -440,6 +438,15 @@ void bucket_plan(int64_t n, int* nbuckets, int* shift) {
   *nbuckets = (int)((n + ((int64_t)1 << kBucketShift) - 1) >> kBucketShift);
 }
 
+void thresholds_launch(ThreshArgs ta, cudaStream_t s) {
+  if (ta.ntiles > kTileTotalMin) {
+    k_tile_total<<<(unsigned)std::min<int64_t>(64, (ta.ntiles + 1023) / 1024), 256, 0, s>>>(ta.tile_mass, ta.ntiles,
+                                                                                         ta.total);
+    ta.tile_mass = nullptr;
+  }
+  k_thresholds<<<(ta.M + kThreshPoints - 1) / kThreshPoints, kThreshThreads, 0, s>>>(ta);
+}
+
 void assign_args(const AssignWork& w, const uint32_t* order, const float* mass, const unsigned long long* tile_mass,
                  int64_t n, const HistoryCoeffs& hc, float* zre, double* F, unsigned int* status,
                  unsigned int spin_limit, const uint32_t* order_b, const float* mass_b, const int* pick,
@@ -481,6 +488,7 @@ void assign_args(const AssignWork& w, const uint32_t* order, const float* mass, 
   a.qtotal = qtotal;
   a.inv_dx = w.inv_dx;
   a.n_table = hc.n_table;
+  a.weighting = hc.weighting;
   a.z_lo = (float)hc.z_lo;
   a.z_hi = (float)hc.z_hi;
   a.dzt = (float)((hc.z_hi - hc.z_lo) / (double)(hc.n_table - 1));
@@ -523,12 +531,13 @@ template <typename A, typename B> static bool disjoint(const A* a, int64_t na, c
 cudaError_t assign_impl(const AssignWork& w, const uint32_t* order, const float* mass, bool mass_in_rank_order,
                         const unsigned long long* tile_mass, int64_t n, const HistoryCoeffs& hc, float* zre, double* F,
                         unsigned int* status, cudaStream_t s, FftProfile* prof, unsigned int spin_limit,
-                        const uint32_t* order_b, const float* mass_b, const int* pick) {
+                        const uint32_t* order_b, const float* mass_b, const int* pick, int64_t nsums) {
   const int64_t tiles = (n + kScanTile - 1) / kScanTile;
   ThreshArgs ta;
   ScanArgs a;
   ScatterArgs xa;
   assign_args(w, order, mass, tile_mass, n, hc, zre, F, status, spin_limit, order_b, mass_b, pick, &ta, &a, &xa);
+  if (tile_mass && nsums >= 0) ta.ntiles = nsums;
   cudaError_t e = cudaMemsetAsync(w.ctrl, 0, kAssignCtrlBytes, s);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(w.state, 0, (size_t)tiles * sizeof(unsigned long long), s);
@@ -543,12 +552,7 @@ cudaError_t assign_impl(const AssignWork& w, const uint32_t* order, const float*
   }
 
   prof_begin(prof, PK_THRESHOLDS, s);
-  if (ta.ntiles > kTileTotalMin) {
-    k_tile_total<<<(unsigned)std::min<int64_t>(64, (ta.ntiles + 1023) / 1024), 256, 0, s>>>(tile_mass, ta.ntiles,
-                                                                                         ta.total);
-    ta.tile_mass = nullptr;
-  }
-  k_thresholds<<<(ta.M + kThreshPoints - 1) / kThreshPoints, kThreshThreads, 0, s>>>(ta);
+  thresholds_launch(ta, s);
   prof_end(prof, PK_THRESHOLDS, s);
 
   prof_begin(prof, PK_SCAN_ASSIGN, s);
@@ -585,8 +589,7 @@ cudaError_t assign_impl(const AssignWork& w, const uint32_t* order, const float*
   prof_end(prof, PK_SCAN_ASSIGN, s);
   if (direct) return cudaGetLastError();
   prof_begin(prof, PK_SCATTER_BACK, s);
-  k_scatter_back<<<(unsigned)(xa.groups * xa.nbuckets), 256, 0, s>>>(xa.bcell, xa.bz, xa.btab, xa.nbuckets, xa.tiles,
-                                                                     xa.groups, xa.wpt, xa.zre);
+  k_scatter_back<<<(unsigned)(xa.groups * xa.nbuckets), 256, 0, s>>>(xa);
   prof_end(prof, PK_SCATTER_BACK, s);
   return cudaGetLastError();
 }

@@ -67,6 +67,7 @@ struct ScanArgs {
   const unsigned long long* qtotal;  // total in that fixed point (for F)
   const float* inv_dx;
   int n_table;
+  int weighting;
   float z_lo, z_hi, dzt;
   double* F;
   unsigned long long* state;
@@ -144,6 +145,9 @@ void assign_args(const AssignWork& w, const uint32_t* order, const float* mass, 
                  ThreshArgs* ta, ScanArgs* sa, ScatterArgs* xa);
 cudaError_t assign_multi(const AssignMulti& m, cudaStream_t s);
 
+// One matching's thresholds.
+void thresholds_launch(ThreshArgs ta, cudaStream_t s);
+
 void bucket_plan(int64_t n, int* nbuckets, int* shift);
 
 // Tomographic matching: fill z with NaN (neutral); give cells with a redshift
@@ -160,6 +164,7 @@ cudaError_t tomo_merge(float* z, const float* ztmp, int64_t n, float z_low, bool
 cudaError_t assign_impl(const AssignWork& w, const uint32_t* order, const float* mass, bool mass_in_rank_order,
                         const unsigned long long* tile_mass, int64_t n, const HistoryCoeffs& hc, float* zre, double* F,
                         unsigned int* status, cudaStream_t s, FftProfile* prof, unsigned int spin_limit,
-                        const uint32_t* order_b = nullptr, const float* mass_b = nullptr, const int* pick = nullptr);
+                        const uint32_t* order_b = nullptr, const float* mass_b = nullptr, const int* pick = nullptr,
+                        int64_t nsums = -1);
 
 }  // namespace amber

@@ -1,0 +1,120 @@
+// Ranking by splitting (see msd.cu): constants, arguments and host entry.
+#pragma once
+
+#include "assign.cuh"
+#include "common.cuh"
+#include "fft.cuh"  // FftProfile, prof_begin/prof_end, ProfKind
+#include "keys.cuh"
+#include "sort.cuh"
+
+namespace amber {
+
+constexpr int kMsdKnotBits = 11;
+constexpr int kMsdKnots = 1 << kMsdKnotBits;  // knots of the distribution map
+constexpr int kMsdMaxDigits = 1024;           // buckets one split can write
+// Tiles of a split: 4096 cells (two CTAs per SM), or 10240 (one) where there are
+// so many buckets that a small tile's runs would be short: with 529 buckets
+// (1024^3) 8.1 against 7.1 ms a split, with 187 (512^3) 0.75 against 0.89.
+constexpr int kMsdTileA = 4096, kMsdTileB = 10240;
+constexpr uint32_t kMsdManyDigits = 320;
+constexpr int kMsdLocalThreads = 512;
+constexpr int kMsdLocalItems = 9;
+constexpr int kMsdCap = kMsdLocalThreads * kMsdLocalItems;  // most cells of a final bucket
+constexpr int kMsdAvg = kMsdCap * 5 / 6;                    // cells per final bucket aimed at,
+constexpr int kMsdMinAvg = 320;                             // fewer where that leaves SMs idle
+constexpr int kMsdSub = 8192;                               // sub-buckets of a final bucket
+
+// Device control block; zero when created, left clean by every ranking.
+struct MsdCtrl {
+  uint32_t overflow;  // bit 0: a first-split bucket, bit 1: a second-split bucket outgrew its region
+  uint32_t done;      // CTAs of the map kernel that finished
+  uint32_t bar;       // grid barrier of the fallback
+  uint32_t pad[61];
+  uint32_t hist[kMsdKnots];
+  uint32_t map[kMsdKnots + 4];
+  uint32_t cnt1[kMsdMaxDigits];
+};
+
+struct MsdArgs {
+  const float* J;
+  const float* mass;   // or null
+  int64_t n;
+  uint2* kv1;          // first split: nb1 regions of cap1 (key, cell) pairs (final ones if nb2 is 1)
+  float* mass1;
+  uint2* kv2;          // second split (nb2 > 1): nb1 nb2 regions of kMsdCap
+  float* mass2;
+  uint32_t cap1, nb1, nb2;
+  int idx_shift;         // cell index << idx_shift fills 32 bits
+  int digit_bits;        // for the pass count reported
+  SortCtrl* ctrl;
+  MsdCtrl* mc;
+  uint32_t* cnt2;      // nb1 nb2 counts
+  unsigned long long* cta_mass;  // per CTA of the first split: exact 128-bit mass sum
+  uint32_t* order;     // the ranking, or null
+  float* mass_out;     // masses in rank order, or null
+  unsigned int* status;
+  // matching in the local sort (SCAN)
+  unsigned char* actrl;          // assign control block, cleared by the map kernel
+  unsigned long long* state;     // scan look-back words, one per final bucket (cleared there too)
+  const uint32_t* fb_order[2];   // the fallback's ranking by parity of its passes
+  const float* fb_mass[2];
+};
+
+struct MsdPlan {
+  uint32_t nb1, nb2, cap1;
+  int idx_shift;
+  int64_t kv1, m1, kv2, m2;  // words of the sets (kv: 2 per cell)
+};
+MsdPlan msd_plan(int64_t n, bool with_mass, int num_sms);
+// No ranking of up to n cells makes more final buckets.
+inline int64_t msd_most_buckets(int64_t n) {
+  const int64_t nb = (n + kMsdAvg - 1) / kMsdAvg;
+  if (nb <= kMsdMaxDigits) return kMsdMaxDigits;
+  int64_t r = 1;
+  while (r * r < nb) ++r;
+  return r * r;
+}
+int msd_split_ctas(int64_t n, const MsdPlan& p, int num_sms);
+
+// Arguments of the other ranking (digit passes in one cooperative launch),
+// which runs when a bucket overflowed.
+struct FallbackArgs {
+  MsdCtrl* mc;
+  HistArgs hist;
+  PassArgs pass[4];
+  int64_t tiles;
+  // second-split overflow: intensities (and masses) kept in workspace were
+  // overwritten by then and are put back from the first split's regions
+  float* J_restore;
+  float* mass_restore;
+  const uint2* kv1;
+  const float* mass1;
+  uint32_t nb1, cap1;
+  uint32_t* order_to;  // or null: the ranking (and masses) are copied here
+  float* mass_to;
+};
+cudaError_t sort_fallback(const FallbackArgs& f, bool with_mass, int num_sms, cudaStream_t s);
+
+// Enqueue the ranking of a.J, to a.order (and a.mass_out); with sa (and masses)
+// the local sort also matches and stores each redshift in its place (ta:
+// thresholds, with cta_mass as partial sums).
+cudaError_t msd_run(const MsdArgs& a, const FallbackArgs& f, int num_sms, const ThreshArgs* ta, const ScanArgs* sa,
+                    cudaStream_t s, FftProfile* prof);
+
+// Knots are 2^L keys wide and aligned to them, so that no knot straddles two
+// octaves of the intensity (a float's keys are half as dense per unit value in
+// the next octave, which would bend the distribution inside the knot); kbase is
+// the smallest key rounded down to a knot.
+struct MsdRange {
+  uint32_t kbase;
+  int L;
+};
+__device__ __forceinline__ MsdRange msd_range(const SortCtrl* ctrl) {
+  const uint32_t lo = (uint32_t)ctrl->kmin, hi = (uint32_t)ctrl->kmax;
+  const int bits = 32 - __clz((int)(hi - lo));
+  int L = bits > kMsdKnotBits ? bits - kMsdKnotBits : 0;
+  if ((hi >> L) - (lo >> L) >= (uint32_t)kMsdKnots) ++L;
+  return {lo >> L << L, L};
+}
+
+}  // namespace amber

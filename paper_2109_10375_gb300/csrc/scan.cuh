@@ -69,6 +69,33 @@ constexpr int kScanWin = 64;  // thresholds one tile may span, staged in shared 
 // allows, each thread from there to the first one its 16 ranks allow, and only
 // then each cell tests margins.  (The first tile of 128^3 spans over 1000 of
 // 2000 points; with every cell testing all of the tile's points it took 1.06 ms.)
+// Largest j in (jall, js] whose margin at (u, v) is not negative, jall if none,
+// for the lanes that ask: lane after lane, the warp testing 32 points at once.
+// (One lane stepping down 253 points for each of its cells took 120 us.)
+static __device__ __noinline__ int lin_walk_far(const ScanArgs& a, bool head, float u, float v, int js, int jall,
+                                                bool far) {
+  const int lane = threadIdx.x & 31;
+  unsigned need = __ballot_sync(0xffffffffu, far);
+  while (need) {
+    const int src = __ffs(need) - 1;
+    need &= need - 1;
+    const float us = __shfl_sync(0xffffffffu, u, src), vs = __shfl_sync(0xffffffffu, v, src);
+    const float* C = __shfl_sync(0xffffffffu, (int)head, src) ? a.linP : a.linQ;
+    int found = jall;
+    for (int top = __shfl_sync(0xffffffffu, js, src); top > jall; top -= 32) {
+      const int j = top - lane;
+      const unsigned m = __ballot_sync(
+          0xffffffffu, j > jall && fmaf(a.linb[max(j, 0)], vs, fmaf(a.lina[max(j, 0)], us, C[max(j, 0)])) >= 0.0f);
+      if (m) {
+        found = top - (__ffs(m) - 1);
+        break;
+      }
+    }
+    if (lane == src) js = found;
+  }
+  return js;
+}
+
 struct ScanShared {
   int s_jall, s_jtop;
   int s_cx[3];  // c(M_last), c(M_first), first staged threshold (-1: none)
@@ -397,17 +424,33 @@ __device__ __forceinline__ void scan_tile(const ScanArgs& a, ScanShared& S, Look
     }
     if (tid * IT < cnt) {
       const Box cb = box_of(start + (uint32_t)(tid * IT), start + (uint32_t)min((tid + 1) * IT, cnt), Mn, Mn + run);
-      for (; jt > jall; --jt) {
+      // mostly a step or two; a long way down eight points at a time, so that
+      // their loads overlap
+      unsigned hit = 0;
+      for (int steps = 0; jt > jall && steps < 6; ++steps, --jt) {
         float hmin, hmax, tol;
         classify(cb, jt, hmin, hmax, tol);
-        if (hmax >= -tol) break;
+        if (hmax >= -tol) {
+          hit = 1;
+          break;
+        }
       }
+#pragma unroll 1
+      for (; jt > jall && !hit; jt -= hit ? __ffs(hit) - 1 : 8) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          float hmin, hmax, tol;
+          classify(cb, max(jt - k, 0), hmin, hmax, tol);
+          hit |= (jt - k > jall && hmax >= -tol) ? 1u << k : 0u;
+        }
+      }
+      jt = max(jt, jall);
     }
 #pragma unroll
     for (int i = 0; i < IT; ++i) {
       const int p = tid * IT + i;
-      if (p >= cnt) continue;
-      Mn += mass_fix(mv[i], qs);
+      const bool ok = p < cnt;
+      if (ok) Mn += mass_fix(mv[i], qs);
       // the cell's own form (a tile can straddle the middle rank; the boxes'
       // classification above carries a tolerance for either form)
       const uint32_t rank1 = start + (uint32_t)p + 1u;
@@ -417,8 +460,12 @@ __device__ __forceinline__ void scan_tile(const ScanArgs& a, ScanShared& S, Look
       const float uu = cs * (chead ? (float)rank1 : (float)(n - rank1));
       const float vv = cs * (chead ? u64_to_float(Mn) * qinv : u64_to_float(qT - Mn) * qinv);
       auto h = [&](int j) { return fmaf(a.linb[j], vv, fmaf(a.lina[j], uu, cC[j])); };
-      int js = jt;
-      while (js > jall && !(h(js) >= 0.0f)) --js;
+      int js = ok ? jt : jall, steps = 0;
+      while (js > jall && steps < 24 && !(h(js) >= 0.0f)) --js, ++steps;
+      // a long way down (the first ranks, and deep voids at the end): 32 points at once
+      const bool far = steps == 24 && js > jall;
+      if (__any_sync(0xffffffffu, far)) js = lin_walk_far(a, chead, uu, vv, js, jall, far);
+      if (!ok) continue;
       float z;
       if (js < 0) z = a.z_lo;
       else if (js == M - 1) z = a.z_hi;

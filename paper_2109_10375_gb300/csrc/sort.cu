@@ -34,6 +34,7 @@
 #include <type_traits>
 
 #include "fixed128.cuh"
+#include "msd.cuh"
 #include "sort.cuh"
 
 namespace amber {
@@ -467,7 +468,7 @@ __device__ __forceinline__ void sort_pass_body(const PassArgs& a) {
   }
   __syncthreads();
   if constexpr (FIRST && MASS) {
-    if (tid == 0) {
+    if (tid == 0 && a.tile_mass) {
       u128 t = 0;
 #pragma unroll
       for (int w = 0; w < NW; ++w) t += wmass[w];
@@ -515,6 +516,82 @@ __global__ void __launch_bounds__(kSortThreads, AMBER_SORT_MINB)
 }
 
 // ---------------------------------------------------------------------------
+// The digit passes as the fallback of the ranking by splitting (msd.cu): one
+// cooperative launch that ends at once unless a bucket overflowed, so that it
+// costs every other ranking one short launch instead of six.
+// ---------------------------------------------------------------------------
+// All CTAs of the (cooperative) grid have arrived `round` times; false when the
+// bounded wait ran out.
+__device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t round, unsigned spin_limit, unsigned* status) {
+  __shared__ int s_ok;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    atomicAdd(bar, 1u);
+    unsigned spins = 0;
+    s_ok = 1;
+    while (ld_acquire_u32(bar) < round * gridDim.x) {
+      if (++spins >= spin_limit) {
+        raise_status(status, AMBER_ERR_DEVICE_TIMEOUT);
+        s_ok = 0;
+        break;
+      }
+      __nanosleep(200);
+    }
+    __threadfence();
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
+template <bool MASS>
+__global__ void __launch_bounds__(kSortThreads, 2) k_sort_fallback(const FallbackArgs f) {
+  constexpr int RB = 8;
+  const uint32_t fell = *reinterpret_cast<volatile uint32_t*>(&f.mc->overflow);
+  if (fell == 0) return;
+  uint32_t round = 0;
+  unsigned* status = f.pass[0].status;
+  if (!(fell & 1u) && (f.J_restore || f.mass_restore)) {
+    const uint32_t kbase = msd_range(f.hist.ctrl).kbase;
+    const int64_t slots = (int64_t)f.nb1 * f.cap1;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < slots; i += (int64_t)gridDim.x * blockDim.x) {
+      const uint32_t d = (uint32_t)(i / f.cap1);
+      if ((uint32_t)(i - (int64_t)d * f.cap1) >= f.mc->cnt1[d]) continue;
+      const uint2 v = f.kv1[i];
+      const uint32_t u = ~(v.x + kbase);  // undo the key's flips
+      if (f.J_restore) f.J_restore[v.y] = __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
+      if (MASS && f.mass_restore) f.mass_restore[v.y] = f.mass1[i];
+    }
+    if (!grid_barrier(&f.mc->bar, ++round, kSpinLimit, status)) return;
+  }
+  sort_histogram_body<float, RB>(reinterpret_cast<const float*>(f.hist.J), f.hist.n, f.hist.ctrl, f.hist.lb0,
+                                 f.hist.lb0_words, blockIdx.x, gridDim.x);
+  if (!grid_barrier(&f.mc->bar, ++round, kSpinLimit, status)) return;
+  if (blockIdx.x == 0) sort_offsets_body<float, RB>(f.hist.ctrl);
+  if (!grid_barrier(&f.mc->bar, ++round, kSpinLimit, status)) return;
+  for (int p = 0; p < 4; ++p) {
+    // as many calls as tiles over the whole grid; each takes one ticket
+    for (int64_t t = blockIdx.x; t < f.tiles; t += gridDim.x) {
+      if (p == 0) sort_pass_body<float, RB, true, MASS, false>(f.pass[0]);
+      else sort_pass_body<float, RB, false, MASS, false>(f.pass[p]);
+      __syncthreads();
+    }
+    if ((p < 3 || f.order_to) && !grid_barrier(&f.mc->bar, ++round, kSpinLimit, status)) return;
+  }
+  if (f.order_to) {
+    // pass p writes the A side if p is even
+    const int last = f.hist.ctrl->npasses - 1;
+    const uint32_t* v = f.pass[last].vout;
+    const float* m = f.pass[last].mout;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < f.hist.n;
+         i += (int64_t)gridDim.x * blockDim.x) {
+      f.order_to[i] = v[i];
+      if (MASS) f.mass_to[i] = m[i];
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Host side.
 // ---------------------------------------------------------------------------
 template <typename SRC, int RB> static size_t pass_smem(bool mass) {
@@ -540,7 +617,7 @@ static void launch_pass_v(const PassArgs& a, int64_t tiles, cudaStream_t s) {
 // GB300 the ballots are faster (35.2 vs 37.7 ms for the three passes at
 // 1024^3).  The caller (the context's tuning) picks; AMBER_SORT_RANK=
 // ballot|match overrides it.
-static int rank_env() {
+int sort_rank_env() {
   static const int m = [] {
     const char* v = getenv("AMBER_SORT_RANK");
     return !v ? -1 : strcmp(v, "match") == 0 ? 1 : strcmp(v, "ballot") == 0 ? 0 : -1;
@@ -558,6 +635,13 @@ cudaError_t sort_ctrl_reset(SortCtrl* ctrl, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(ctrl, 0, sizeof(SortCtrl), s);
   if (e != cudaSuccess) return e;
   return cudaMemsetAsync(&ctrl->kmin, 0xff, sizeof(ctrl->kmin), s);
+}
+
+cudaError_t key_range_impl(const float* J, int64_t n, SortCtrl* ctrl, int num_sms, unsigned int* status,
+                           cudaStream_t s) {
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((n / 4 + 255) / 256, (int64_t)num_sms * 8));
+  k_key_range<float><<<grid, 256, 0, s>>>(J, n, ctrl, status);
+  return cudaGetLastError();
 }
 
 template <typename SRC, int RB>
@@ -641,7 +725,7 @@ cudaError_t rank_impl(const SortWork& w, const SRC* J, int64_t n, uint32_t* orde
                       float* mass_out, unsigned long long* tile_mass, bool range_ready, unsigned int* status,
                       cudaStream_t s, FftProfile* prof, unsigned int spin_limit, int digit_bits, int match,
                       bool hist_ready) {
-  const int env = rank_env();
+  const int env = sort_rank_env();
   const bool m = env >= 0 ? env == 1 : match == 1;
   if (digit_bits == 0) digit_bits = KeyOf<SRC>::RB;
   if constexpr (sizeof(SRC) == 4) {
@@ -709,6 +793,26 @@ int rank_args(const SortWork& w, const SRC* J, int64_t n, uint32_t* order, const
   return P;
 }
 
+template <bool MASS> static cudaError_t launch_fallback(const FallbackArgs& f, int num_sms, cudaStream_t s) {
+  const size_t smem = pass_smem<float, 8>(MASS);
+  static std::atomic<unsigned long long> attr{0};  // per instantiation and device
+  static std::atomic<int> per_sm{0};
+  if (first_use_on_device(attr)) {
+    cudaFuncSetAttribute(k_sort_fallback<MASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sort_fallback<MASS>, kSortThreads, smem) == cudaSuccess)
+      per_sm = b;
+  }
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const unsigned grid = (unsigned)std::min<int64_t>(f.tiles, (int64_t)num_sms * per_sm);
+  void* args[] = {const_cast<FallbackArgs*>(&f)};
+  return cudaLaunchCooperativeKernel(k_sort_fallback<MASS>, dim3(grid), dim3(kSortThreads), args, smem, s);
+}
+
+cudaError_t sort_fallback(const FallbackArgs& f, bool with_mass, int num_sms, cudaStream_t s) {
+  return with_mass ? launch_fallback<true>(f, num_sms, s) : launch_fallback<false>(f, num_sms, s);
+}
+
 template <int RB, bool FIRST, bool MATCH>
 static void launch_pass_multi(const RankMulti& r, int p, cudaStream_t s) {
   const size_t smem = pass_smem<float, RB>(true);
@@ -737,7 +841,7 @@ static cudaError_t rank_multi_rb(const RankMulti& r, bool match, cudaStream_t s)
 }
 
 cudaError_t rank_multi(const RankMulti& r, int digit_bits, bool match, cudaStream_t s) {
-  const int env = rank_env();
+  const int env = sort_rank_env();
   const bool m = env >= 0 ? env == 1 : match;
   if (digit_bits == 8) return rank_multi_rb<8>(r, m, s);
   if (digit_bits == 9) return rank_multi_rb<9>(r, m, s);

@@ -97,6 +97,10 @@ cudaError_t rank_multi(const RankMulti& r, int digit_bits, bool match, cudaStrea
 
 int64_t sort_tiles(int64_t n);
 size_t sort_lookback_words(int64_t n);
+// AMBER_SORT_RANK: 0 ballot, 1 match (digit passes asked for), -1 unset
+int sort_rank_env();
+// the key range of J folded into ctrl (reset beforehand)
+cudaError_t key_range_impl(const float* J, int64_t n, SortCtrl* ctrl, int num_sms, unsigned int* status, cudaStream_t s);
 cudaError_t sort_ctrl_reset(SortCtrl* ctrl, cudaStream_t s);
 
 // Stable descending rank of J into order.  With mass_in != NULL the masses
