@@ -1168,8 +1168,12 @@ struct amber_batch {
 };
 
 
-int amber_batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, const amber_batch_item* items,
-                       int nitems) {
+constexpr int kBatchSplitN = 256;
+
+// split: the 256^3 items are ranked by splitting (over 2 words per cell more
+// workspace than the digit passes).
+static int batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, const amber_batch_item* items, int nitems,
+                        bool split) {
   if (!out || !ctxs || nctx < 1 || !items || nitems < 1) return AMBER_ERR_INVALID_ARG;
   *out = nullptr;
   amber_ctx* c0 = ctxs[0];
@@ -1213,13 +1217,26 @@ int amber_batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, cons
     size_t J, kA, iA, iB, mA, mB, spec, lb, actrl, Xq, inv, lin, state, btab, tmass;
     int64_t sort_tiles, scan_tiles;
     int nbuckets;
+    bool msd;
+    MsdPlan plan;
+    size_t mc, cnt2;
   };
   std::vector<ItemWs> iw(nitems);
-  int64_t cells = 0;
-  for (int i : ord) cells += (int64_t)items[i].params.n * items[i].params.n * items[i].params.n;
+  int64_t cells = 0, digit_cells = 0;
+  for (int i : ord) {
+    ItemWs& w = iw[i];
+    w.C = (int64_t)items[i].params.n * items[i].params.n * items[i].params.n;
+    // Several rankings by splitting share their launches where they are of one
+    // size and matched in place: 256^3.  Smaller grids stay with the digit
+    // passes, which take mixed sizes in one launch.
+    w.msd = split && items[i].params.n == kBatchSplitN && sort_rank_env() < 0;
+    if (w.msd) w.plan = msd_plan(w.C, true, c0->num_sms);
+    cells += w.C;
+    if (!w.msd) digit_cells += w.C;
+  }
   // per-cell arrays: one run per kind, items in size order
-  const size_t offJ = L.take(cells * 4), offKA = L.take(cells * 4), offIA = L.take(cells * 4),
-               offIB = L.take(cells * 4), offMA = L.take(cells * 4), offMB = L.take(cells * 4);
+  const size_t offJ = L.take(cells * 4), offKA = L.take(digit_cells * 4), offIA = L.take(digit_cells * 4),
+               offIB = L.take(digit_cells * 4), offMA = L.take(digit_cells * 4), offMB = L.take(digit_cells * 4);
   size_t spec_total = 0;
   for (int i : ord) {
     const int n = items[i].params.n;
@@ -1229,18 +1246,30 @@ int amber_batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, cons
   const size_t offCtrl = L.take((size_t)nitems * sizeof(SortCtrl));  // one control block per item, in size order
   const size_t offACtrl = L.take((size_t)nitems * kAssignCtrlBytes);
   {
-    int64_t co = 0;
+    int64_t co = 0, dco = 0;
     size_t so = 0;
     for (int i : ord) {
       const int n = items[i].params.n;
       ItemWs& w = iw[i];
-      w.C = (int64_t)n * n * n;
       w.J = offJ + co * 4;
-      w.kA = offKA + co * 4;
-      w.iA = offIA + co * 4;
-      w.iB = offIB + co * 4;
-      w.mA = offMA + co * 4;
-      w.mB = offMB + co * 4;
+      if (w.msd) {
+        // the buckets' regions, over which the fallback's five arrays lie
+        const MsdPlan& q = w.plan;
+        w.kA = L.take((size_t)std::max<int64_t>(q.kv1 + q.m1 + q.kv2 + q.m2, 5 * w.C) * 4);
+        w.iA = w.kA + w.C * 4;
+        w.iB = w.iA + w.C * 4;
+        w.mA = w.iB + w.C * 4;
+        w.mB = w.mA + w.C * 4;
+        w.mc = L.take(sizeof(MsdCtrl));
+        w.cnt2 = L.take((size_t)q.nb1 * q.nb2 * 4);
+      } else {
+        w.kA = offKA + dco * 4;
+        w.iA = offIA + dco * 4;
+        w.iB = offIB + dco * 4;
+        w.mA = offMA + dco * 4;
+        w.mB = offMB + dco * 4;
+        dco += w.C;
+      }
       w.spec = offSpec + so;
       co += w.C;
       so += (size_t)n * n * (n / 2 + 2) * 8;
@@ -1250,7 +1279,7 @@ int amber_batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, cons
   for (int i : ord) {
     ItemWs& w = iw[i];
     w.sort_tiles = sort_tiles(w.C);
-    w.scan_tiles = (w.C + kScanTile - 1) / kScanTile;
+    w.scan_tiles = w.msd ? (int64_t)w.plan.nb1 * w.plan.nb2 : (w.C + kScanTile - 1) / kScanTile;
     int shift;
     bucket_plan(w.C, &w.nbuckets, &shift);
     state_total += align256((size_t)w.scan_tiles * 8);
@@ -1266,8 +1295,8 @@ int amber_batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, cons
       w.Xq = L.take((size_t)hcs[i].n_table * 8);
       w.inv = L.take((size_t)hcs[i].n_table * 4);
       w.lin = L.take((size_t)4 * kMaxTable * 4);
-      w.btab = L.take((size_t)w.scan_tiles * (w.nbuckets + 1) * 2);
-      w.tmass = L.take((size_t)w.sort_tiles * 16);
+      w.btab = w.msd ? 0 : L.take((size_t)w.scan_tiles * (w.nbuckets + 1) * 2);
+      w.tmass = L.take((size_t)w.sort_tiles * 16);  // (or the sums of a split's CTAs, fewer)
     }
   }
   // per-item argument arrays (device copies of host-built structs)
@@ -1276,8 +1305,9 @@ int amber_batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, cons
     const int n = items[i].params.n;
     if (sizes.empty() || sizes.back() != n) sizes.push_back(n);
   }
-  for (int n : sizes) {
-    const int rb = c0->tune[ilog2i(n)].sort_digit_bits;
+  for (int i : ord) {
+    if (iw[i].msd) continue;
+    const int rb = c0->tune[ilog2i(items[i].params.n)].sort_digit_bits;
     if (std::find(rbs.begin(), rbs.end(), rb) == rbs.end()) rbs.push_back(rb);
   }
   amber_batch* b = new (std::nothrow) amber_batch();
@@ -1366,7 +1396,7 @@ int amber_batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, cons
     for (int k = 0; k < nitems; ++k) {
       const int i = ord[k];
       const amber_tuning_t& tu = c0->tune[ilog2i(items[i].params.n)];
-      if (tu.sort_digit_bits != rb) continue;
+      if (iw[i].msd || tu.sort_digit_bits != rb) continue;
       q.match = tu.sort_match;
       HistArgs h;
       uint32_t hb;
@@ -1389,12 +1419,17 @@ int amber_batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, cons
   }
   // ---- matching: thresholds and scatter for every item, scans per weighting form
   AssignMulti am{};
+  MsdMulti mm{};
+  size_t o_margs = 0, o_mscan = 0, o_mfall = 0;
   size_t o_thresh, o_scan[2], o_spre[2], o_scatter, o_xpre;
   {
     std::vector<ThreshArgs> th;
     std::vector<ScanArgs> sc[2];
     std::vector<uint32_t> spre[2] = {{0}, {0}}, xpre{0};
     std::vector<ScatterArgs> xs;
+    std::vector<MsdArgs> margs[2];
+    std::vector<ScanArgs> mscan[2];
+    std::vector<FallbackArgs> mfall[2];
     for (int k = 0; k < nitems; ++k) {
       const int i = ord[k];
       ThreshArgs ta;
@@ -1402,8 +1437,53 @@ int amber_batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, cons
       ScatterArgs xa;
       assign_args(aw[i], sw[i].idxA, sw[i].massA, tile_mass[i], iw[i].C, hcs[i], items[i].d_zre, nullptr, c0->status,
                   kSpinLimit, sw[i].idxB, sw[i].massB, &sw[i].ctrl->npasses, &ta, &sa, &xa);
-      th.push_back(ta);
       const int f = hcs[i].weighting != AMBER_WEIGHT_MASS ? 1 : 0;
+      if (iw[i].msd) {
+        const MsdPlan& q = iw[i].plan;
+        ta.ntiles = msd_split_ctas(iw[i].C, q, c0->num_sms);
+        th.push_back(ta);
+        sa.zre = items[i].d_zre;
+        MsdArgs m{};
+        m.J = reinterpret_cast<const float*>(sw[i].keysB);
+        m.mass = items[i].d_mass;
+        m.n = iw[i].C;
+        uint32_t* at = reinterpret_cast<uint32_t*>(W + iw[i].kA);
+        m.kv1 = reinterpret_cast<uint2*>(at);
+        m.mass1 = reinterpret_cast<float*>(at + q.kv1);
+        m.kv2 = reinterpret_cast<uint2*>(at + q.kv1 + q.m1);
+        m.mass2 = reinterpret_cast<float*>(at + q.kv1 + q.m1 + q.kv2);
+        m.cap1 = q.cap1;
+        m.nb1 = q.nb1;
+        m.nb2 = q.nb2;
+        m.idx_shift = q.idx_shift;
+        m.digit_bits = c0->tune[ilog2i(items[i].params.n)].sort_digit_bits;
+        m.ctrl = sw[i].ctrl;
+        m.mc = reinterpret_cast<MsdCtrl*>(W + iw[i].mc);
+        m.cnt2 = reinterpret_cast<uint32_t*>(W + iw[i].cnt2);
+        m.cta_mass = tile_mass[i];
+        m.status = c0->status;
+        m.actrl = aw[i].ctrl;
+        m.state = aw[i].state;
+        m.fb_order[0] = sw[i].idxA;
+        m.fb_order[1] = sw[i].idxB;
+        m.fb_mass[0] = sw[i].massA;
+        m.fb_mass[1] = sw[i].massB;
+        FallbackArgs fb{};
+        uint32_t blocks;
+        fb.mc = m.mc;
+        rank_args<float>(sw[i], m.J, m.n, nullptr, m.mass, nullptr, nullptr, c0->status, kSpinLimit, 8, &fb.hist,
+                         &blocks, fb.pass);
+        fb.tiles = sort_tiles(m.n);
+        margs[f].push_back(m);
+        mscan[f].push_back(sa);
+        mfall[f].push_back(fb);
+        mm.split_ctas = (int)ta.ntiles;
+        mm.buckets = (int)(q.nb1 * q.nb2);
+        mm.two_splits = q.nb2 > 1;
+        mm.tiles = fb.tiles;
+        continue;
+      }
+      th.push_back(ta);
       sc[f].push_back(sa);
       spre[f].push_back(spre[f].back() + (uint32_t)iw[i].scan_tiles);
       xs.push_back(xa);
@@ -1418,6 +1498,15 @@ int amber_batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, cons
       o_spre[f] = place(spre[f]);
     }
     am.scatter_blocks = xpre.back();
+    am.Ms = (int)xs.size();
+    for (int f = 0; f < 2; ++f) mm.Mg[f] = (int)margs[f].size();
+    mm.M = mm.Mg[0] + mm.Mg[1];
+    margs[0].insert(margs[0].end(), margs[1].begin(), margs[1].end());
+    mscan[0].insert(mscan[0].end(), mscan[1].begin(), mscan[1].end());
+    mfall[0].insert(mfall[0].end(), mfall[1].begin(), mfall[1].end());
+    o_margs = place(margs[0]);
+    o_mscan = place(mscan[0]);
+    o_mfall = place(mfall[0]);
     o_thresh = place(th);
     o_scatter = place(xs);
     o_xpre = place(xpre);
@@ -1432,6 +1521,11 @@ int amber_batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, cons
     am.scan[f] = reinterpret_cast<const ScanArgs*>(G + o_scan[f]);
     am.scan_prefix[f] = reinterpret_cast<const uint32_t*>(G + o_spre[f]);
   }
+  mm.args = reinterpret_cast<const MsdArgs*>(G + o_margs);
+  mm.scans = reinterpret_cast<const ScanArgs*>(G + o_mscan);
+  mm.fallback = reinterpret_cast<const FallbackArgs*>(G + o_mfall);
+  for (int i = 0; i < nitems; ++i)
+    if (iw[i].msd && e == cudaSuccess) e = cudaMemset(W + iw[i].mc, 0, sizeof(MsdCtrl));
   am.scatter = reinterpret_cast<const ScatterArgs*>(G + o_scatter);
   am.scatter_prefix = reinterpret_cast<const uint32_t*>(G + o_xpre);
   for (SortGroup& q : sg) {
@@ -1466,9 +1560,14 @@ int amber_batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, cons
   }
   for (const SortGroup& q : sg)
     if (e == cudaSuccess) e = rank_multi(q.r, q.rb, q.match == 1, origin);
+  if (e == cudaSuccess && mm.M) e = msd_multi(mm, c0->num_sms, origin);
   if (e == cudaSuccess) e = cudaMemsetAsync(W + offACtrl, 0, (size_t)nitems * kAssignCtrlBytes, origin);
   if (e == cudaSuccess) e = cudaMemsetAsync(W + offState, 0, state_total, origin);
   if (e == cudaSuccess) e = assign_multi(am, origin);
+  if (e == cudaSuccess && mm.M) {
+    msd_multi_match(mm, origin);
+    e = cudaGetLastError();
+  }
   if (capturing) {
     const cudaError_t e2 = cudaStreamEndCapture(origin, &b->graph);
     if (e == cudaSuccess) e = e2;
@@ -1497,6 +1596,13 @@ int amber_batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, cons
   }
   *out = b;
   return AMBER_OK;
+}
+
+int amber_batch_create(amber_batch** batch, amber_ctx* const* ctxs, int nctx, const amber_batch_item* items,
+                       int nitems) {
+  // where the buckets' regions do not fit the device's memory, the digit passes
+  const int st = batch_create(batch, ctxs, nctx, items, nitems, true);
+  return st == AMBER_ERR_OOM ? batch_create(batch, ctxs, nctx, items, nitems, false) : st;
 }
 
 int amber_batch_launch(amber_batch* b, void* stream) {

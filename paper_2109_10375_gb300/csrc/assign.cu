@@ -599,7 +599,7 @@ cudaError_t assign_multi(const AssignMulti& m, cudaStream_t s) {
                        kThreshThreads, 0, s>>>(m.thresh);
   if (m.scan_tiles[0]) k_scan_assign_multi<false><<<m.scan_tiles[0], kScanThreads, 0, s>>>(m.scan[0], m.scan_prefix[0], m.Mg[0]);
   if (m.scan_tiles[1]) k_scan_assign_multi<true><<<m.scan_tiles[1], kScanThreads, 0, s>>>(m.scan[1], m.scan_prefix[1], m.Mg[1]);
-  k_scatter_back_multi<<<m.scatter_blocks, 256, 0, s>>>(m.scatter, m.scatter_prefix, m.M);
+  if (m.scatter_blocks) k_scatter_back_multi<<<m.scatter_blocks, 256, 0, s>>>(m.scatter, m.scatter_prefix, m.Ms);
   return cudaGetLastError();
 }
 

@@ -132,6 +132,7 @@ struct AssignMulti {
   const uint32_t* scan_prefix[2];
   int Mg[2];
   uint32_t scan_tiles[2];
+  int Ms;  // items with a scatter
   const ScatterArgs* scatter;
   const uint32_t* scatter_prefix;
   uint32_t scatter_blocks;

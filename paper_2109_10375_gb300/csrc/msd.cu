@@ -38,12 +38,14 @@
 
 namespace amber {
 
-__global__ void __launch_bounds__(1024) k_msd_map(const MsdArgs a) {
+// Each kernel's work is that of CTA blk of nblk on one ranking: of the launch, or
+// (k_msd_*_multi) of the launch's row blockIdx.y, one ranking each.
+__device__ __forceinline__ void msd_map_body(const MsdArgs& a, uint32_t blk, uint32_t nblk) {
   __shared__ uint32_t h[kMsdKnots];
   __shared__ uint32_t s_last, wsum[32];
   const int tid = threadIdx.x, NT = blockDim.x;
   for (int i = tid; i < kMsdKnots; i += NT) h[i] = 0;
-  const uint32_t gt = blockIdx.x * NT + tid, ng = gridDim.x * NT;
+  const uint32_t gt = blk * NT + tid, ng = nblk * NT;
   for (uint32_t i = gt; i < a.nb1; i += ng) a.mc->cnt1[i] = 0;
   if (a.nb2 > 1)
     for (uint32_t i = gt; i < a.nb1 * a.nb2; i += ng) a.cnt2[i] = 0;
@@ -93,7 +95,7 @@ __global__ void __launch_bounds__(1024) k_msd_map(const MsdArgs a) {
     if (h[i]) atomicAdd(&a.mc->hist[i], h[i]);
   __threadfence();
   __syncthreads();
-  if (tid == 0) s_last = atomicAdd(&a.mc->done, 1u) == gridDim.x - 1;
+  if (tid == 0) s_last = atomicAdd(&a.mc->done, 1u) == nblk - 1;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
@@ -131,6 +133,15 @@ __global__ void __launch_bounds__(1024) k_msd_map(const MsdArgs a) {
   }
 }
 
+__global__ void __launch_bounds__(1024) k_msd_map(const MsdArgs a) { msd_map_body(a, blockIdx.x, gridDim.x); }
+
+__global__ void __launch_bounds__(1024) k_msd_map_multi(const MsdArgs* __restrict__ args) {
+  __shared__ MsdArgs a;
+  if (threadIdx.x == 0) a = args[blockIdx.y];
+  __syncthreads();
+  msd_map_body(a, blockIdx.x, gridDim.x);
+}
+
 // Sum of the first `warp` entries of per-warp totals (at most 32 of them).
 __device__ __forceinline__ uint32_t warps_before(const uint32_t* wsum, int nw, int lane, int warp) {
   return __reduce_add_sync(0xffffffffu, lane < nw && lane < warp ? wsum[lane] : 0u);
@@ -153,7 +164,7 @@ struct MassSum {
 };
 
 template <int NT, int IT, bool FIRST, bool MASS>
-__global__ void __launch_bounds__(NT, 1024 / NT) k_msd_split(const MsdArgs a) {
+__device__ __forceinline__ void msd_split_body(const MsdArgs& a, uint32_t blk, uint32_t nblk) {
   constexpr int TILE = NT * IT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint4* rec = reinterpret_cast<uint4*>(smem_raw);               // [TILE] (key, cell, mass, digit)
@@ -181,7 +192,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_msd_split(const MsdArgs a) {
   float* __restrict__ mo = FIRST ? a.mass1 : a.mass2;
   bool bad = false;
   MassSum msum;
-  for (uint32_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+  for (uint32_t tile = blk; tile < tiles; tile += nblk) {
     uint32_t start, have, bucket = 0;
     if (FIRST) {
       start = tile * (uint32_t)TILE;
@@ -310,18 +321,31 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_msd_split(const MsdArgs a) {
     if (tid == 0) {
       t = 0;
       for (int w = 0; w < NT / 32; ++w) t += wmass[w];
-      a.cta_mass[2 * blockIdx.x] = (unsigned long long)t;
-      a.cta_mass[2 * blockIdx.x + 1] = (unsigned long long)(t >> 64);
+      a.cta_mass[2 * blk] = (unsigned long long)t;
+      a.cta_mass[2 * blk + 1] = (unsigned long long)(t >> 64);
     }
   }
   if (FIRST && __any_sync(0xffffffffu, bad) && lane == 0)
     raise_status(a.status, MASS ? (AMBER_ERR_NONFINITE | AMBER_ERR_INVALID_MASS) : AMBER_ERR_NONFINITE);
 }
 
+template <int NT, int IT, bool FIRST, bool MASS>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_msd_split(const MsdArgs a) {
+  msd_split_body<NT, IT, FIRST, MASS>(a, blockIdx.x, gridDim.x);
+}
+
+template <bool FIRST>
+__global__ void __launch_bounds__(512, 2) k_msd_split_multi(const MsdArgs* __restrict__ args) {
+  __shared__ MsdArgs a;
+  if (threadIdx.x == 0) a = args[blockIdx.y];
+  __syncthreads();
+  msd_split_body<512, kMsdTileA / 512, FIRST, true>(a, blockIdx.x, gridDim.x);
+}
+
 // SCAN: with the masses, matched here as well (LIN: see scan.cuh), each redshift
 // stored in its place.
 template <bool MASS, bool SCAN, bool LIN>
-__global__ void __launch_bounds__(kMsdLocalThreads, 2) k_msd_local(const MsdArgs a, const ScanArgs sa) {
+__device__ __forceinline__ void msd_local_body(const MsdArgs& a, const ScanArgs& sa) {
   constexpr int NT = kMsdLocalThreads, IT = kMsdLocalItems, CAP = kMsdCap, S = kMsdSub;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned long long* comp = reinterpret_cast<unsigned long long*>(smem_raw);  // [CAP]
@@ -582,6 +606,22 @@ __global__ void __launch_bounds__(kMsdLocalThreads, 2) k_msd_local(const MsdArgs
   }
 }
 
+template <bool MASS, bool SCAN, bool LIN>
+__global__ void __launch_bounds__(kMsdLocalThreads, 2) k_msd_local(const MsdArgs a, const ScanArgs sa) {
+  msd_local_body<MASS, SCAN, LIN>(a, sa);
+}
+
+template <bool LIN>
+__global__ void __launch_bounds__(kMsdLocalThreads, 2)
+    k_msd_local_multi(const MsdArgs* __restrict__ args, const ScanArgs* __restrict__ scans) {
+  __shared__ MsdArgs a;
+  __shared__ ScanArgs sa;
+  if (threadIdx.x == 0) a = args[blockIdx.y];
+  if (threadIdx.x == 32) sa = scans[blockIdx.y];
+  __syncthreads();
+  msd_local_body<true, true, LIN>(a, sa);
+}
+
 // ---------------------------------------------------------------------------
 // Host side.
 // ---------------------------------------------------------------------------
@@ -677,6 +717,35 @@ cudaError_t msd_run(const MsdArgs& a, const FallbackArgs& f, int num_sms, const 
     prof_end(prof, PK_SORT_PASS, s);
   }
   return cudaGetLastError();
+}
+
+cudaError_t msd_multi(const MsdMulti& m, int num_sms, cudaStream_t s) {
+  constexpr size_t ssmem = (size_t)kMsdTileA * 16 + kMsdKnots * 8 + 2 * kMsdMaxDigits * 4;
+  constexpr size_t lsmem = (size_t)kMsdCap * 8 + (kMsdSub / 2 + 4) * 4;
+  static std::atomic<unsigned long long> attr{0};  // per device
+  if (first_use_on_device(attr)) {
+    cudaFuncSetAttribute(k_msd_split_multi<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem);
+    cudaFuncSetAttribute(k_msd_split_multi<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem);
+    cudaFuncSetAttribute(k_msd_local_multi<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsmem);
+    cudaFuncSetAttribute(k_msd_local_multi<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsmem);
+  }
+  const dim3 g((unsigned)m.split_ctas, (unsigned)m.M);
+  k_msd_map_multi<<<dim3((unsigned)num_sms, (unsigned)m.M), 1024, 0, s>>>(m.args);
+  k_msd_split_multi<true><<<g, 512, ssmem, s>>>(m.args);
+  if (m.two_splits) k_msd_split_multi<false><<<g, 512, ssmem, s>>>(m.args);
+  return sort_fallback_multi(m.fallback, m.M, m.tiles, num_sms, s);
+}
+
+void msd_multi_match(const MsdMulti& m, cudaStream_t s) {
+  constexpr size_t lsmem = (size_t)kMsdCap * 8 + (kMsdSub / 2 + 4) * 4;
+  for (int f = 0; f < 2; ++f) {
+    if (!m.Mg[f]) continue;
+    const dim3 g((unsigned)m.buckets, (unsigned)m.Mg[f]);
+    const MsdArgs* a = m.args + (f ? m.Mg[0] : 0);
+    const ScanArgs* sa = m.scans + (f ? m.Mg[0] : 0);
+    if (f) k_msd_local_multi<true><<<g, kMsdLocalThreads, lsmem, s>>>(a, sa);
+    else k_msd_local_multi<false><<<g, kMsdLocalThreads, lsmem, s>>>(a, sa);
+  }
 }
 
 }  // namespace amber

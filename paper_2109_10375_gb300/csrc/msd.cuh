@@ -101,6 +101,22 @@ cudaError_t sort_fallback(const FallbackArgs& f, bool with_mass, int num_sms, cu
 cudaError_t msd_run(const MsdArgs& a, const FallbackArgs& f, int num_sms, const ThreshArgs* ta, const ScanArgs* sa,
                     cudaStream_t s, FftProfile* prof);
 
+// Several rankings of one size (one or two splits over 4096-cell tiles), matched
+// in place: one launch per stage, a row of CTAs per ranking.  args, scans and
+// fallback are device arrays of M, those of the mass weighting (Mg[0]) first.
+struct MsdMulti {
+  int M, Mg[2];
+  const MsdArgs* args;
+  const ScanArgs* scans;
+  const FallbackArgs* fallback;
+  int split_ctas, buckets;
+  bool two_splits;
+  int64_t tiles;  // sort tiles of one ranking
+};
+cudaError_t msd_multi(const MsdMulti& m, int num_sms, cudaStream_t s);  // up to the fallback
+void msd_multi_match(const MsdMulti& m, cudaStream_t s);                // local sorts with the matching
+cudaError_t sort_fallback_multi(const FallbackArgs* f, int M, int64_t tiles, int num_sms, cudaStream_t s);
+
 // Knots are 2^L keys wide and aligned to them, so that no knot straddles two
 // octaves of the intensity (a float's keys are half as dense per unit value in
 // the next octave, which would bend the distribution inside the knot); kbase is

@@ -545,7 +545,7 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* bar, uint32_t round, unsi
 }
 
 template <bool MASS>
-__global__ void __launch_bounds__(kSortThreads, 2) k_sort_fallback(const FallbackArgs f) {
+__device__ __forceinline__ void sort_fallback_body(const FallbackArgs& f) {
   constexpr int RB = 8;
   const uint32_t fell = *reinterpret_cast<volatile uint32_t*>(&f.mc->overflow);
   if (fell == 0) return;
@@ -588,6 +588,23 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_sort_fallback(const Fallbac
       f.order_to[i] = v[i];
       if (MASS) f.mass_to[i] = m[i];
     }
+  }
+}
+
+template <bool MASS>
+__global__ void __launch_bounds__(kSortThreads, 2) k_sort_fallback(const FallbackArgs f) {
+  sort_fallback_body<MASS>(f);
+}
+
+// Several rankings, one after another (each with its own barrier word).
+__global__ void __launch_bounds__(kSortThreads, 2) k_sort_fallback_multi(const FallbackArgs* __restrict__ args, int M) {
+  __shared__ FallbackArgs f;
+  for (int i = 0; i < M; ++i) {
+    if (*reinterpret_cast<volatile uint32_t*>(&args[i].mc->overflow) == 0) continue;  // the same on every thread
+    __syncthreads();
+    if (threadIdx.x == 0) f = args[i];
+    __syncthreads();
+    sort_fallback_body<true>(f);
   }
 }
 
@@ -807,6 +824,22 @@ template <bool MASS> static cudaError_t launch_fallback(const FallbackArgs& f, i
   const unsigned grid = (unsigned)std::min<int64_t>(f.tiles, (int64_t)num_sms * per_sm);
   void* args[] = {const_cast<FallbackArgs*>(&f)};
   return cudaLaunchCooperativeKernel(k_sort_fallback<MASS>, dim3(grid), dim3(kSortThreads), args, smem, s);
+}
+
+cudaError_t sort_fallback_multi(const FallbackArgs* f, int M, int64_t tiles, int num_sms, cudaStream_t s) {
+  const size_t smem = pass_smem<float, 8>(true);
+  static std::atomic<unsigned long long> attr{0};  // per device
+  static std::atomic<int> per_sm{0};
+  if (first_use_on_device(attr)) {
+    cudaFuncSetAttribute(k_sort_fallback_multi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sort_fallback_multi, kSortThreads, smem) == cudaSuccess)
+      per_sm = b;
+  }
+  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+  const unsigned grid = (unsigned)std::min<int64_t>(tiles, (int64_t)num_sms * per_sm);
+  void* args[] = {&f, &M};
+  return cudaLaunchCooperativeKernel(k_sort_fallback_multi, dim3(grid), dim3(kSortThreads), args, smem, s);
 }
 
 cudaError_t sort_fallback(const FallbackArgs& f, bool with_mass, int num_sms, cudaStream_t s) {

@@ -114,3 +114,28 @@ def test_solve_in_a_captured_graph(B):
             torch.cuda.synchronize()
             assert torch.equal(z, ref)
         assert ctx.sync_status() == 0
+
+
+def test_batch_of_split_rankings(B, monkeypatch):
+    # 256^3 items share their launches (both weightings; one whose extremes
+    # overflow a bucket takes the fallback) beside a smaller grid
+    from paper_2109_10375_gb300 import synth
+    monkeypatch.setenv("AMBER_AUTOTUNE", "0")
+    items, ref = [], []
+    with B.Context(256 ** 3) as ctx:
+        for k, (n, w) in enumerate([(256, 0), (64, 1), (256, 1), (256, 0), (256, 1)]):
+            box = 100.0 * n / 128
+            S, m = synth.realisation(n, box, k, device="cuda")
+            if k == 3:
+                S = torch.randn(S.shape, generator=torch.Generator(device="cuda").manual_seed(5), device="cuda")
+            h = B.history(7.0 + 0.4 * k, 4.0, 3.0, weighting=w)
+            ref.append(ctx.solve(S, m, box, 3.0 + k, h))
+            items.append((S, m, box, 3.0 + k, h, torch.empty_like(S)))
+        batch = B.Batch([ctx], items)
+        for _ in range(2):
+            for it in items:
+                it[5].zero_()
+            batch.launch()
+            assert ctx.sync_status() == 0
+            assert all(torch.equal(it[5], r) for it, r in zip(items, ref))
+        batch.close()
