@@ -316,16 +316,21 @@ int amber_get_tuning(amber_ctx *ctx, int n, amber_tuning_t *out);
 /* Batched solves: many realisations of mixed grid sizes, every stage of
  * every item in one launch per stage, captured once into a CUDA graph.
  *  - The transforms run one launch per pass and grid size (the items of a
- *    size back to back), the ranking one histogram, one digit-offset and one
- *    launch per digit pass per digit width, the matching one thresholds, one
- *    scan per weighting form and one scatter launch for all items.  Inside a
- *    launch each CTA finds its item from a prefix of the items' tile counts;
- *    ticket-ordered kernels (digit passes, scan) take tiles from the item's
- *    own ticket, so their look-backs stay within the item.  The graph's
- *    kernel nodes number 5 per grid size plus 6 per digit width plus 3 or 4,
- *    whatever the item count (amber_batch_kernel_nodes).
+ *    size back to back).  A size of 64^3 to 256^3 with more than 2^23 cells in
+ *    all is ranked by splitting, one launch per stage and size, the last of
+ *    which also matches; the other items one histogram, one digit-offset and one
+ *    launch per digit pass per digit width, one scan per weighting form and one
+ *    scatter launch; thresholds are one launch for all.  Inside a launch each
+ *    CTA finds its item from its row of the grid or from a prefix of the items'
+ *    tile counts; ticket-ordered kernels (digit passes, scan, local sorts) take
+ *    tiles from the item's own ticket, so their look-backs stay within the
+ *    item.  The graph's kernel nodes number 5 per grid size plus 6 per digit
+ *    width plus 3 or 4, whatever the item count, with 4 to 6 for each size
+ *    ranked by splitting (amber_batch_kernel_nodes).
  *  - The batch allocates its own workspace at creation (about 30 bytes per
- *    cell of all items together, plus the items' arguments); amber_batch_create
+ *    cell of all items together, 37 for those ranked by splitting, which are
+ *    laid out for digit passes where that does not fit, plus the items'
+ *    arguments); amber_batch_create
  *    and amber_create are the only calls that allocate.
  *  - ctxs[0] gives the device, the FFT twiddles (its max_cells must hold the
  *    largest grid), the status word that amber_sync_status(ctxs[0]) reads and

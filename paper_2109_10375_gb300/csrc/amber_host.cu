@@ -1168,9 +1168,9 @@ struct amber_batch {
 };
 
 
-constexpr int kBatchSplitN = 256;
+constexpr int64_t kBatchSplitCells = (int64_t)1 << 23;
 
-// split: the 256^3 items are ranked by splitting (over 2 words per cell more
+// split: sizes with enough cells are ranked by splitting (over 2 words per cell more
 // workspace than the digit passes).
 static int batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, const amber_batch_item* items, int nitems,
                         bool split) {
@@ -1226,13 +1226,21 @@ static int batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, con
   for (int i : ord) {
     ItemWs& w = iw[i];
     w.C = (int64_t)items[i].params.n * items[i].params.n * items[i].params.n;
-    // Several rankings by splitting share their launches where they are of one
-    // size and matched in place: 256^3.  Smaller grids stay with the digit
-    // passes, which take mixed sizes in one launch.
-    w.msd = split && items[i].params.n == kBatchSplitN && sort_rank_env() < 0;
-    if (w.msd) w.plan = msd_plan(w.C, true, c0->num_sms);
     cells += w.C;
-    if (!w.msd) digit_cells += w.C;
+  }
+  for (int i : ord) {
+    // Rankings by splitting share their launches where they are of one size and
+    // matched in place (64^3 to 256^3); that size's launches, five or six, are
+    // worth it from some 10^7 cells on (16 x 256^3: 16 -> 10.6 ms of the 48-item
+    // batch).  The other items stay with the digit passes, which take mixed
+    // sizes in one launch.
+    ItemWs& w = iw[i];
+    int64_t of_size = 0;
+    for (int k : ord) of_size += items[k].params.n == items[i].params.n ? w.C : 0;
+    w.msd = split && items[i].params.n >= 64 && w.C <= kDirectMaxCells && of_size > kBatchSplitCells &&
+            sort_rank_env() < 0;
+    if (w.msd) w.plan = msd_plan(w.C, true, c0->num_sms);
+    else digit_cells += w.C;
   }
   // per-cell arrays: one run per kind, items in size order
   const size_t offJ = L.take(cells * 4), offKA = L.take(digit_cells * 4), offIA = L.take(digit_cells * 4),
@@ -1419,17 +1427,21 @@ static int batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, con
   }
   // ---- matching: thresholds and scatter for every item, scans per weighting form
   AssignMulti am{};
-  MsdMulti mm{};
-  size_t o_margs = 0, o_mscan = 0, o_mfall = 0;
+  struct SplitGroup {  // the items of one size ranked by splitting; [0] mass, [1] linear weightings
+    int n;
+    MsdMulti m;
+    std::vector<MsdArgs> args[2];
+    std::vector<ScanArgs> scan[2];
+    std::vector<FallbackArgs> fall[2];
+    size_t o_args, o_scan, o_fall;
+  };
+  std::vector<SplitGroup> split_groups;
   size_t o_thresh, o_scan[2], o_spre[2], o_scatter, o_xpre;
   {
     std::vector<ThreshArgs> th;
     std::vector<ScanArgs> sc[2];
     std::vector<uint32_t> spre[2] = {{0}, {0}}, xpre{0};
     std::vector<ScatterArgs> xs;
-    std::vector<MsdArgs> margs[2];
-    std::vector<ScanArgs> mscan[2];
-    std::vector<FallbackArgs> mfall[2];
     for (int k = 0; k < nitems; ++k) {
       const int i = ord[k];
       ThreshArgs ta;
@@ -1474,13 +1486,19 @@ static int batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, con
         rank_args<float>(sw[i], m.J, m.n, nullptr, m.mass, nullptr, nullptr, c0->status, kSpinLimit, 8, &fb.hist,
                          &blocks, fb.pass);
         fb.tiles = sort_tiles(m.n);
-        margs[f].push_back(m);
-        mscan[f].push_back(sa);
-        mfall[f].push_back(fb);
-        mm.split_ctas = (int)ta.ntiles;
-        mm.buckets = (int)(q.nb1 * q.nb2);
-        mm.two_splits = q.nb2 > 1;
-        mm.tiles = fb.tiles;
+        // (items come in size order)
+        if (split_groups.empty() || split_groups.back().n != items[i].params.n) {
+          split_groups.push_back(SplitGroup{items[i].params.n});
+          MsdMulti& mm = split_groups.back().m;
+          mm.split_ctas = (int)ta.ntiles;
+          mm.buckets = (int)(q.nb1 * q.nb2);
+          mm.two_splits = q.nb2 > 1;
+          mm.tiles = fb.tiles;
+        }
+        SplitGroup& sgp = split_groups.back();
+        sgp.args[f].push_back(m);
+        sgp.scan[f].push_back(sa);
+        sgp.fall[f].push_back(fb);
         continue;
       }
       th.push_back(ta);
@@ -1499,14 +1517,16 @@ static int batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, con
     }
     am.scatter_blocks = xpre.back();
     am.Ms = (int)xs.size();
-    for (int f = 0; f < 2; ++f) mm.Mg[f] = (int)margs[f].size();
-    mm.M = mm.Mg[0] + mm.Mg[1];
-    margs[0].insert(margs[0].end(), margs[1].begin(), margs[1].end());
-    mscan[0].insert(mscan[0].end(), mscan[1].begin(), mscan[1].end());
-    mfall[0].insert(mfall[0].end(), mfall[1].begin(), mfall[1].end());
-    o_margs = place(margs[0]);
-    o_mscan = place(mscan[0]);
-    o_mfall = place(mfall[0]);
+    for (SplitGroup& q : split_groups) {
+      for (int f = 0; f < 2; ++f) q.m.Mg[f] = (int)q.args[f].size();
+      q.m.M = q.m.Mg[0] + q.m.Mg[1];
+      q.args[0].insert(q.args[0].end(), q.args[1].begin(), q.args[1].end());
+      q.scan[0].insert(q.scan[0].end(), q.scan[1].begin(), q.scan[1].end());
+      q.fall[0].insert(q.fall[0].end(), q.fall[1].begin(), q.fall[1].end());
+      q.o_args = place(q.args[0]);
+      q.o_scan = place(q.scan[0]);
+      q.o_fall = place(q.fall[0]);
+    }
     o_thresh = place(th);
     o_scatter = place(xs);
     o_xpre = place(xpre);
@@ -1521,9 +1541,11 @@ static int batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, con
     am.scan[f] = reinterpret_cast<const ScanArgs*>(G + o_scan[f]);
     am.scan_prefix[f] = reinterpret_cast<const uint32_t*>(G + o_spre[f]);
   }
-  mm.args = reinterpret_cast<const MsdArgs*>(G + o_margs);
-  mm.scans = reinterpret_cast<const ScanArgs*>(G + o_mscan);
-  mm.fallback = reinterpret_cast<const FallbackArgs*>(G + o_mfall);
+  for (SplitGroup& q : split_groups) {
+    q.m.args = reinterpret_cast<const MsdArgs*>(G + q.o_args);
+    q.m.scans = reinterpret_cast<const ScanArgs*>(G + q.o_scan);
+    q.m.fallback = reinterpret_cast<const FallbackArgs*>(G + q.o_fall);
+  }
   for (int i = 0; i < nitems; ++i)
     if (iw[i].msd && e == cudaSuccess) e = cudaMemset(W + iw[i].mc, 0, sizeof(MsdCtrl));
   am.scatter = reinterpret_cast<const ScatterArgs*>(G + o_scatter);
@@ -1560,14 +1582,16 @@ static int batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, con
   }
   for (const SortGroup& q : sg)
     if (e == cudaSuccess) e = rank_multi(q.r, q.rb, q.match == 1, origin);
-  if (e == cudaSuccess && mm.M) e = msd_multi(mm, c0->num_sms, origin);
+  for (const SplitGroup& q : split_groups)
+    if (e == cudaSuccess) e = msd_multi(q.m, c0->num_sms, origin);
   if (e == cudaSuccess) e = cudaMemsetAsync(W + offACtrl, 0, (size_t)nitems * kAssignCtrlBytes, origin);
   if (e == cudaSuccess) e = cudaMemsetAsync(W + offState, 0, state_total, origin);
   if (e == cudaSuccess) e = assign_multi(am, origin);
-  if (e == cudaSuccess && mm.M) {
-    msd_multi_match(mm, origin);
-    e = cudaGetLastError();
-  }
+  for (const SplitGroup& q : split_groups)
+    if (e == cudaSuccess) {
+      msd_multi_match(q.m, origin);
+      e = cudaGetLastError();
+    }
   if (capturing) {
     const cudaError_t e2 = cudaStreamEndCapture(origin, &b->graph);
     if (e == cudaSuccess) e = e2;

@@ -34,17 +34,36 @@ namespace amber {
 __global__ void __launch_bounds__(256) k_mass_reduce(const float* __restrict__ mass, int64_t n,
                                                      unsigned long long* __restrict__ total,
                                                      unsigned int* __restrict__ status) {
-  u128 acc = 0;
+  MassSum sum;
   bool bad = false;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  // 16-byte loads only from a 16-byte aligned array, else element by element
+  // 16-byte loads, four in flight, only from a 16-byte aligned array, else
+  // element by element
   const int64_t nvec = (reinterpret_cast<uintptr_t>(mass) & 15) == 0 ? n / 4 : 0;
-  for (int64_t v = gtid; v < nvec; v += stride) {
-    const float4 m = reinterpret_cast<const float4*>(mass)[v];
-    acc += mass_q64(m.x, bad) + mass_q64(m.y, bad) + mass_q64(m.z, bad) + mass_q64(m.w, bad);
+  const float4* mass4 = reinterpret_cast<const float4*>(mass);
+  auto add4 = [&](float4 m) {
+    sum.add(m.x, bad);
+    sum.add(m.y, bad);
+    sum.add(m.z, bad);
+    sum.add(m.w, bad);
+  };
+  int64_t v = gtid;
+  for (; v + 3 * stride < nvec; v += 4 * stride) {
+    const float4 a = mass4[v], b = mass4[v + stride], c = mass4[v + 2 * stride], d = mass4[v + 3 * stride];
+    add4(a);
+    add4(b);
+    add4(c);
+    add4(d);
+    sum.flush();
   }
-  for (int64_t i = nvec * 4 + gtid; i < n; i += stride) acc += mass_q64(mass[i], bad);
+  for (; v < nvec; v += stride) add4(mass4[v]);
+  sum.flush();
+  for (int64_t i = nvec * 4 + gtid; i < n; i += stride) {
+    sum.add(mass[i], bad);
+    sum.flush();
+  }
+  u128 acc = sum.slow;
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1) acc += shfl_down_u128(acc, o);
   __shared__ u128 ws[8];

@@ -60,6 +60,22 @@ __device__ __forceinline__ double u128_to_double(u128 v) {
   return __ull2double_rn(hi) * 18446744073709551616.0 + __ull2double_rn(lo);
 }
 
+// Exact mass sums: masses in [2^-16, 2^8), nearly all of them, are whole
+// multiples of 2^-40, so they add up in 64 bits (below 2^48 each: 2^13 of them
+// stay below 2^61); the others take the 128-bit path.
+struct MassSum {
+  unsigned long long fast = 0;  // 2^-40 units
+  u128 slow = 0;                // 2^-64 units
+  __device__ __forceinline__ void add(float m, bool& bad) {
+    if (m >= 1.52587890625e-5f && m < 256.0f) fast += floor_u64(m * 1099511627776.0f);
+    else slow += mass_q64(m, bad);
+  }
+  __device__ __forceinline__ void flush() {  // at least once per 2^13 masses
+    slow += (u128)fast << 24;
+    fast = 0;
+  }
+};
+
 // total += v for a 128-bit total held as two 64-bit words (exact; order-free).
 __device__ __forceinline__ void atomic_add_u128(unsigned long long* total, u128 v) {
   const unsigned long long lo = (unsigned long long)v, hi = (unsigned long long)(v >> 64);

@@ -147,22 +147,6 @@ __device__ __forceinline__ uint32_t warps_before(const uint32_t* wsum, int nw, i
   return __reduce_add_sync(0xffffffffu, lane < nw && lane < warp ? wsum[lane] : 0u);
 }
 
-// Exact mass sums: masses in [2^-16, 2^8), nearly all of them, are whole
-// multiples of 2^-40, so they add up in 64 bits (fewer than 2^13 of them per
-// thread stay below 2^61); the others take the 128-bit path.
-struct MassSum {
-  unsigned long long fast = 0;  // 2^-40 units
-  u128 slow = 0;                // 2^-64 units
-  __device__ __forceinline__ void add(float m, bool& bad) {
-    if (m >= 1.52587890625e-5f && m < 256.0f) fast += floor_u64(m * 1099511627776.0f);
-    else slow += mass_q64(m, bad);
-  }
-  __device__ __forceinline__ void flush() {
-    slow += (u128)fast << 24;
-    fast = 0;
-  }
-};
-
 template <int NT, int IT, bool FIRST, bool MASS>
 __device__ __forceinline__ void msd_split_body(const MsdArgs& a, uint32_t blk, uint32_t nblk) {
   constexpr int TILE = NT * IT;

@@ -116,19 +116,23 @@ def test_solve_in_a_captured_graph(B):
         assert ctx.sync_status() == 0
 
 
-def test_batch_of_split_rankings(B, monkeypatch):
-    # 256^3 items share their launches (both weightings; one whose extremes
-    # overflow a bucket takes the fallback) beside a smaller grid
+@pytest.mark.parametrize("specs", [[(256, 0), (64, 1), (256, 1), (256, 0), (256, 1)],
+                                   [(128, k % 2) for k in range(5)] + [(256, 0), (32, 0)],
+                                   [(64, k % 2) for k in range(33)]])
+def test_batch_of_split_rankings(B, monkeypatch, specs):
+    # sizes with over 2^23 cells share the launches of their split rankings
+    # (both weightings; an item whose extremes overflow a bucket takes the
+    # fallback) beside sizes ranked by digit passes, or alone
     from paper_2109_10375_gb300 import synth
     monkeypatch.setenv("AMBER_AUTOTUNE", "0")
     items, ref = [], []
-    with B.Context(256 ** 3) as ctx:
-        for k, (n, w) in enumerate([(256, 0), (64, 1), (256, 1), (256, 0), (256, 1)]):
+    with B.Context(max(n for n, _ in specs) ** 3) as ctx:
+        for k, (n, w) in enumerate(specs):
             box = 100.0 * n / 128
             S, m = synth.realisation(n, box, k, device="cuda")
             if k == 3:
                 S = torch.randn(S.shape, generator=torch.Generator(device="cuda").manual_seed(5), device="cuda")
-            h = B.history(7.0 + 0.4 * k, 4.0, 3.0, weighting=w)
+            h = B.history(7.0 + 0.04 * k, 4.0, 3.0, weighting=w)
             ref.append(ctx.solve(S, m, box, 3.0 + k, h))
             items.append((S, m, box, 3.0 + k, h, torch.empty_like(S)))
         batch = B.Batch([ctx], items)
