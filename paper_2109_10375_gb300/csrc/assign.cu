@@ -194,6 +194,7 @@ __device__ __forceinline__ void thresholds_body(const ThreshArgs& A, int blk) {
       beta = g;
     }
   }
+  pdl_begin();  // the table's values need nothing of the kernels before
   if (A.tile_mass) {
     const u128 s = sum_tile_mass(A.tile_mass, A.ntiles, threadIdx.x, blockDim.x);
     if (threadIdx.x == 0) sT = s;
@@ -308,6 +309,7 @@ __device__ __forceinline__ void scan_assign_body(const ScanArgs& a) {
 
 template <bool GATHER, bool WANT_F, bool LIN, bool DIRECT>
 __global__ void __launch_bounds__(kScanThreads, AMBER_SCAN_MINB) k_scan_assign(const ScanArgs a) {
+  pdl_begin();
   scan_assign_body<GATHER, WANT_F, LIN, DIRECT>(a);
 }
 
@@ -388,7 +390,10 @@ __device__ __forceinline__ void scatter_back_body(const ScatterArgs& x, uint32_t
   }
 }
 
-__global__ void __launch_bounds__(256) k_scatter_back(const ScatterArgs x) { scatter_back_body(x, blockIdx.x); }
+__global__ void __launch_bounds__(256) k_scatter_back(const ScatterArgs x) {
+  pdl_begin();
+  scatter_back_body(x, blockIdx.x);
+}
 
 // Several scatters at once: CTA b works on item find_item(prefix, M, b).
 __global__ void __launch_bounds__(256) k_scatter_back_multi(const ScatterArgs* __restrict__ args,
@@ -463,7 +468,7 @@ void thresholds_launch(ThreshArgs ta, cudaStream_t s) {
                                                                                          ta.total);
     ta.tile_mass = nullptr;
   }
-  k_thresholds<<<(ta.M + kThreshPoints - 1) / kThreshPoints, kThreshThreads, 0, s>>>(ta);
+  launch_pdl(k_thresholds, (ta.M + kThreshPoints - 1) / kThreshPoints, kThreshThreads, 0, s, ta);
 }
 
 void assign_args(const AssignWork& w, const uint32_t* order, const float* mass, const unsigned long long* tile_mass,
@@ -588,8 +593,8 @@ cudaError_t assign_impl(const AssignWork& w, const uint32_t* order, const float*
                       disjoint(zre, n, order_b, n) && disjoint(zre, n, mass_b, n) && disjoint(zre, n, F, n);
   if (direct) a.zre = zre;
   auto launch = [&](auto gt, auto ft, auto lt, auto dt) {
-    k_scan_assign<decltype(gt)::value, decltype(ft)::value, decltype(lt)::value, decltype(dt)::value>
-        <<<g, kScanThreads, 0, s>>>(a);
+    launch_pdl(k_scan_assign<decltype(gt)::value, decltype(ft)::value, decltype(lt)::value, decltype(dt)::value>, g,
+               kScanThreads, 0, s, a);
   };
   auto pick4 = [&](auto gt, auto ft, auto lt) {
     if (direct) launch(gt, ft, lt, std::true_type{});
@@ -608,7 +613,7 @@ cudaError_t assign_impl(const AssignWork& w, const uint32_t* order, const float*
   prof_end(prof, PK_SCAN_ASSIGN, s);
   if (direct) return cudaGetLastError();
   prof_begin(prof, PK_SCATTER_BACK, s);
-  k_scatter_back<<<(unsigned)(xa.groups * xa.nbuckets), 256, 0, s>>>(xa);
+  launch_pdl(k_scatter_back, (unsigned)(xa.groups * xa.nbuckets), 256, 0, s, xa);
   prof_end(prof, PK_SCATTER_BACK, s);
   return cudaGetLastError();
 }

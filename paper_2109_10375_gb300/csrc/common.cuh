@@ -117,6 +117,36 @@ __device__ __forceinline__ void dft(cpx<T>* v) {
 __device__ __forceinline__ bool not_finite(float x) { return (__float_as_uint(x) & 0x7f800000u) == 0x7f800000u; }
 __device__ __forceinline__ bool not_finite(double x) { return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000; }
 
+// Programmatic dependent launch: a kernel of few CTAs launched with launch_pdl
+// may be set up while the kernel before it in the stream still runs; it begins
+// with pdl_begin, which waits until all earlier work is done and visible and
+// lets the next one be set up in turn.  Saves most of the 2-3 us between the
+// dozen launches of a small solve (32^3 91 -> 72 us, 128^3 growth 196 -> 167).
+// Grids above kPdlMaxCtas are launched ordinarily and skip the wait: with it in
+// every CTA a 512^3 2LPT displacement took 10.2 instead of 8.0 ms.
+constexpr unsigned kPdlMaxCtas = 1024;
+__device__ __forceinline__ void pdl_begin() {
+  if (gridDim.x * gridDim.y <= kPdlMaxCtas) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+  }
+}
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                              const A&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = grid.x * grid.y <= kPdlMaxCtas ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // True the first time it is called with a given device current (per flag):
 // kernel attributes such as the dynamic shared-memory limit are set per device.
 inline bool first_use_on_device(std::atomic<unsigned long long>& mask) {

@@ -113,6 +113,7 @@ __device__ __forceinline__ void tile_kernel(T* Kt, int kx0, int ky, int tid, T k
 constexpr int kernel_table_size(int n) { return 3 * (n / 2) * (n / 2) + 1; }
 template <typename T>
 __global__ void __launch_bounds__(64) k_kernel_table(T* __restrict__ table, int count, T kf, T l_mfp, T norm) {
+  pdl_begin();
   const int i = blockIdx.x * 64 + threadIdx.x;
   if (i < count) table[i] = kernel_K<T>((T)i, l_mfp, kf, norm);
 }
@@ -157,6 +158,7 @@ k_fft_strided(cpx<T>* __restrict__ H, int64_t elem_stride, int64_t outer_stride,
   constexpr int QA = E / R0, QB = (R1 > 1) ? E / R1 : 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* sm = reinterpret_cast<cpx<T>*>(smem_raw);
+  pdl_begin();
 
   const int tid = threadIdx.x;
   int outer = blockIdx.x / ntx;
@@ -397,6 +399,7 @@ k_fft_zconv_tma(const __grid_constant__ CUtensorMap tmap, cpx<float>* __restrict
   // dynamic shared memory only (its base is 1024-byte aligned): the staged
   // tile / exchange area, the K table, the mbarrier
   extern __shared__ __align__(1024) unsigned char smem_tma[];
+  pdl_begin();
   cpx<T>* sm = reinterpret_cast<cpx<T>*>(smem_tma);
   T* Kt = reinterpret_cast<T*>(sm + L::elems);  // K over |kz| = 0..N/2 for the tile's columns
   const uint32_t buf = smem_u32(sm), mbar = buf + (uint32_t)zpass_tma_mbar_offset<N, V>();
@@ -536,6 +539,7 @@ k_fft_r2c_x(const T* __restrict__ src, cpx<T>* __restrict__ H, int64_t nrows, in
   constexpr int QA = E / R0, QB = (R1 > 1) ? E / R1 : 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* sm = reinterpret_cast<cpx<T>*>(smem_raw);
+  pdl_begin();
   const int tid = threadIdx.x;
   const int64_t row0 = (int64_t)blockIdx.x * 2 * XP;
   // first element of row ra of the launch
@@ -645,6 +649,7 @@ k_fft_c2r_x(const cpx<T>* __restrict__ H, T* __restrict__ J, int64_t nrows, int 
   constexpr int QA = E / R0, QB = (R1 > 1) ? E / R1 : 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<T>* sm = reinterpret_cast<cpx<T>*>(smem_raw);
+  pdl_begin();
   const int tid = threadIdx.x;
   const int64_t row0 = (int64_t)blockIdx.x * 2 * XP;
   if (tid == 0) {
@@ -808,6 +813,26 @@ k_fft_c2r_x(const cpx<T>* __restrict__ H, T* __restrict__ J, int64_t nrows, int 
   }
 }
 
+// Launches (see launch_pdl).
+template <typename T, int N, int MODE, int V = 0, bool OOP = false, bool MULTI = false, class OP = NoOp>
+void run_strided(int grid, size_t smem, cudaStream_t s, cpx<T>* H, int64_t elem_stride, int64_t outer_stride, int ncol,
+                 int ntx, const cpx<T>* tw, T kf, T l_mfp, T norm, const cpx<T>* Hin = nullptr,
+                 int64_t item_stride = 0, const T* kp = nullptr, const OP& op = OP()) {
+  launch_pdl(k_fft_strided<T, N, MODE, V, OOP, MULTI, OP>, grid, strided_threads<N, V>(), smem, s, H, elem_stride,
+             outer_stride, ncol, ntx, tw, kf, l_mfp, norm, Hin, item_stride, kp, op);
+}
+template <typename T, int N, int V = 0, bool MULTI = false>
+void run_r2c(int grid, size_t smem, cudaStream_t s, const T* src, cpx<T>* H, int64_t nrows, int RS, const cpx<T>* tw,
+             const T* const* srcs = nullptr, int64_t rpi = 0) {
+  launch_pdl(k_fft_r2c_x<T, N, V, MULTI>, grid, xpass_threads<N, V>(), smem, s, src, H, nrows, RS, tw, srcs, rpi);
+}
+template <typename T, int N, int V = 0, bool MULTI = false, bool HIST = false, class EPI = EpiKeys>
+void run_c2r(int grid, size_t smem, cudaStream_t s, const cpx<T>* H, T* J, int64_t nrows, int RS, const cpx<T>* tw,
+             unsigned int* status, SortCtrl* krange, int64_t rpi = 0, const EPI& epi = EPI()) {
+  launch_pdl(k_fft_c2r_x<T, N, V, MULTI, HIST, EPI>, grid, xpass_threads<N, V>(), smem, s, H, J, nrows, RS, tw, status,
+             krange, rpi, epi);
+}
+
 // ---------------------------------------------------------------------------
 // Host launcher for one radiation field of size N.
 // ---------------------------------------------------------------------------
@@ -860,18 +885,18 @@ cudaError_t radiation_field_n(const T* src, T* J, cpx<T>* H, const cpx<T>* tw, d
 
   if (!spec_in) {
     prof_begin(prof, PK_R2C_X, s);
-    k_fft_r2c_x<T, N, V><<<xgrid, xpass_threads<N, V>(), xs, s>>>(src, H, nrows, RS, tw);
+    run_r2c<T, N, V>(xgrid, xs, s, src, H, nrows, RS, tw);
     prof_end(prof, PK_R2C_X, s);
     // y-pass: lines (z, kx); element stride RS; outer (z) stride N*RS
     prof_begin(prof, PK_FFT_Y_FWD, s);
-    k_fft_strided<T, N, PASS_FWD, V><<<sgrid, strided_threads<N, V>(), ss, s>>>(H, RS, (int64_t)N * RS, ncol, ntx,
+    run_strided<T, N, PASS_FWD, V>(sgrid, ss, s, H, RS, (int64_t)N * RS, ncol, ntx,
                                                                              tw, kf, (T)l_mfp, norm);
     prof_end(prof, PK_FFT_Y_FWD, s);
   }
   // z-pass: lines (y, kx); element stride N*RS; outer (y) stride RS
   prof_begin(prof, PK_FFT_Z_CONV, s);
   if constexpr (sizeof(T) == 8)
-    k_kernel_table<T><<<(kernel_table_size(N) + 63) / 64, 64, 0, s>>>(ktable, kernel_table_size(N), kf, (T)l_mfp, norm);
+    launch_pdl(k_kernel_table<T>, (kernel_table_size(N) + 63) / 64, 64, 0, s, ktable, kernel_table_size(N), kf, (T)l_mfp, norm);
   bool z_done = false;
   if constexpr (sizeof(T) == 4 && C::R1 > 1) {
     CUtensorMap map;
@@ -884,31 +909,28 @@ cudaError_t radiation_field_n(const T* src, T* J, cpx<T>* H, const cpx<T>* tw, d
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
       const int grid = sgrid < 2 * sms ? sgrid : 2 * sms;
-      k_fft_zconv_tma<N, V><<<grid, strided_threads<N, V>(), zpass_tma_smem<N, V>(), s>>>(
-          map, H, ncol, ntx, sgrid, tw, kf, (T)l_mfp, norm, status);
+      launch_pdl(k_fft_zconv_tma<N, V>, grid, strided_threads<N, V>(), zpass_tma_smem<N, V>(), s, map, H, ncol, ntx, sgrid, tw, kf, (T)l_mfp, norm, status);
       z_done = true;
     }
   }
   if (z_done) {
   } else if (spec_in)
-    k_fft_strided<T, N, PASS_CONV, V, true><<<sgrid, strided_threads<N, V>(), sc, s>>>(
-        H, (int64_t)N * RS, RS, ncol, ntx, tw, kf, (T)l_mfp, norm, spec_in);
+    run_strided<T, N, PASS_CONV, V, true>(sgrid, sc, s, H, (int64_t)N * RS, RS, ncol, ntx, tw, kf, (T)l_mfp, norm, spec_in);
   else
-    k_fft_strided<T, N, PASS_CONV, V><<<sgrid, strided_threads<N, V>(), sc, s>>>(
-        H, (int64_t)N * RS, RS, ncol, ntx, tw, kf, (T)l_mfp, norm, nullptr, 0, ktable);
+    run_strided<T, N, PASS_CONV, V>(sgrid, sc, s, H, (int64_t)N * RS, RS, ncol, ntx, tw, kf, (T)l_mfp, norm, nullptr, 0, ktable);
   prof_end(prof, PK_FFT_Z_CONV, s);
   prof_begin(prof, PK_FFT_Y_INV, s);
-  k_fft_strided<T, N, PASS_INV, V><<<sgrid, strided_threads<N, V>(), ss, s>>>(H, RS, (int64_t)N * RS, ncol, ntx, tw,
+  run_strided<T, N, PASS_INV, V>(sgrid, ss, s, H, RS, (int64_t)N * RS, ncol, ntx, tw,
                                                                        kf, (T)l_mfp, norm);
   prof_end(prof, PK_FFT_Y_INV, s);
   prof_begin(prof, PK_C2R_X, s);
   if constexpr (sizeof(T) == 4) {
     if (hist8 && krange)
-      k_fft_c2r_x<T, N, V, false, true><<<xgrid, xpass_threads<N, V>(), xs, s>>>(H, J, nrows, RS, tw, status, krange);
+      run_c2r<T, N, V, false, true>(xgrid, xs, s, H, J, nrows, RS, tw, status, krange);
     else
-      k_fft_c2r_x<T, N, V><<<xgrid, xpass_threads<N, V>(), xs, s>>>(H, J, nrows, RS, tw, status, krange);
+      run_c2r<T, N, V>(xgrid, xs, s, H, J, nrows, RS, tw, status, krange);
   } else {
-    k_fft_c2r_x<T, N, V><<<xgrid, xpass_threads<N, V>(), xs, s>>>(H, J, nrows, RS, tw, status, krange);
+    run_c2r<T, N, V>(xgrid, xs, s, H, J, nrows, RS, tw, status, krange);
   }
   prof_end(prof, PK_C2R_X, s);
   return cudaGetLastError();
@@ -947,15 +969,14 @@ cudaError_t radiation_field_multi_n(const T* const* srcs, int M, T* J, cpx<T>* H
   const int ntx = (ncol + C::SB - 1) / C::SB;
   const int sgrid = M * N * ntx;
   const T zero = (T)0;
-  k_fft_r2c_x<T, N, V, true><<<xgrid, xpass_threads<N, V>(), xs, s>>>(nullptr, H, nrows, RS, tw, srcs, rpi);
+  run_r2c<T, N, V, true>(xgrid, xs, s, nullptr, H, nrows, RS, tw, srcs, rpi);
   // y passes: the z planes of all items are one run of M N planes
-  k_fft_strided<T, N, PASS_FWD, V><<<sgrid, strided_threads<N, V>(), ss, s>>>(H, RS, (int64_t)N * RS, ncol, ntx, tw,
+  run_strided<T, N, PASS_FWD, V>(sgrid, ss, s, H, RS, (int64_t)N * RS, ncol, ntx, tw,
                                                                            zero, zero, zero);
-  k_fft_strided<T, N, PASS_CONV, V, false, true><<<sgrid, strided_threads<N, V>(), sc, s>>>(
-      H, (int64_t)N * RS, RS, ncol, ntx, tw, zero, zero, norm, nullptr, item_stride, kp);
-  k_fft_strided<T, N, PASS_INV, V><<<sgrid, strided_threads<N, V>(), ss, s>>>(H, RS, (int64_t)N * RS, ncol, ntx, tw,
+  run_strided<T, N, PASS_CONV, V, false, true>(sgrid, sc, s, H, (int64_t)N * RS, RS, ncol, ntx, tw, zero, zero, norm, nullptr, item_stride, kp);
+  run_strided<T, N, PASS_INV, V>(sgrid, ss, s, H, RS, (int64_t)N * RS, ncol, ntx, tw,
                                                                            zero, zero, zero);
-  k_fft_c2r_x<T, N, V, true><<<xgrid, xpass_threads<N, V>(), xs, s>>>(H, J, nrows, RS, tw, status, kranges, rpi);
+  run_c2r<T, N, V, true>(xgrid, xs, s, H, J, nrows, RS, tw, status, kranges, rpi);
   return cudaGetLastError();
 }
 
@@ -979,10 +1000,10 @@ cudaError_t forward_spectrum_n(const T* src, cpx<T>* H, const cpx<T>* tw, cudaSt
   const int ntx = (ncol + C::SB - 1) / C::SB;
   const int sgrid = N * ntx;
   const T zero = (T)0;
-  k_fft_r2c_x<T, N><<<xgrid, xpass_threads<N>(), xs, s>>>(src, H, nrows, RS, tw);
-  k_fft_strided<T, N, PASS_FWD><<<sgrid, strided_threads<N>(), ss, s>>>(H, RS, (int64_t)N * RS, ncol, ntx, tw,
+  run_r2c<T, N>(xgrid, xs, s, src, H, nrows, RS, tw);
+  run_strided<T, N, PASS_FWD>(sgrid, ss, s, H, RS, (int64_t)N * RS, ncol, ntx, tw,
                                                                        zero, zero, zero);
-  k_fft_strided<T, N, PASS_FWD><<<sgrid, strided_threads<N>(), ss, s>>>(H, (int64_t)N * RS, RS, ncol, ntx, tw,
+  run_strided<T, N, PASS_FWD>(sgrid, ss, s, H, (int64_t)N * RS, RS, ncol, ntx, tw,
                                                                        zero, zero, zero);
   return cudaGetLastError();
 }
@@ -1009,10 +1030,10 @@ cudaError_t source_spectrum_n(const T* src, cpx<T>* H, const cpx<T>* tw, cudaStr
   const int sgrid = N * ntx;
   const T zero = (T)0;
   prof_begin(prof, PK_R2C_X, s);
-  k_fft_r2c_x<T, N, V><<<xgrid, xpass_threads<N, V>(), xs, s>>>(src, H, nrows, RS, tw);
+  run_r2c<T, N, V>(xgrid, xs, s, src, H, nrows, RS, tw);
   prof_end(prof, PK_R2C_X, s);
   prof_begin(prof, PK_FFT_Y_FWD, s);
-  k_fft_strided<T, N, PASS_FWD, V><<<sgrid, strided_threads<N, V>(), ss, s>>>(H, RS, (int64_t)N * RS, ncol, ntx, tw,
+  run_strided<T, N, PASS_FWD, V>(sgrid, ss, s, H, RS, (int64_t)N * RS, ncol, ntx, tw,
                                                                            zero, zero, zero);
   prof_end(prof, PK_FFT_Y_FWD, s);
   return cudaGetLastError();

@@ -25,9 +25,8 @@ cudaError_t zy_passes(const OP& op, size_t table, cpx<float>* tmp, const cpx<flo
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(G::ss + table));
     cudaFuncSetAttribute(k_fft_strided<float, N, PASS_INV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::ss);
   }
-  k_fft_strided<float, N, MODE, 0, false, false, OP><<<G::sgrid, strided_threads<N>(), G::ss + table, s>>>(
-      tmp, (int64_t)N * G::RS, G::RS, G::ncol, G::ntx, tw, 0.f, 0.f, norm, nullptr, 0, nullptr, op);
-  k_fft_strided<float, N, PASS_INV><<<G::sgrid, strided_threads<N>(), G::ss, s>>>(tmp, G::RS, (int64_t)N * G::RS,
+  run_strided<float, N, MODE, 0, false, false, OP>(G::sgrid, G::ss + table, s, tmp, (int64_t)N * G::RS, G::RS, G::ncol, G::ntx, tw, 0.f, 0.f, norm, nullptr, 0, nullptr, op);
+  run_strided<float, N, PASS_INV>(G::sgrid, G::ss, s, tmp, G::RS, (int64_t)N * G::RS,
                                                                                 G::ncol, G::ntx, tw, 0.f, 0.f, 0.f);
   return cudaGetLastError();
 }
@@ -40,8 +39,7 @@ cudaError_t x_pass(const EPI& epi, const cpx<float>* tmp, float* out, const cpx<
   if (first_use_on_device(attr))
     cudaFuncSetAttribute(k_fft_c2r_x<float, N, 0, false, false, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)G::xs);
-  k_fft_c2r_x<float, N, 0, false, false, EPI><<<G::xgrid, xpass_threads<N>(), G::xs, s>>>(
-      tmp, out, G::nrows, G::RS, tw, status, nullptr, 0, epi);
+  run_c2r<float, N, 0, false, false, EPI>(G::xgrid, G::xs, s, tmp, out, G::nrows, G::RS, tw, status, nullptr, 0, epi);
   return cudaGetLastError();
 }
 

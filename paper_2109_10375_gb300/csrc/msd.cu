@@ -133,7 +133,10 @@ __device__ __forceinline__ void msd_map_body(const MsdArgs& a, uint32_t blk, uin
   }
 }
 
-__global__ void __launch_bounds__(1024) k_msd_map(const MsdArgs a) { msd_map_body(a, blockIdx.x, gridDim.x); }
+__global__ void __launch_bounds__(1024) k_msd_map(const MsdArgs a) {
+  pdl_begin();
+  msd_map_body(a, blockIdx.x, gridDim.x);
+}
 
 __global__ void __launch_bounds__(1024) k_msd_map_multi(const MsdArgs* __restrict__ args) {
   __shared__ MsdArgs a;
@@ -176,6 +179,7 @@ __device__ __forceinline__ void msd_split_body(const MsdArgs& a, uint32_t blk, u
   float* __restrict__ mo = FIRST ? a.mass1 : a.mass2;
   bool bad = false;
   MassSum msum;
+  uint32_t done = 0;
   for (uint32_t tile = blk; tile < tiles; tile += nblk) {
     uint32_t start, have, bucket = 0;
     if (FIRST) {
@@ -294,6 +298,7 @@ __device__ __forceinline__ void msd_split_body(const MsdArgs& a, uint32_t blk, u
     };
     if (full) place(std::true_type{});
     else place(std::false_type{});
+    if (FIRST && MASS && (++done & 511u) == 0) msum.flush();
   }
   if (FIRST && MASS) {
     msum.flush();
@@ -315,6 +320,7 @@ __device__ __forceinline__ void msd_split_body(const MsdArgs& a, uint32_t blk, u
 
 template <int NT, int IT, bool FIRST, bool MASS>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_msd_split(const MsdArgs a) {
+  pdl_begin();
   msd_split_body<NT, IT, FIRST, MASS>(a, blockIdx.x, gridDim.x);
 }
 
@@ -592,6 +598,7 @@ __device__ __forceinline__ void msd_local_body(const MsdArgs& a, const ScanArgs&
 
 template <bool MASS, bool SCAN, bool LIN>
 __global__ void __launch_bounds__(kMsdLocalThreads, 2) k_msd_local(const MsdArgs a, const ScanArgs sa) {
+  pdl_begin();
   msd_local_body<MASS, SCAN, LIN>(a, sa);
 }
 
@@ -649,7 +656,7 @@ static void launch_split_v(const MsdArgs& a, int grid, cudaStream_t s) {
   static std::atomic<unsigned long long> attr{0};  // per instantiation and device
   if (first_use_on_device(attr))
     cudaFuncSetAttribute(k_msd_split<NT, IT, FIRST, MASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_msd_split<NT, IT, FIRST, MASS><<<grid, NT, smem, s>>>(a);
+  launch_pdl(k_msd_split<NT, IT, FIRST, MASS>, grid, NT, smem, s, a);
 }
 template <bool FIRST, bool MASS>
 static void launch_split(const MsdArgs& a, int grid, cudaStream_t s) {
@@ -664,14 +671,14 @@ static void launch_local(const MsdArgs& a, const ScanArgs& sa, cudaStream_t s) {
   static std::atomic<unsigned long long> attr{0};
   if (first_use_on_device(attr))
     cudaFuncSetAttribute(k_msd_local<MASS, SCAN, LIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_msd_local<MASS, SCAN, LIN><<<a.nb1 * a.nb2, kMsdLocalThreads, smem, s>>>(a, sa);
+  launch_pdl(k_msd_local<MASS, SCAN, LIN>, a.nb1 * a.nb2, kMsdLocalThreads, smem, s, a, sa);
 }
 
 cudaError_t msd_run(const MsdArgs& a, const FallbackArgs& f, int num_sms, const ThreshArgs* ta, const ScanArgs* sa,
                     cudaStream_t s, FftProfile* prof) {
   const int sg = (int)std::max<int64_t>(1, std::min<int64_t>(num_sms * 2, (a.n + 8191) / 8192));
   prof_begin(prof, PK_SORT_HIST, s);
-  k_msd_map<<<sg, 1024, 0, s>>>(a);
+  launch_pdl(k_msd_map, sg, 1024, 0, s, a);
   prof_end(prof, PK_SORT_HIST, s);
   const int g1 = msd_split_ctas(a.n, MsdPlan{a.nb1, a.nb2, a.cap1}, num_sms);
   prof_begin(prof, PK_SORT_PASS, s);
@@ -684,12 +691,14 @@ cudaError_t msd_run(const MsdArgs& a, const FallbackArgs& f, int num_sms, const 
     else launch_split<false, false>(a, g1, s);
     prof_end(prof, PK_SORT_PASS, s);
   }
-  cudaError_t e = sort_fallback(f, a.mass != nullptr, num_sms, s);
-  if (e != cudaSuccess) return e;
   if (sa) {
     prof_begin(prof, PK_THRESHOLDS, s);
     thresholds_launch(*ta, s);
     prof_end(prof, PK_THRESHOLDS, s);
+  }
+  cudaError_t e = sort_fallback(f, a.mass != nullptr, num_sms, s);
+  if (e != cudaSuccess) return e;
+  if (sa) {
     prof_begin(prof, PK_SCAN_ASSIGN, s);
     if (sa->weighting != AMBER_WEIGHT_MASS) launch_local<true, true, true>(a, *sa, s);
     else launch_local<true, true, false>(a, *sa, s);
