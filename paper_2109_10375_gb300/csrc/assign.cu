@@ -331,30 +331,25 @@ __global__ void __launch_bounds__(kScanThreads, AMBER_SCAN_MINB)
 // stores, so the dependent load -> store chains overlap.  A
 // bucket's cells span a bounded region of z_re, so the permuted writes of
 // the CTAs working on it stay close together.
-// wpt (1, 2, 4 or 8) warps share one tile's run, each taking a contiguous
-// part: with few buckets (small grids) a run holds most of a tile's 8192
-// pairs, and one warp copying it alone would wait through dozens of rounds.
 __device__ __forceinline__ void scatter_back_body(const ScatterArgs& x, uint32_t blk) {
   const uint32_t* __restrict__ bcell = x.bcell;
   const float* __restrict__ bz = x.bz;
   const uint16_t* __restrict__ btab = x.btab;
   float* __restrict__ zre = x.zre;
-  const int nbuckets = x.nbuckets, groups = x.groups, wpt = x.wpt;
+  const int nbuckets = x.nbuckets, groups = x.groups;
   const int64_t tiles = x.tiles;
   constexpr int TPW = 1;  // tiles per warp
   const int b = blk / groups;
   const int64_t g = blk - (int64_t)b * groups;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned long long stream_pol = l2_evict_first(), keep_pol = l2_evict_last();
-  const int tiles_per_cta = kBackTilesPerCta / wpt, part = warp % wpt;
-  const int64_t t0 = g * tiles_per_cta + warp / wpt;
-  // lane 0 fetches the tile's run bounds and keeps this warp's part of it
+  const int64_t t0 = g * kBackTilesPerCta + warp;
+  // lane 0 fetches the tile's run bounds
   int s_l = 0, e_l = 0;
   if (lane < TPW && t0 + lane < tiles) {
     const uint16_t* row = btab + (t0 + lane) * (nbuckets + 1);
-    const int s = row[b], e = row[b + 1];
-    s_l = s + ((e - s) * part) / wpt;
-    e_l = s + ((e - s) * (part + 1)) / wpt;
+    s_l = row[b];
+    e_l = row[b + 1];
   }
   // rounds of 4 x 32 pairs per run: the loads of all the warp's runs, then the stores
   constexpr int G = 4;
@@ -455,11 +450,21 @@ cudaError_t tomo_merge(float* z, const float* ztmp, int64_t n, float z_low, bool
 }
 
 // ---------------------------------------------------------------------------
+// Buckets of consecutive cells: 33 to 64 of them, or (above 2^29 cells) up to
+// 128 of 2^23 cells, 32 MB of z_re, so that the bucket being written stays in
+// L2.  A tile's 8192 cells take their places by shared-memory adds on their
+// buckets' counters, so few buckets collide, and a smaller bucket's sectors
+// fill up sooner: with 2^23 cells per bucket at every size (16 buckets at
+// 512^3, equal buckets of a warp found by a match first) the scan took 0.95 ms
+// and the scatter 0.98 ms at 512^3, with 64 buckets 0.77 and 0.73.  128 buckets,
+// with runs of 64 pairs for the scatter, are 2 % slower there; 30 and 60 million
+// cells and 24 grids of 64^3 show the same optimum, and 1024^3 differs by 1.5 %
+// between 64 and 256 buckets.
 void bucket_plan(int64_t n, int* nbuckets, int* shift) {
-  // buckets of 2^23 consecutive cells: 32 MB of z_re each, so the active
-  // bucket stays in L2; at most 128 buckets for 2^30 cells
-  *shift = kBucketShift;
-  *nbuckets = (int)((n + ((int64_t)1 << kBucketShift) - 1) >> kBucketShift);
+  int bits = 0;
+  while (((int64_t)1 << bits) < n) ++bits;
+  *shift = std::min(std::max(bits - 6, 0), 23);
+  *nbuckets = (int)((n + ((int64_t)1 << *shift) - 1) >> *shift);
 }
 
 void thresholds_launch(ThreshArgs ta, cudaStream_t s) {
@@ -538,12 +543,7 @@ void assign_args(const AssignWork& w, const uint32_t* order, const float* mass, 
   x.btab = w.btab;
   x.nbuckets = a.nbuckets;
   x.tiles = tiles;
-  // warps per tile run: about 128 pairs each on average (a tile's 8192 pairs
-  // spread over the buckets)
-  x.wpt = 1;
-  while (x.wpt < 8 && kScanTile / a.nbuckets >= 256 * x.wpt) x.wpt *= 2;
-  const int tiles_per_cta = kBackTilesPerCta / x.wpt;
-  x.groups = (int)((tiles + tiles_per_cta - 1) / tiles_per_cta);
+  x.groups = (int)((tiles + kBackTilesPerCta - 1) / kBackTilesPerCta);
   x.zre = zre;
 }
 

@@ -23,12 +23,11 @@ constexpr int kScanThreads = AMBER_SCAN_THREADS;
 constexpr int kScanItems = AMBER_SCAN_ITEMS;
 constexpr int kScanTile = kScanThreads * kScanItems;
 constexpr int kMaxTable = 1 << 16;
-constexpr int kMaxBuckets = 128;  // 2^30 cells in buckets of 2^23
+constexpr int kMaxBuckets = 128;  // 2^30 cells in buckets of 2^23 (bucket_plan)
 
 // the scan writes z in place up to these sizes (masses in rank order; gathered)
 constexpr int64_t kDirectMaxCells = (int64_t)1 << 24, kDirectGatherMaxCells = (int64_t)1 << 22;
 constexpr int kBackTilesPerCta = 8;  // scan tiles one scatter-back CTA covers
-constexpr int kBucketShift = 23;  // 2^23 cells (32 MB of z_re) per bucket by default
 
 // ctrl: exact total mass (2 x u64) at 0, tile ticket (u32) at 16, scan
 // fixed-point shift (int) at 32, scan total (u64) at 40; zeroed per call
@@ -115,7 +114,6 @@ struct ScatterArgs {
   int nbuckets;
   int64_t tiles;   // scan tiles
   int groups;      // scatter CTAs per bucket
-  int wpt;         // warps sharing one tile's run (1, 2, 4, 8); a CTA covers 8 / wpt tiles
   float* zre;
 };
 

@@ -67,3 +67,24 @@ def test_assign_forms_agree(B, n, weighting):
         over = ctx.assign_zre_ranked(order, ranked, h, ranked)
         assert ctx.sync_status() == 0
     assert torch.equal(gathered, placed) and torch.equal(gathered, with_F) and torch.equal(gathered, over)
+
+
+@pytest.mark.parametrize("n", [1, 63, 64, 65, 8_191, 8_192, 65_537, (1 << 20) + 1, (1 << 25) + 5])
+@pytest.mark.parametrize("spread", [True, False])
+def test_assign_buckets(B, n, spread):
+    # through the buckets (the result overwrites the rank-order masses) at the
+    # edges of the bucket counts (up to 64, 33 just above a power of two), with
+    # neighbouring ranks in buckets far apart or all in one: against the
+    # gathered form, bit for bit, and every cell written
+    g = torch.Generator(device="cuda").manual_seed(n)
+    mass = torch.rand(n, generator=g, device="cuda") * 2.9 + 0.01
+    order = torch.randperm(n, generator=g, device="cuda") if spread else torch.arange(n, device="cuda")
+    order = order.to(torch.int32)
+    ranked = mass[order.long()].contiguous()
+    h = B.history(8.0, 4.0, 3.0)
+    with B.Context(n) as ctx:
+        gathered = ctx.assign_zre(order, mass, h)
+        over = ctx.assign_zre_ranked(order, ranked, h, ranked)
+        assert ctx.sync_status() == 0
+    assert torch.equal(gathered, over)
+    assert bool(torch.isfinite(over).all())
