@@ -298,7 +298,10 @@ def design_bytes(n: int, sort_passes: int) -> dict:
     """Algorithmic bytes per step of each kernel as this design moves them:
     the half spectrum at its true size, the mass riding through the sort as a
     second payload (+8 B/cell per pass), and the scan's (cell, z) pairs
-    written and read back by the scatter to cell order."""
+    written and read back by the scatter to cell order.  The ranking by
+    splitting moves what as many digit passes would: a split reads and writes
+    key, cell and mass (the first reads J and mass), the local sort writes
+    order and mass."""
     C = n ** 3
     H = 8 * n * n * (n // 2 + 1)  # half spectrum, complex64
     if sort_passes == 1:
@@ -308,7 +311,7 @@ def design_bytes(n: int, sort_passes: int) -> dict:
     return {
         "fft_r2c_x": 4 * C + H, "fft_y_fwd": 2 * H, "fft_z_conv": 2 * H, "fft_y_inv": 2 * H,
         "fft_c2r_x": H + 4 * C,
-        "sort_histogram": 4 * C,            # digit histograms (the key range comes with the inverse x pass)
+        "sort_histogram": 4 * C,            # key histogram (the key range comes with the inverse x pass)
         "sort_pass": sort,
         "mass_reduce": 4 * C, "thresholds": 0, "scan_assign": 16 * C, "scatter_back": 12 * C,
     }
@@ -316,7 +319,7 @@ def design_bytes(n: int, sort_passes: int) -> dict:
 
 # The translation unit that holds each kernel kind; its hash covers that unit
 # and every csrc/ header it includes, directly or not.
-_KERNEL_SOURCES = {"fft": "fft_f32.cu", "sort": "sort.cu", "scan_assign": "assign.cu", "scatter_back": "assign.cu",
+_KERNEL_SOURCES = {"fft": "fft_f32.cu", "sort": "msd.cu", "scan_assign": "assign.cu", "scatter_back": "assign.cu",
                    "thresholds": "assign.cu", "mass_reduce": "assign.cu"}
 
 
@@ -429,7 +432,9 @@ def run_amber(args):
     ms = e0.elapsed_time(e1) / args.steps
     prof = ctx.profile_read()
     ctx.profile(False)
-    passes = ctx.sort_passes()  # digit passes of the timed solves' ranking
+    # passes over the cells of the timed solves' ranking: two splits and the
+    # local sort, or the digit passes (whose count is the key range's)
+    passes = round(prof["sort_pass"][1] / args.steps) or ctx.sort_passes()
     tuning = ctx.get_tuning(n)  # the choices the timed solves ran with
     st = ctx.sync_status()
     if st != 0:
@@ -639,9 +644,10 @@ def run_amber(args):
             raise RuntimeError(f"device status after autotuning: {B.status_string(st)}")
     del S_d, m_d, z_h
 
-    # each timed bracket is one kernel launch, except the histogram's, which
-    # also holds the one-CTA digit-offset scan (k_sort_offsets) -- alone when
-    # the inverse x pass counted the digits
+    # each timed bracket is one kernel launch; beside them runs one more: the
+    # one-CTA digit-offset scan (k_sort_offsets, in the histogram's bracket;
+    # alone there when the inverse x pass counted the digits) or, ranking by
+    # splitting, the fallback launch, which ends at once if no bucket overflowed
     fused = bool(tuning.get("fuse_histogram")) and tuning["sort_digit_bits"] == 8
     launches_per_step = (sum(v[1] for v in prof.values()) + (0 if fused else prof["sort_histogram"][1])) / args.steps
     mb, db = model_bytes(n, passes), design_bytes(n, passes)

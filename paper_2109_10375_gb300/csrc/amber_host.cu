@@ -387,7 +387,7 @@ bool msd_match(amber_ctx* c, const float* J, bool J_inside, const float* mass, b
   // Matched in the local sort where redshifts are stored in place (assign.cu;
   // a result inside the workspace would lie among what the local sort reads).
   // With pairs and buckets to form as well it is slower than the scan on its
-  // 8192-rank tiles (512^3: local sort with matching 2.31 ms, apart 1.13 + 0.92).
+  // 8192-rank tiles (512^3: local sort with matching 2.31 ms, apart 1.13 + 0.92, now 1.16 + 0.72).
   if (n <= kDirectMaxCells && (z < c->ws || z >= c->ws + pl.total)) {
     ThreshArgs ta;
     ScanArgs sa;

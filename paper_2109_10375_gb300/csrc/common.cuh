@@ -121,7 +121,7 @@ __device__ __forceinline__ bool not_finite(double x) { return (__double2hiint(x)
 // may be set up while the kernel before it in the stream still runs; it begins
 // with pdl_begin, which waits until all earlier work is done and visible and
 // lets the next one be set up in turn.  Saves most of the 2-3 us between the
-// dozen launches of a small solve (32^3 91 -> 72 us, 128^3 growth 196 -> 167).
+// dozen launches of a small solve (32^3 91 -> 72 us, 128^3 growth 205 -> 182).
 // Grids above kPdlMaxCtas are launched ordinarily and skip the wait: with it in
 // every CTA a 512^3 2LPT displacement took 10.2 instead of 8.0 ms.
 constexpr unsigned kPdlMaxCtas = 1024;
