@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <mutex>
 #include <utility>
 
 #include "../../include/amber.h"
@@ -147,13 +148,37 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
-// True the first time it is called with a given device current (per flag):
-// kernel attributes such as the dynamic shared-memory limit are set per device.
-inline bool first_use_on_device(std::atomic<unsigned long long>& mask) {
+// What a kernel needs set once per device before its first launch (such as its
+// dynamic shared-memory limit).
+struct PerDeviceOnce {
+  std::atomic<unsigned long long> done{0};  // a bit per device
+  std::mutex mu;
+};
+struct DeviceSetUp {
+  cudaError_t e = cudaSuccess;  // the first error
+  void also(cudaError_t r) {
+    if (e == cudaSuccess) e = r;
+  }
+  template <class K> void smem(K* kernel, size_t bytes) {
+    also(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  }
+};
+// Runs set_up(DeviceSetUp&) unless it has succeeded on the current device
+// before.  A thread that finds another one at it waits: going ahead, it would
+// launch a kernel whose limit is not set yet, which the driver refuses.  After
+// a failure the next call tries again.
+template <class F> inline cudaError_t once_on_device(PerDeviceOnce& once, F&& set_up) {
   int dev = 0;
-  cudaGetDevice(&dev);
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
   const unsigned long long bit = 1ull << (dev & 63);
-  return (mask.fetch_or(bit) & bit) == 0;
+  if (once.done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  std::lock_guard<std::mutex> lk(once.mu);
+  if (once.done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+  DeviceSetUp u;
+  set_up(u);
+  if (u.e == cudaSuccess) once.done.fetch_or(bit, std::memory_order_release);
+  return u.e;
 }
 
 // L2 eviction-priority policies for loads and stores that should (evict_last)

@@ -867,18 +867,17 @@ cudaError_t radiation_field_n(const T* src, T* J, cpx<T>* H, const cpx<T>* tw, d
   const size_t ss = StridedSmem<T, N, V>::elems * sizeof(cpx<T>);
   // the z pass adds its table of K over |kz| = 0..N/2 for the tile's columns
   const size_t sc = ss + (size_t)(N / 2 + 1) * C::SB * sizeof(T);
-  static std::atomic<unsigned long long> attr_done{0};  // per instantiation and device
-  if (first_use_on_device(attr_done)) {
-    cudaFuncSetAttribute(k_fft_r2c_x<T, N, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xs);
-    cudaFuncSetAttribute(k_fft_c2r_x<T, N, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xs);
-    cudaFuncSetAttribute(k_fft_strided<T, N, PASS_FWD, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
-    cudaFuncSetAttribute(k_fft_strided<T, N, PASS_INV, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
-    cudaFuncSetAttribute(k_fft_strided<T, N, PASS_CONV, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc);
-    cudaFuncSetAttribute(k_fft_strided<T, N, PASS_CONV, V, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sc);
+  static PerDeviceOnce attr_done;  // per instantiation and device
+  once_on_device(attr_done, [&](DeviceSetUp& u) {
+    u.smem(k_fft_r2c_x<T, N, V>, xs);
+    u.smem(k_fft_c2r_x<T, N, V>, xs);
+    u.smem(k_fft_strided<T, N, PASS_FWD, V>, ss);
+    u.smem(k_fft_strided<T, N, PASS_INV, V>, ss);
+    u.smem(k_fft_strided<T, N, PASS_CONV, V>, sc);
+    u.smem(k_fft_strided<T, N, PASS_CONV, V, true>, sc);
     if constexpr (sizeof(T) == 4)
-      cudaFuncSetAttribute(k_fft_c2r_x<T, N, V, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xs);
-  }
+      u.smem(k_fft_c2r_x<T, N, V, false, true>, xs);
+  });
   const int xgrid = (int)((nrows / 2 + C::XP - 1) / C::XP);
   const int ntx = (ncol + C::SB - 1) / C::SB;
   const int sgrid = N * ntx;
@@ -901,10 +900,10 @@ cudaError_t radiation_field_n(const T* src, T* J, cpx<T>* H, const cpx<T>* tw, d
   if constexpr (sizeof(T) == 4 && C::R1 > 1) {
     CUtensorMap map;
     if (tma && zpass_tensor_map(&map, spec_in ? (const void*)spec_in : (const void*)H, N, C::SB)) {
-      static std::atomic<unsigned long long> tma_attr{0};
-      if (first_use_on_device(tma_attr))
-        cudaFuncSetAttribute(k_fft_zconv_tma<N, V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)zpass_tma_smem<N, V>());
+      static PerDeviceOnce tma_attr;
+      once_on_device(tma_attr, [&](DeviceSetUp& u) {
+        u.smem(k_fft_zconv_tma<N, V>, zpass_tma_smem<N, V>());
+      });
       int dev = 0, sms = 0;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -956,15 +955,14 @@ cudaError_t radiation_field_multi_n(const T* const* srcs, int M, T* J, cpx<T>* H
   const size_t xs = XSmem<T, N, V>::elems * sizeof(cpx<T>);
   const size_t ss = StridedSmem<T, N, V>::elems * sizeof(cpx<T>);
   const size_t sc = ss + (size_t)(N / 2 + 1) * C::SB * sizeof(T);
-  static std::atomic<unsigned long long> attr_done{0};  // per instantiation and device
-  if (first_use_on_device(attr_done)) {
-    cudaFuncSetAttribute(k_fft_r2c_x<T, N, V, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xs);
-    cudaFuncSetAttribute(k_fft_c2r_x<T, N, V, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xs);
-    cudaFuncSetAttribute(k_fft_strided<T, N, PASS_FWD, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
-    cudaFuncSetAttribute(k_fft_strided<T, N, PASS_INV, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
-    cudaFuncSetAttribute(k_fft_strided<T, N, PASS_CONV, V, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sc);
-  }
+  static PerDeviceOnce attr_done;  // per instantiation and device
+  once_on_device(attr_done, [&](DeviceSetUp& u) {
+    u.smem(k_fft_r2c_x<T, N, V, true>, xs);
+    u.smem(k_fft_c2r_x<T, N, V, true>, xs);
+    u.smem(k_fft_strided<T, N, PASS_FWD, V>, ss);
+    u.smem(k_fft_strided<T, N, PASS_INV, V>, ss);
+    u.smem(k_fft_strided<T, N, PASS_CONV, V, false, true>, sc);
+  });
   const int xgrid = (int)((nrows / 2 + C::XP - 1) / C::XP);
   const int ntx = (ncol + C::SB - 1) / C::SB;
   const int sgrid = M * N * ntx;
@@ -991,11 +989,11 @@ cudaError_t forward_spectrum_n(const T* src, cpx<T>* H, const cpx<T>* tw, cudaSt
   const int64_t nrows = (int64_t)N * N;
   const size_t xs = XSmem<T, N>::elems * sizeof(cpx<T>);
   const size_t ss = StridedSmem<T, N>::elems * sizeof(cpx<T>);
-  static std::atomic<unsigned long long> attr_done{0};  // per instantiation and device
-  if (first_use_on_device(attr_done)) {
-    cudaFuncSetAttribute(k_fft_r2c_x<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xs);
-    cudaFuncSetAttribute(k_fft_strided<T, N, PASS_FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
-  }
+  static PerDeviceOnce attr_done;  // per instantiation and device
+  once_on_device(attr_done, [&](DeviceSetUp& u) {
+    u.smem(k_fft_r2c_x<T, N>, xs);
+    u.smem(k_fft_strided<T, N, PASS_FWD>, ss);
+  });
   const int xgrid = (int)((nrows / 2 + C::XP - 1) / C::XP);
   const int ntx = (ncol + C::SB - 1) / C::SB;
   const int sgrid = N * ntx;
@@ -1020,11 +1018,11 @@ cudaError_t source_spectrum_n(const T* src, cpx<T>* H, const cpx<T>* tw, cudaStr
   const int64_t nrows = (int64_t)N * N;
   const size_t xs = XSmem<T, N, V>::elems * sizeof(cpx<T>);
   const size_t ss = StridedSmem<T, N, V>::elems * sizeof(cpx<T>);
-  static std::atomic<unsigned long long> attr_done{0};  // per instantiation and device
-  if (first_use_on_device(attr_done)) {
-    cudaFuncSetAttribute(k_fft_r2c_x<T, N, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)xs);
-    cudaFuncSetAttribute(k_fft_strided<T, N, PASS_FWD, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ss);
-  }
+  static PerDeviceOnce attr_done;  // per instantiation and device
+  once_on_device(attr_done, [&](DeviceSetUp& u) {
+    u.smem(k_fft_r2c_x<T, N, V>, xs);
+    u.smem(k_fft_strided<T, N, PASS_FWD, V>, ss);
+  });
   const int xgrid = (int)((nrows / 2 + C::XP - 1) / C::XP);
   const int ntx = (ncol + C::SB - 1) / C::SB;
   const int sgrid = N * ntx;

@@ -19,12 +19,11 @@ template <int N> struct Geom {
 template <int N, int MODE, class OP>
 cudaError_t zy_passes(const OP& op, size_t table, cpx<float>* tmp, const cpx<float>* tw, float norm, cudaStream_t s) {
   using G = Geom<N>;
-  static std::atomic<unsigned long long> attr{0};  // per instantiation and device
-  if (first_use_on_device(attr)) {
-    cudaFuncSetAttribute(k_fft_strided<float, N, MODE, 0, false, false, OP>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(G::ss + table));
-    cudaFuncSetAttribute(k_fft_strided<float, N, PASS_INV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::ss);
-  }
+  static PerDeviceOnce attr;  // per instantiation and device
+  once_on_device(attr, [&](DeviceSetUp& u) {
+    u.smem(k_fft_strided<float, N, MODE, 0, false, false, OP>, G::ss + table);
+    u.smem(k_fft_strided<float, N, PASS_INV>, G::ss);
+  });
   run_strided<float, N, MODE, 0, false, false, OP>(G::sgrid, G::ss + table, s, tmp, (int64_t)N * G::RS, G::RS, G::ncol, G::ntx, tw, 0.f, 0.f, norm, nullptr, 0, nullptr, op);
   run_strided<float, N, PASS_INV>(G::sgrid, G::ss, s, tmp, G::RS, (int64_t)N * G::RS,
                                                                                 G::ncol, G::ntx, tw, 0.f, 0.f, 0.f);
@@ -35,10 +34,10 @@ template <int N, class EPI>
 cudaError_t x_pass(const EPI& epi, const cpx<float>* tmp, float* out, const cpx<float>* tw, unsigned int* status,
                    cudaStream_t s) {
   using G = Geom<N>;
-  static std::atomic<unsigned long long> attr{0};
-  if (first_use_on_device(attr))
-    cudaFuncSetAttribute(k_fft_c2r_x<float, N, 0, false, false, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)G::xs);
+  static PerDeviceOnce attr;
+  once_on_device(attr, [&](DeviceSetUp& u) {
+    u.smem(k_fft_c2r_x<float, N, 0, false, false, EPI>, G::xs);
+  });
   run_c2r<float, N, 0, false, false, EPI>(G::xgrid, G::xs, s, tmp, out, G::nrows, G::RS, tw, status, nullptr, 0, epi);
   return cudaGetLastError();
 }

@@ -317,9 +317,10 @@ static cudaError_t assign_p(int n, float inv_dx, const float* px, const float* p
   const int64_t n3 = (int64_t)n * n * n;
   if (n >= kAsgX) {
     constexpr size_t smem = 2 * kAsgBox * sizeof(int);
-    static std::atomic<unsigned long long> attr{0};  // per instantiation and device
-    if (first_use_on_device(attr))
-      cudaFuncSetAttribute(k_assign<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static PerDeviceOnce attr;  // per instantiation and device
+    once_on_device(attr, [&](DeviceSetUp& u) {
+      u.smem(k_assign<P>, smem);
+    });
     k_assign<P><<<(unsigned)(n3 / (kAsgX * kAsgY * kAsgZ)), kAsgThreads, smem, s>>>(px, py, pz, mass, n, inv_dx, mesh0, mesh1);
   } else {
     int lg = 0;

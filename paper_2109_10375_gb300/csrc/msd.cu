@@ -653,9 +653,10 @@ int msd_split_ctas(int64_t n, const MsdPlan& p, int num_sms) {
 template <int NT, int IT, bool FIRST, bool MASS>
 static void launch_split_v(const MsdArgs& a, int grid, cudaStream_t s) {
   constexpr size_t smem = (size_t)NT * IT * 16 + kMsdKnots * 8 + 2 * kMsdMaxDigits * 4;
-  static std::atomic<unsigned long long> attr{0};  // per instantiation and device
-  if (first_use_on_device(attr))
-    cudaFuncSetAttribute(k_msd_split<NT, IT, FIRST, MASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static PerDeviceOnce attr;  // per instantiation and device
+  once_on_device(attr, [&](DeviceSetUp& u) {
+    u.smem(k_msd_split<NT, IT, FIRST, MASS>, smem);
+  });
   launch_pdl(k_msd_split<NT, IT, FIRST, MASS>, grid, NT, smem, s, a);
 }
 template <bool FIRST, bool MASS>
@@ -668,9 +669,10 @@ static void launch_split(const MsdArgs& a, int grid, cudaStream_t s) {
 template <bool MASS, bool SCAN, bool LIN>
 static void launch_local(const MsdArgs& a, const ScanArgs& sa, cudaStream_t s) {
   constexpr size_t smem = (size_t)kMsdCap * 8 + (kMsdSub / 2 + 4) * 4;
-  static std::atomic<unsigned long long> attr{0};
-  if (first_use_on_device(attr))
-    cudaFuncSetAttribute(k_msd_local<MASS, SCAN, LIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static PerDeviceOnce attr;
+  once_on_device(attr, [&](DeviceSetUp& u) {
+    u.smem(k_msd_local<MASS, SCAN, LIN>, smem);
+  });
   launch_pdl(k_msd_local<MASS, SCAN, LIN>, a.nb1 * a.nb2, kMsdLocalThreads, smem, s, a, sa);
 }
 
@@ -715,13 +717,13 @@ cudaError_t msd_run(const MsdArgs& a, const FallbackArgs& f, int num_sms, const 
 cudaError_t msd_multi(const MsdMulti& m, int num_sms, cudaStream_t s) {
   constexpr size_t ssmem = (size_t)kMsdTileA * 16 + kMsdKnots * 8 + 2 * kMsdMaxDigits * 4;
   constexpr size_t lsmem = (size_t)kMsdCap * 8 + (kMsdSub / 2 + 4) * 4;
-  static std::atomic<unsigned long long> attr{0};  // per device
-  if (first_use_on_device(attr)) {
-    cudaFuncSetAttribute(k_msd_split_multi<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem);
-    cudaFuncSetAttribute(k_msd_split_multi<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem);
-    cudaFuncSetAttribute(k_msd_local_multi<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsmem);
-    cudaFuncSetAttribute(k_msd_local_multi<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsmem);
-  }
+  static PerDeviceOnce attr;  // per device
+  once_on_device(attr, [&](DeviceSetUp& u) {
+    u.smem(k_msd_split_multi<true>, ssmem);
+    u.smem(k_msd_split_multi<false>, ssmem);
+    u.smem(k_msd_local_multi<true>, lsmem);
+    u.smem(k_msd_local_multi<false>, lsmem);
+  });
   const dim3 g((unsigned)m.split_ctas, (unsigned)m.M);
   k_msd_map_multi<<<dim3((unsigned)num_sms, (unsigned)m.M), 1024, 0, s>>>(m.args);
   k_msd_split_multi<true><<<g, 512, ssmem, s>>>(m.args);

@@ -623,10 +623,10 @@ size_t sort_lookback_words(int64_t n) { return (size_t)sort_tiles(n) * kMaxRadix
 template <typename SRC, int RB, bool FIRST, bool MASS, bool MATCH>
 static void launch_pass_v(const PassArgs& a, int64_t tiles, cudaStream_t s) {
   const size_t smem = pass_smem<SRC, RB>(MASS);
-  static std::atomic<unsigned long long> attr{0};  // per instantiation and device
-  if (first_use_on_device(attr))
-    cudaFuncSetAttribute(k_sort_pass<SRC, RB, FIRST, MASS, MATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
+  static PerDeviceOnce attr;  // per instantiation and device
+  once_on_device(attr, [&](DeviceSetUp& u) {
+    u.smem(k_sort_pass<SRC, RB, FIRST, MASS, MATCH>, smem);
+  });
   k_sort_pass<SRC, RB, FIRST, MASS, MATCH><<<(unsigned)tiles, kSortThreads, smem, s>>>(a);
 }
 
@@ -812,15 +812,16 @@ int rank_args(const SortWork& w, const SRC* J, int64_t n, uint32_t* order, const
 
 template <bool MASS> static cudaError_t launch_fallback(const FallbackArgs& f, int num_sms, cudaStream_t s) {
   const size_t smem = pass_smem<float, 8>(MASS);
-  static std::atomic<unsigned long long> attr{0};  // per instantiation and device
-  static std::atomic<int> per_sm{0};
-  if (first_use_on_device(attr)) {
-    cudaFuncSetAttribute(k_sort_fallback<MASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static PerDeviceOnce attr;  // per instantiation and device
+  static std::atomic<int> per_sm{0};  // the same on every device: they are all of one kind
+  const cudaError_t e = once_on_device(attr, [&](DeviceSetUp& u) {
+    u.smem(k_sort_fallback<MASS>, smem);
     int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sort_fallback<MASS>, kSortThreads, smem) == cudaSuccess)
-      per_sm = b;
-  }
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    u.also(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sort_fallback<MASS>, kSortThreads, smem));
+    u.also(b > 0 ? cudaSuccess : cudaErrorInvalidConfiguration);
+    per_sm = b;
+  });
+  if (e != cudaSuccess) return e;
   const unsigned grid = (unsigned)std::min<int64_t>(f.tiles, (int64_t)num_sms * per_sm);
   void* args[] = {const_cast<FallbackArgs*>(&f)};
   return cudaLaunchCooperativeKernel(k_sort_fallback<MASS>, dim3(grid), dim3(kSortThreads), args, smem, s);
@@ -828,15 +829,16 @@ template <bool MASS> static cudaError_t launch_fallback(const FallbackArgs& f, i
 
 cudaError_t sort_fallback_multi(const FallbackArgs* f, int M, int64_t tiles, int num_sms, cudaStream_t s) {
   const size_t smem = pass_smem<float, 8>(true);
-  static std::atomic<unsigned long long> attr{0};  // per device
-  static std::atomic<int> per_sm{0};
-  if (first_use_on_device(attr)) {
-    cudaFuncSetAttribute(k_sort_fallback_multi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static PerDeviceOnce attr;  // per device
+  static std::atomic<int> per_sm{0};  // the same on every device: they are all of one kind
+  const cudaError_t e = once_on_device(attr, [&](DeviceSetUp& u) {
+    u.smem(k_sort_fallback_multi, smem);
     int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sort_fallback_multi, kSortThreads, smem) == cudaSuccess)
-      per_sm = b;
-  }
-  if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    u.also(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_sort_fallback_multi, kSortThreads, smem));
+    u.also(b > 0 ? cudaSuccess : cudaErrorInvalidConfiguration);
+    per_sm = b;
+  });
+  if (e != cudaSuccess) return e;
   const unsigned grid = (unsigned)std::min<int64_t>(tiles, (int64_t)num_sms * per_sm);
   void* args[] = {&f, &M};
   return cudaLaunchCooperativeKernel(k_sort_fallback_multi, dim3(grid), dim3(kSortThreads), args, smem, s);
@@ -849,10 +851,10 @@ cudaError_t sort_fallback(const FallbackArgs& f, bool with_mass, int num_sms, cu
 template <int RB, bool FIRST, bool MATCH>
 static void launch_pass_multi(const RankMulti& r, int p, cudaStream_t s) {
   const size_t smem = pass_smem<float, RB>(true);
-  static std::atomic<unsigned long long> attr{0};  // per instantiation and device
-  if (first_use_on_device(attr))
-    cudaFuncSetAttribute(k_sort_pass_multi<float, RB, FIRST, true, MATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
+  static PerDeviceOnce attr;  // per instantiation and device
+  once_on_device(attr, [&](DeviceSetUp& u) {
+    u.smem(k_sort_pass_multi<float, RB, FIRST, true, MATCH>, smem);
+  });
   k_sort_pass_multi<float, RB, FIRST, true, MATCH><<<r.tiles, kSortThreads, smem, s>>>(r.pass[p], r.tile_prefix, r.M);
 }
 

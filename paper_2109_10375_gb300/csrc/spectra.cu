@@ -226,9 +226,10 @@ cudaError_t epsilon_pdf_impl(const float* z, const float* zref, int64_t n, doubl
   if (e == cudaSuccess && moments) e = cudaMemsetAsync(moments, 0, 2 * sizeof(double), s);
   if (e != cudaSuccess) return e;
   const size_t smem = (size_t)(nbins + 2) * sizeof(unsigned int);
-  static std::atomic<unsigned long long> attr{0};
-  if (first_use_on_device(attr))
-    cudaFuncSetAttribute(k_eps_pdf, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+  static PerDeviceOnce attr;
+  once_on_device(attr, [&](DeviceSetUp& u) {
+    u.smem(k_eps_pdf, 64 * 1024);
+  });
   k_eps_pdf<<<grid_for(n, num_sms), 256, smem, s>>>(z, zref, n, (float)lo, (float)hi, (float)(nbins / (hi - lo)),
                                                     nbins, counts, moments);
   return cudaGetLastError();
@@ -241,11 +242,11 @@ cudaError_t power_impl(const void* Ha, const void* Hb, int n, double box, double
   cudaError_t e = cudaMemsetAsync(acc, 0, (size_t)kPowerAcc * nb * sizeof(double), s);
   if (e != cudaSuccess) return e;
   const size_t smem = (size_t)kPowerAcc * nb * sizeof(double);
-  static std::atomic<unsigned long long> attr{0};
-  if (first_use_on_device(attr)) {
-    cudaFuncSetAttribute(k_power_bins<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kPowerAcc * kMaxPowerBins * 8));
-    cudaFuncSetAttribute(k_power_bins<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kPowerAcc * kMaxPowerBins * 8));
-  }
+  static PerDeviceOnce attr;
+  once_on_device(attr, [&](DeviceSetUp& u) {
+    u.smem(k_power_bins<true>, kPowerAcc * kMaxPowerBins * 8);
+    u.smem(k_power_bins<false>, kPowerAcc * kMaxPowerBins * 8);
+  });
   const int64_t rows = (int64_t)n * n;
   const int g = (int)std::max<int64_t>(1, std::min<int64_t>((rows + 7) / 8, (int64_t)num_sms * 4));
   const auto* a = reinterpret_cast<const float2*>(Ha);
