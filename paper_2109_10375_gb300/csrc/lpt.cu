@@ -1,7 +1,7 @@
 // Source-field pipeline on the GPU (Sec. 3.2, Eq. xlpt; Sec. 3.2.1, Eqs.
 // interlace and Wofk; Sec. 3.3, Eq. fcoll).
 //
-//   k_assign<P>   : NGP / CIC / TSC assignment of one particle per lattice
+//   k_assign      : NGP / CIC / TSC assignment of one particle per lattice
 //                   point (FP32 sums, in any order)
 //   k_scale_mesh  : plain assignment's normalisation
 //
@@ -62,11 +62,12 @@ __device__ __forceinline__ void deposit_global(float* __restrict__ mesh, const f
   }
 }
 
-// Grids below one block: one particle per thread; lattice point (ix, iy, iz)
-// displaced by psi (box units, inv_dx cells per unit) plus `shift` cells on
-// every axis.
+// Grids below one block, and plain nearest-point meshes, whose one mesh point per
+// particle leaves nothing to gather (512^3 0.85 ms, by blocks 1.43): one particle
+// per thread; lattice point (ix, iy, iz) displaced by psi (box units, inv_dx
+// cells per unit) plus `shift` cells on every axis.
 template <int P>
-__global__ void __launch_bounds__(256) k_assign_small(const float* __restrict__ px, const float* __restrict__ py,
+__global__ void __launch_bounds__(256) k_assign_direct(const float* __restrict__ px, const float* __restrict__ py,
                                                       const float* __restrict__ pz, const float* __restrict__ mass,
                                                       int n, int lg, float inv_dx, float shift,
                                                       float* __restrict__ mesh) {
@@ -86,25 +87,44 @@ __global__ void __launch_bounds__(256) k_assign_small(const float* __restrict__ 
 // window point, 27 per particle for TSC, were bound by the packets they send to
 // L2 (two 512^3 TSC meshes 9.84 ms); float atomics in shared memory are a
 // compare-and-swap loop here (9.7 wavefronts per warp, 9.28 ms).  Integer ones
-// take 2, so the box holds two 32-bit fixed-point words per point: with S the
-// power of two that brings the block's mass total M below 2^30, a contribution
-// c adds round(c S) to the first and the rest, in units of 2^-20 / S, to the
-// second.  No sum can overflow (|c| adds up to at most M; 2048 rests of at most
-// 1/2), and the resolution, 2^-50 M, is below float's 2^-24 of any point above
-// 2^-26 M.  Particles of equal mass need one word where no mesh point is the
-// nearest of more than 8 of them (counted first): a point then sums to at most
-// 8 (CIC; 5.4 for TSC) times that count, so a resolution of 2^-25 or finer
-// fits, under float's own rounding of a mean density of 1.  A block whose box
-// does not fit, or whose total is 0, not finite or out of the scale's range, or
-// that has a position that is not finite, deposits straight to the mesh.  Both
-// meshes of an interlaced density (the second's particles half a cell on) come
-// from one read of psi.  Two 512^3 TSC meshes now take 4.00 ms (5.40 with two
-// words), bound by the shared-memory pipe (69 % busy; 83 % with two words).
+// take 2, so the box holds 32-bit fixed-point words, two per point or one.  With
+// two, S the scale of the first and 2^-k the unit of the second, a contribution
+// c adds round(c S) to the first and the rest, at most 1/2, to the second.
+//
+// An interlaced density (PLAIN false: both meshes, the second's particles half
+// a cell on, from one read of psi) goes through transforms that mix all mesh
+// points, so what counts is an error against the field's own scale.  S brings
+// the block's mass total M below 2^30 (no sum can overflow), k is 20 (2048 rests
+// of at most 1/2 fit): a resolution between 2^-49 and 2^-48 of M.  Particles of
+// equal mass take one word where no mesh point is the nearest of more than 8 of
+// them (counted first): a point's window weights then sum to less than 8 (CIC;
+// 5.4 for TSC) times that count, so that a resolution of 2^-25 or finer fits,
+// under float's rounding of a mean density of 1.  Two 512^3 TSC meshes take 4.00
+// ms (5.40 with two words), bound by the shared-memory pipe (69 % busy; 83 %).
+//
+// A plain mesh (PLAIN) is itself the result, and its points differ by many
+// orders: in a void a point may hold only the far tail of one window.  It always
+// takes two words, as fine as they go: with c the most particles that any mesh
+// point is the nearest of (2^lc >= c) and 2^e above every mass, S = 2^(27 - lc -
+// e), and k = 23 up to c = 16 (27 c rests fit), 20 above: a resolution of 2^-48
+// of a particle for c <= 4.  It has to lie 40 bits below the lightest mass, which
+// leaves the masses of a block 8 bits to differ by (c <= 4): collapsed fractions,
+// which span many orders, go straight to the mesh.  Against 64-bit sums the
+// errors are then those of float atomics or less at every density (256^3 CIC of
+// particles 2 cells off their places, FP32-exact positions: 3e-8 rms at density 1
+// against 4e-8, both exact below 0.1; with one word of 2^-25 2e-6 at 1e-2, 1e-4
+// at 1e-4).  512^3 TSC 2.61 -> 3.31 ms (float atomics 5.27).
+//
+// A block whose box does not fit, or whose masses are all 0, not finite or out
+// of the scale's range, or that has a position that is not finite, deposits
+// straight to the mesh.
 constexpr int kAsgX = 32, kAsgY = 8, kAsgZ = 8, kAsgPer = 4;
 constexpr int kAsgThreads = kAsgX * kAsgY * kAsgZ / kAsgPer;
 constexpr int kAsgBox = 14000;  // mesh points a block's box may hold (two CTAs per SM)
 
-template <int P>
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }  // |e| <= 126
+
+template <int P, bool PLAIN>
 __global__ void __launch_bounds__(kAsgThreads, 2)
     k_assign(const float* __restrict__ px, const float* __restrict__ py, const float* __restrict__ pz,
              const float* __restrict__ mass, int n, float inv_dx, float* __restrict__ mesh0,
@@ -112,8 +132,9 @@ __global__ void __launch_bounds__(kAsgThreads, 2)
   constexpr int NW = kAsgThreads / 32;
   extern __shared__ __align__(16) int box_hi[];  // [kAsgBox], then the second words
   int* box_lo = box_hi + kAsgBox;
-  __shared__ int s_lo[3][NW], s_hi[3][NW];
+  __shared__ int s_lo[3][NW], s_hi[3][NW], s_most[NW];
   __shared__ float s_mass[NW];
+  __shared__ unsigned s_heavy[NW], s_light[NW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nx = n / kAsgX, ny = n / kAsgY;
   const int bx = blockIdx.x % nx, by = (blockIdx.x / nx) % ny, bz = blockIdx.x / (nx * ny);
@@ -128,6 +149,7 @@ __global__ void __launch_bounds__(kAsgThreads, 2)
     m[q] = mass ? mass[i] : 1.0f;
   }
   float msum = 0.f;
+  unsigned heavy = 0, light = 0xffffffffu;  // bits of the largest and the smallest |m| > 0
 #pragma unroll
   for (int q = 0; q < kAsgPer; ++q) {
     pos[q][0] = ix + pos[q][0] * inv_dx;
@@ -135,14 +157,28 @@ __global__ void __launch_bounds__(kAsgThreads, 2)
     pos[q][2] = iz0 + q + pos[q][2] * inv_dx;
     // a position that is not finite makes the sum NaN (straight to the mesh)
     msum += fabsf(m[q]) + 0.f * (pos[q][0] + pos[q][1] + pos[q][2]);
+    if (PLAIN) {
+      const unsigned u = __float_as_uint(fabsf(m[q]));
+      heavy = max(heavy, u);
+      light = min(light, u - 1u);  // (0 becomes the largest)
+    }
   }
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1) msum += __shfl_xor_sync(0xffffffffu, msum, o);
-  if (lane == 0) s_mass[warp] = msum;
+  if (PLAIN) {
+    heavy = __reduce_max_sync(0xffffffffu, heavy);
+    light = __reduce_min_sync(0xffffffffu, light);
+  }
+  if (lane == 0) {
+    s_mass[warp] = msum;
+    if (PLAIN) {
+      s_heavy[warp] = heavy;
+      s_light[warp] = light;
+    }
+  }
   float scale = 0.f, unscale = 0.f;
-  for (int pass = 0; pass < 2; ++pass) {
+  for (int pass = 0; pass < (PLAIN ? 1 : 2); ++pass) {
     float* __restrict__ mesh = pass ? mesh1 : mesh0;
-    if (!mesh) break;
     const float shift = pass ? 0.5f : 0.f;
     // the box of mesh points the block's windows reach
     int ext[3], org[3];
@@ -164,15 +200,22 @@ __global__ void __launch_bounds__(kAsgThreads, 2)
       }
     }
     __syncthreads();
+    int mexp = 0;      // PLAIN: every |m| is below 2^mexp
+    float lightest = 0.f;
     if (pass == 0) {
       float t = s_mass[lane % NW];  // NW = 16: every sum twice
 #pragma unroll
       for (int o = NW / 2; o >= 1; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
       // t < 2^(e - 126) (one more bit for the rounding of this sum)
       const int e = (__float_as_int(t) >> 23) + 1;
-      if (t > 0.f && e > 40 && e < 250 && 30 - (e - 126) < 120) {
-        scale = __int_as_float((127 + 30 - (e - 126)) << 23);
-        unscale = __int_as_float((127 - 30 + (e - 126)) << 23);
+      if (PLAIN) {
+        mexp = (int)(__reduce_max_sync(0xffffffffu, s_heavy[lane % NW]) >> 23) - 126;
+        lightest = __uint_as_float(__reduce_min_sync(0xffffffffu, s_light[lane % NW]) + 1u);
+        // (a first guess, for one particle per point; replaced when they are counted)
+        if (t > 0.f && e < 250 && mexp > -80 && mexp < 100 && lightest >= pow2f(40 - 23 - 27 + mexp)) scale = 1.f;
+      } else if (t > 0.f && e > 40 && e < 250 && 30 - (e - 126) < 120) {
+        scale = pow2f(30 - (e - 126));
+        unscale = pow2f(e - 126 - 30);
       }
     }
     bool fits = scale != 0.f;
@@ -185,7 +228,48 @@ __global__ void __launch_bounds__(kAsgThreads, 2)
       ext[a] = fits ? hi - org[a] + P : 0;
     }
     const int plane = ext[0] * ext[1], cells = plane * ext[2];
-    if (!fits || cells > kAsgBox) {  // the same on every thread
+    fits = fits && cells <= kAsgBox;  // the same on every thread
+    float one = 0.f;  // the scale of a single word, or 0: two words
+    int k = 20;
+    if (fits) {
+      for (int c = tid * 4; c < cells; c += kAsgThreads * 4) {
+        *reinterpret_cast<int4*>(box_hi + c) = make_int4(0, 0, 0, 0);
+        *reinterpret_cast<int4*>(box_lo + c) = make_int4(0, 0, 0, 0);
+      }
+      __syncthreads();
+      if (PLAIN || !mass) {
+#pragma unroll
+        for (int q = 0; q < kAsgPer; ++q) {
+          int b[3];
+#pragma unroll
+          for (int a = 0; a < 3; ++a) b[a] = (int)floorf(pos[q][a] + shift + 0.5f) - org[a];
+          atomicAdd(box_lo + b[2] * plane + b[1] * ext[0] + b[0], 1);
+        }
+        __syncthreads();
+        int most = 0;
+        for (int c = tid * 4; c < cells; c += kAsgThreads * 4) {
+          int4* at = reinterpret_cast<int4*>(box_lo + c);
+          const int4 v = *at;
+          most = max(most, max(max(v.x, v.y), max(v.z, v.w)));
+          *at = make_int4(0, 0, 0, 0);
+        }
+        if (PLAIN) {
+          most = __reduce_max_sync(0xffffffffu, most);
+          if (lane == 0) s_most[warp] = most;
+          __syncthreads();
+          most = __reduce_max_sync(0xffffffffu, s_most[lane % NW]);
+          const int lc = 32 - __clz(most - 1);  // 2^lc >= most
+          if (lc <= 4) k = 23;
+          // unit of the second word: 2^(lc + mexp - 27 - k)
+          fits = lightest >= pow2f(40 + lc + mexp - 27 - k);
+          scale = pow2f(27 - lc - mexp);
+          unscale = pow2f(lc + mexp - 27);
+        } else if (!__syncthreads_or(most > (P == 2 ? 7 : 8))) {  // (8 x 8 x 2^25 would be 2^31)
+          one = __syncthreads_or(most > 4) ? 33554432.f : 67108864.f;  // 2^25, 2^26
+        }
+      }
+    }
+    if (!fits) {
 #pragma unroll 1
       for (int q = 0; q < kAsgPer; ++q) {
         const float at[3] = {pos[q][0] + shift, pos[q][1] + shift, pos[q][2] + shift};
@@ -194,30 +278,7 @@ __global__ void __launch_bounds__(kAsgThreads, 2)
       __syncthreads();  // s_lo, s_hi are read
       continue;
     }
-    for (int c = tid * 4; c < cells; c += kAsgThreads * 4) {
-      *reinterpret_cast<int4*>(box_hi + c) = make_int4(0, 0, 0, 0);
-      *reinterpret_cast<int4*>(box_lo + c) = make_int4(0, 0, 0, 0);
-    }
-    __syncthreads();
-    float one = 0.f;  // the scale of a single word, or 0: two words
-    if (!mass) {
-#pragma unroll
-      for (int q = 0; q < kAsgPer; ++q) {
-        int b[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) b[a] = (int)floorf(pos[q][a] + shift + 0.5f) - org[a];
-        atomicAdd(box_lo + b[2] * plane + b[1] * ext[0] + b[0], 1);
-      }
-      __syncthreads();
-      int most = 0;
-      for (int c = tid * 4; c < cells; c += kAsgThreads * 4) {
-        int4* at = reinterpret_cast<int4*>(box_lo + c);
-        const int4 v = *at;
-        most = max(most, max(max(v.x, v.y), max(v.z, v.w)));
-        *at = make_int4(0, 0, 0, 0);
-      }
-      if (!__syncthreads_or(most > 8)) one = __syncthreads_or(most > 4) ? 33554432.f : 67108864.f;  // 2^25, 2^26
-    }
+    const float rest = (float)(1 << k);
     auto deposit = [&](auto words) {
 #pragma unroll
       for (int q = 0; q < kAsgPer; ++q) {
@@ -239,21 +300,21 @@ __global__ void __launch_bounds__(kAsgThreads, 2)
               const int h = __float2int_rn(c);
               atomicAdd(row + ox, h);
               if (decltype(words)::value == 2)
-                atomicAdd(row + ox + kAsgBox, __float2int_rn((c - (float)h) * 1048576.f));
+                atomicAdd(row + ox + kAsgBox, __float2int_rn((c - (float)h) * rest));
             }
           }
         }
       }
     };
-    if (one != 0.f) deposit(std::integral_constant<int, 1>{});
+    if (!PLAIN && one != 0.f) deposit(std::integral_constant<int, 1>{});
     else deposit(std::integral_constant<int, 2>{});
     __syncthreads();
-    const float back = one != 0.f ? 1.f / one : unscale;
+    const float back = !PLAIN && one != 0.f ? 1.f / one : unscale, unit = 1.f / rest;
     const unsigned mask = (unsigned)n - 1u;
     const unsigned mx = 0xffffffffu / (unsigned)ext[0] + 1u, my = 0xffffffffu / (unsigned)ext[1] + 1u;
     for (int c = tid; c < cells; c += kAsgThreads) {
-      const int l = box_lo[c], h = box_hi[c] + (l >> 20);
-      const float v = ((float)h + (float)(l & 0xfffff) * 9.5367431640625e-7f) * back;
+      const int l = box_lo[c], h = box_hi[c] + (l >> k);
+      const float v = ((float)h + (float)(l & ((1 << k) - 1)) * unit) * back;
       if (v != 0.f) {
         // c = (z ext1 + y) ext0 + x; the reciprocals are exact for c < 2^16
         const unsigned yz = ext[0] == 1 ? (unsigned)c : __umulhi((unsigned)c, mx), x = c - yz * ext[0];
@@ -315,19 +376,22 @@ template <int P>
 static cudaError_t assign_p(int n, float inv_dx, const float* px, const float* py, const float* pz, const float* mass,
                             float* mesh0, float* mesh1, int num_sms, cudaStream_t s) {
   const int64_t n3 = (int64_t)n * n * n;
-  if (n >= kAsgX) {
+  if (n >= kAsgX && (P > 1 || mesh1)) {
     constexpr size_t smem = 2 * kAsgBox * sizeof(int);
     static PerDeviceOnce attr;  // per instantiation and device
     once_on_device(attr, [&](DeviceSetUp& u) {
-      u.smem(k_assign<P>, smem);
+      if constexpr (P > 1) u.smem(k_assign<P, true>, smem);
+      u.smem(k_assign<P, false>, smem);
     });
-    k_assign<P><<<(unsigned)(n3 / (kAsgX * kAsgY * kAsgZ)), kAsgThreads, smem, s>>>(px, py, pz, mass, n, inv_dx, mesh0, mesh1);
+    const unsigned grid = (unsigned)(n3 / (kAsgX * kAsgY * kAsgZ));
+    if (mesh1) k_assign<P, false><<<grid, kAsgThreads, smem, s>>>(px, py, pz, mass, n, inv_dx, mesh0, mesh1);
+    else if constexpr (P > 1) k_assign<P, true><<<grid, kAsgThreads, smem, s>>>(px, py, pz, mass, n, inv_dx, mesh0, nullptr);
   } else {
     int lg = 0;
     while ((1 << lg) < n) ++lg;
     for (int pass = 0; pass < 2; ++pass)
       if (pass ? mesh1 : mesh0)
-        k_assign_small<P><<<grid_of(n3, num_sms), 256, 0, s>>>(px, py, pz, mass, n, lg, inv_dx, pass ? 0.5f : 0.f,
+        k_assign_direct<P><<<grid_of(n3, num_sms), 256, 0, s>>>(px, py, pz, mass, n, lg, inv_dx, pass ? 0.5f : 0.f,
                                                                pass ? mesh1 : mesh0);
   }
   return cudaGetLastError();
