@@ -41,7 +41,8 @@ template <int P> __device__ __forceinline__ int window(float pos, float w[P]) {
 }
 
 // Straight to the mesh: one global atomic per mesh point the particle reaches
-// (n is a power of two, so a coordinate wraps by its low bits).
+// (n is a power of two, so a coordinate wraps by its low bits).  Points of weight
+// 0 are not reached: a mass that is not finite stays where its window is.
 template <int P>
 __device__ __forceinline__ void deposit_global(float* __restrict__ mesh, const float pos[3], float m, int n) {
   float w[3][P];
@@ -51,13 +52,16 @@ __device__ __forceinline__ void deposit_global(float* __restrict__ mesh, const f
   const unsigned mask = (unsigned)n - 1u;
 #pragma unroll
   for (int oz = 0; oz < P; ++oz) {
+    if (w[2][oz] == 0.f) continue;
     const int64_t zo = (int64_t)(((unsigned)b[2] + oz) & mask) * n;
 #pragma unroll
     for (int oy = 0; oy < P; ++oy) {
+      if (w[1][oy] == 0.f) continue;
       float* row = mesh + (zo + (((unsigned)b[1] + oy) & mask)) * n;
       const float wzy = m * w[2][oz] * w[1][oy];
 #pragma unroll
-      for (int ox = 0; ox < P; ++ox) atomicAdd(&row[((unsigned)b[0] + ox) & mask], wzy * w[0][ox]);
+      for (int ox = 0; ox < P; ++ox)
+        if (w[0][ox] != 0.f) atomicAdd(&row[((unsigned)b[0] + ox) & mask], wzy * w[0][ox]);
     }
   }
 }

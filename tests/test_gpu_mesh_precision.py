@@ -66,3 +66,24 @@ def test_plain_density_keeps_fp32_precision_at_every_point(B, n, masses, order):
     light = (ref > 1e-6) & (ref < 1e-2)
     assert light.sum() > 500
     assert np.all(np.abs(got - ref) <= tol), np.max((np.abs(got - ref) / np.maximum(tol, 1e-300))[tol > 0])
+
+
+@pytest.mark.parametrize("n", [8, 32])
+@pytest.mark.parametrize("order,shift", [(1, 0.0), (2, 0.0), (3, -0.5)])
+def test_an_infinite_mass_stays_where_its_window_is(B, n, order, shift):
+    # particles exactly on mesh points (CIC: one point of weight 1) or half way
+    # (TSC: two per axis, the third's weight is 0): the mesh is normalised by an
+    # infinite total, so a point with mass becomes NaN if the mass is infinite, else 0
+    psi = torch.full((n, n, n), shift, device="cuda")
+    mass = torch.ones(n, n, n, device="cuda")
+    mass[3, 2, 5] = float("inf")
+    with B.Context(n ** 3) as ctx:
+        got = ctx.mesh_density((psi, psi, psi), float(n), order, False, mass=mass)
+        ctx.sync_status()
+    bad = torch.zeros(n, n, n, dtype=torch.bool, device="cuda")
+    if order == 3:
+        bad[2:4, 1:3, 4:6] = True
+    else:
+        bad[3, 2, 5] = True
+    assert torch.equal(got.isnan(), bad)
+    assert torch.all(got[~bad] == 0)
