@@ -342,6 +342,8 @@ bool msd_setup(amber_ctx* c, const float* J, bool J_inside, const float* mass, b
   a.nb1 = p.nb1;
   a.nb2 = p.nb2;
   a.idx_shift = p.idx_shift;
+  a.fine = p.fine;
+  a.scale = (0xffffffffull << 32) / (unsigned long long)n;
   a.digit_bits = digit_bits;
   a.ctrl = c->sortw.ctrl;
   a.mc = reinterpret_cast<MsdCtrl*>(c->ws + pl.off_msd);
@@ -370,6 +372,7 @@ bool msd_setup(amber_ctx* c, const float* J, bool J_inside, const float* mass, b
   f.mass1 = a.mass1;
   f.nb1 = p.nb1;
   f.cap1 = p.cap1;
+  f.fine = p.fine;
   return true;
 }
 
@@ -1468,6 +1471,8 @@ static int batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, con
         m.nb1 = q.nb1;
         m.nb2 = q.nb2;
         m.idx_shift = q.idx_shift;
+        m.fine = q.fine;
+        m.scale = (0xffffffffull << 32) / (unsigned long long)m.n;
         m.digit_bits = c0->tune[ilog2i(items[i].params.n)].sort_digit_bits;
         m.ctrl = sw[i].ctrl;
         m.mc = reinterpret_cast<MsdCtrl*>(W + iw[i].mc);
@@ -1493,6 +1498,7 @@ static int batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, con
           mm.split_ctas = (int)ta.ntiles;
           mm.buckets = (int)(q.nb1 * q.nb2);
           mm.two_splits = q.nb2 > 1;
+          mm.fine = q.fine;
           mm.tiles = fb.tiles;
         }
         SplitGroup& sgp = split_groups.back();

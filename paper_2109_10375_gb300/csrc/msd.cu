@@ -2,12 +2,19 @@
 // sort.cu, from two splits and a sort in shared memory instead of four digit
 // passes over memory.
 //
-//   k_msd_map    : histogram of the intensities' keys over 2048 knots and from
+//   k_msd_map    : histogram of the intensities' keys over 2^14 counters and from
 //                  it a piecewise-linear map of (key, cell) to [0, 2^32) that
 //                  follows the distribution; it only balances the buckets, no
 //                  result depends on it.  Every cell is counted: samples of 1/4
 //                  to 1/16 misjudged the extremes, which lie together in a few
-//                  peaks and voids, and overflowed their buckets
+//                  peaks and voids, and overflowed their buckets.  The map's 2048
+//                  knots go where the cells are: one to each of 512 spans of the
+//                  key range, and 2^g, as many as there are, to those that hold
+//                  more than half a final bucket.  A few intensities at or below
+//                  zero, which mean free paths below 3 leave in any large field,
+//                  stretch the key range over all exponents; equal knots, a
+//                  quarter octave wide there, then misjudged the bulk and
+//                  overflowed (512^3, l = 2: a solve 10.05 ms, with the spans 5.73)
 //   k_msd_split  : cells to buckets of the map, by tiles: shared-memory atomics
 //                  give each cell a slot of its bucket's run in the tile and
 //                  global ones each run a place in the bucket's region (any
@@ -40,11 +47,14 @@ namespace amber {
 
 // Each kernel's work is that of CTA blk of nblk on one ranking: of the launch, or
 // (k_msd_*_multi) of the launch's row blockIdx.y, one ranking each.
+template <int FINE>
 __device__ __forceinline__ void msd_map_body(const MsdArgs& a, uint32_t blk, uint32_t nblk) {
-  __shared__ uint32_t h[kMsdKnots];
-  __shared__ uint32_t s_last, wsum[32];
-  const int tid = threadIdx.x, NT = blockDim.x;
-  for (int i = tid; i < kMsdKnots; i += NT) h[i] = 0;
+  constexpr int NC = kMsdSpans << FINE, NT = 1024;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint32_t* h = reinterpret_cast<uint32_t*>(smem_raw);  // [NC]
+  __shared__ uint32_t s_last, wsum[32], whvy[32];
+  const int tid = threadIdx.x;
+  for (int i = tid; i < NC; i += NT) h[i] = 0;
   const uint32_t gt = blk * NT + tid, ng = nblk * NT;
   for (uint32_t i = gt; i < a.nb1; i += ng) a.mc->cnt1[i] = 0;
   if (a.nb2 > 1)
@@ -60,12 +70,13 @@ __device__ __forceinline__ void msd_map_body(const MsdArgs& a, uint32_t blk, uin
     for (uint32_t i = gt; i < a.nb1 * a.nb2; i += ng) a.state[i] = 0;
     if (gt < kAssignCtrlBytes / 4) reinterpret_cast<uint32_t*>(a.actrl)[gt] = 0;
   }
-  const MsdRange R = msd_range(a.ctrl);
+  const MsdRange R = msd_range(a.ctrl, FINE);
+  const int shift = R.L - FINE;
   __syncthreads();
   const uint32_t n = (uint32_t)a.n;
   bool bad = false;
   auto count = [&](float x) {
-    atomicAdd(&h[min((enc_desc(x, bad) - R.kbase) >> R.L, (uint32_t)kMsdKnots - 1u)], 1u);
+    atomicAdd(&h[min((enc_desc(x, bad) - R.kbase) >> shift, (uint32_t)NC - 1u)], 1u);
   };
   // 16-byte loads from a 16-byte aligned array, else element by element
   const uint32_t nv = (reinterpret_cast<uintptr_t>(a.J) & 15) == 0 ? n / 4 : 0;
@@ -91,21 +102,34 @@ __device__ __forceinline__ void msd_map_body(const MsdArgs& a, uint32_t blk, uin
   }
   for (uint32_t i = nv * 4 + gt; i < n; i += ng) count(a.J[i]);
   __syncthreads();
-  for (int i = tid; i < kMsdKnots; i += NT)
-    if (h[i]) atomicAdd(&a.mc->hist[i], h[i]);
+  // two counters per atomic (none exceeds 32 bits), each CTA from a place of its
+  // own: all of them walking the same lines together took twice as long
+  unsigned long long* hist2 = reinterpret_cast<unsigned long long*>(a.mc->hist);
+  for (int i = tid; i < NC / 2; i += NT) {
+    const int at = (int)((i + blk * 96u) & (NC / 2 - 1u));
+    const unsigned long long v = reinterpret_cast<const unsigned long long*>(h)[at];
+    if (v) atomicAdd(hist2 + at, v);
+  }
   __threadfence();
   __syncthreads();
   if (tid == 0) s_last = atomicAdd(&a.mc->done, 1u) == nblk - 1;
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  constexpr int PER = kMsdKnots / 1024;
+  // two threads to a span, half of its counters each
+  constexpr int PER = NC / NT;
+  static_assert(PER % 4 == 0 && PER * 2 == 1 << FINE, "whole 16-byte words; two threads per span");
   uint32_t c[PER], sum = 0;
+  uint4* hist4 = reinterpret_cast<uint4*>(a.mc->hist) + tid * (PER / 4);
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    c[q] = __ldcg(&a.mc->hist[tid * PER + q]);
-    a.mc->hist[tid * PER + q] = 0;  // clean for the next ranking
-    sum += c[q];
+  for (int q = 0; q < PER / 4; ++q) {
+    const uint4 v4 = __ldcg(hist4 + q);
+    hist4[q] = make_uint4(0, 0, 0, 0);  // clean for the next ranking
+    c[4 * q] = v4.x;
+    c[4 * q + 1] = v4.y;
+    c[4 * q + 2] = v4.z;
+    c[4 * q + 3] = v4.w;
+    sum += v4.x + v4.y + v4.z + v4.w;
   }
   uint32_t x = sum;
   const int lane = tid & 31, warp = tid >> 5;
@@ -114,35 +138,53 @@ __device__ __forceinline__ void msd_map_body(const MsdArgs& a, uint32_t blk, uin
     const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
+  const bool heavy = sum + __shfl_xor_sync(0xffffffffu, sum, 1) > n / (2u * a.nb1 * a.nb2);
+  const uint32_t hm = __ballot_sync(0xffffffffu, heavy);
   if (lane == 31) wsum[warp] = x;
+  if (lane == 0) whvy[warp] = __popc(hm);
   __syncthreads();
-  uint32_t pre = 0, tot = 0;
+  uint32_t pre = 0, hpre = 0, H = 0;
   for (int w = 0; w < 32; ++w) {
     pre += w < warp ? wsum[w] : 0u;
-    tot += wsum[w];
+    hpre += w < warp ? whvy[w] : 0u;
+    H += whvy[w];
   }
+  hpre = (hpre + __popc(hm & ((1u << (lane & ~1)) - 1u))) / 2;  // heavy spans before this one
+  H /= 2;
+  int g = 0;  // the heavy spans take 2^g knots each
+  while (g < FINE && H * ((2u << g) - 1u) <= (uint32_t)(kMsdKnots - kMsdSpans)) ++g;
+  // where the heavy spans are that many, all get four: the splits then find a
+  // knot without the table (their lookups: 512^3 53 us of a split's 750)
+  static_assert(kMsdKnots == kMsdSpans * 4, "four knots per span");
+  const bool equal = g <= 3;
+  const int ls = equal ? 2 : heavy ? g : 0, span = tid / 2;
+  const uint32_t first = equal ? span * 4u : span + hpre * ((1u << g) - 1u);
+  const uint32_t total = equal ? (uint32_t)kMsdKnots : kMsdSpans + H * ((1u << g) - 1u);
   uint32_t run = pre + x - sum;
 #pragma unroll
   for (int q = 0; q < PER; ++q) {
-    a.mc->map[tid * PER + q] = (uint32_t)(((unsigned long long)run * 0xffffffffull) / tot);
+    const int at = (tid & 1) * PER + q;
+    if ((at & ((1 << (FINE - ls)) - 1)) == 0) a.mc->map[first + (at >> (FINE - ls))] = (uint32_t)((run * a.scale) >> 32);
     run += c[q];
   }
+  if ((tid & 1) == 0) a.mc->span[span] = ((int)first - (span << ls)) * 32 + (R.L - ls);
+  for (uint32_t i = total + tid; i <= (uint32_t)kMsdKnots; i += NT) a.mc->map[i] = 0xffffffffu;
   if (tid == 0) {
-    a.mc->map[kMsdKnots] = 0xffffffffu;
+    a.mc->equal = equal ? R.L - 2 : -1;
     a.mc->done = 0;
   }
 }
 
-__global__ void __launch_bounds__(1024) k_msd_map(const MsdArgs a) {
+template <int FINE> __global__ void __launch_bounds__(1024, 2) k_msd_map(const MsdArgs a) {
   pdl_begin();
-  msd_map_body(a, blockIdx.x, gridDim.x);
+  msd_map_body<FINE>(a, blockIdx.x, gridDim.x);
 }
 
-__global__ void __launch_bounds__(1024) k_msd_map_multi(const MsdArgs* __restrict__ args) {
+template <int FINE> __global__ void __launch_bounds__(1024, 2) k_msd_map_multi(const MsdArgs* __restrict__ args) {
   __shared__ MsdArgs a;
   if (threadIdx.x == 0) a = args[blockIdx.y];
   __syncthreads();
-  msd_map_body(a, blockIdx.x, gridDim.x);
+  msd_map_body<FINE>(a, blockIdx.x, gridDim.x);
 }
 
 // Sum of the first `warp` entries of per-warp totals (at most 32 of them).
@@ -156,7 +198,8 @@ __device__ __forceinline__ void msd_split_body(const MsdArgs& a, uint32_t blk, u
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint4* rec = reinterpret_cast<uint4*>(smem_raw);               // [TILE] (key, cell, mass, digit)
   uint2* map = reinterpret_cast<uint2*>(rec + TILE);             // [knots] (start, width)
-  uint32_t* cnt = reinterpret_cast<uint32_t*>(map + kMsdKnots);  // [digits] counts, then starts
+  int32_t* spans = reinterpret_cast<int32_t*>(map + kMsdKnots);  // [spans]
+  uint32_t* cnt = reinterpret_cast<uint32_t*>(spans + kMsdSpans);  // [digits] counts, then starts
   uint32_t* gb = cnt + kMsdMaxDigits;                            // [digits] global base - start
   __shared__ uint32_t wsum[NT / 32];
   __shared__ u128 wmass[NT / 32];
@@ -167,7 +210,9 @@ __device__ __forceinline__ void msd_split_body(const MsdArgs& a, uint32_t blk, u
     const uint32_t b0 = a.mc->map[i];
     map[i] = make_uint2(b0, a.mc->map[i + 1] - b0);
   }
-  const MsdRange R = msd_range(a.ctrl);
+  for (int i = tid; i < kMsdSpans; i += NT) spans[i] = a.mc->span[i];
+  const MsdRange R = msd_range(a.ctrl, a.fine);
+  const int equal = a.mc->equal;
   const uint32_t n = (uint32_t)a.n;
   const uint32_t per = FIRST ? 1u : (a.cap1 + TILE - 1) / TILE;  // tiles per first-split bucket
   const uint32_t tiles = FIRST ? (n + TILE - 1) / TILE : a.nb1 * per;
@@ -196,8 +241,8 @@ __device__ __forceinline__ void msd_split_body(const MsdArgs& a, uint32_t blk, u
     __syncthreads();  // also: the previous tile's staged cells are written
     uint32_t key[IT], idx[IT], ds[IT];
     float m[IT];
-    auto digits = [&](auto full_tag) {
-      constexpr bool FULL = decltype(full_tag)::value;
+    auto digits = [&](auto full_tag, auto equal_tag) {
+      constexpr bool FULL = decltype(full_tag)::value, EQUAL = decltype(equal_tag)::value;
       const uint32_t p0 = start + tid;
 #pragma unroll
       for (int it = 0; it < IT; ++it)
@@ -222,16 +267,24 @@ __device__ __forceinline__ void msd_split_body(const MsdArgs& a, uint32_t blk, u
             key[it] = enc_desc(__uint_as_float(key[it]), bad) - R.kbase;
             idx[it] = p0 + it * NT;
           }
-          const uint2 k = map[min(key[it] >> R.L, (uint32_t)kMsdKnots - 1u)];
-          const uint32_t phi = k.x + __umulhi(__funnelshift_r(idx[it] << ishift, key[it], R.L), k.y);
+          // (a NaN's key may lie outside the range: the last span and knot)
+          const int32_t sp = EQUAL ? equal : spans[min(key[it] >> R.L, (uint32_t)kMsdSpans - 1u)];
+          const uint32_t kn = EQUAL ? key[it] >> equal : (key[it] >> (sp & 31)) + (uint32_t)(sp >> 5);
+          const uint2 k = map[min(kn, (uint32_t)kMsdKnots - 1u)];
+          const uint32_t phi = k.x + __umulhi(__funnelshift_r(idx[it] << ishift, key[it], sp & 31), k.y);
           const uint32_t d = FIRST ? __umulhi(phi, nb1) : __umulhi(phi * nb1, nb2);
           ds[it] = d << 16 | atomicAdd(&cnt[d], 1u);
           if (MASS && FIRST) msum.add(m[it], bad);
         }
     };
     const bool full = have == (uint32_t)TILE;
-    if (full) digits(std::true_type{});
-    else digits(std::false_type{});
+    if (equal >= 0) {
+      if (full) digits(std::true_type{}, std::true_type{});
+      else digits(std::false_type{}, std::true_type{});
+    } else {
+      if (full) digits(std::true_type{}, std::false_type{});
+      else digits(std::false_type{}, std::false_type{});
+    }
     __syncthreads();
     // starts of the tile's runs, and their places in the buckets' regions
     {
@@ -635,6 +688,7 @@ MsdPlan msd_plan(int64_t n, bool with_mass, int num_sms) {
   int lg = 1;
   while (((int64_t)1 << lg) < n) ++lg;
   p.idx_shift = 32 - lg;
+  p.fine = msd_fine(n);
   const int64_t c1 = (int64_t)p.nb1 * p.cap1, c2 = p.nb2 > 1 ? (int64_t)p.nb1 * p.nb2 * kMsdCap : 0;
   p.kv1 = 2 * c1;
   p.m1 = with_mass ? c1 : 0;
@@ -652,7 +706,7 @@ int msd_split_ctas(int64_t n, const MsdPlan& p, int num_sms) {
 
 template <int NT, int IT, bool FIRST, bool MASS>
 static void launch_split_v(const MsdArgs& a, int grid, cudaStream_t s) {
-  constexpr size_t smem = (size_t)NT * IT * 16 + kMsdKnots * 8 + 2 * kMsdMaxDigits * 4;
+  constexpr size_t smem = (size_t)NT * IT * 16 + kMsdKnots * 8 + kMsdSpans * 4 + 2 * kMsdMaxDigits * 4;
   static PerDeviceOnce attr;  // per instantiation and device
   once_on_device(attr, [&](DeviceSetUp& u) {
     u.smem(k_msd_split<NT, IT, FIRST, MASS>, smem);
@@ -676,11 +730,22 @@ static void launch_local(const MsdArgs& a, const ScanArgs& sa, cudaStream_t s) {
   launch_pdl(k_msd_local<MASS, SCAN, LIN>, a.nb1 * a.nb2, kMsdLocalThreads, smem, s, a, sa);
 }
 
+template <int FINE> static void launch_map(const MsdArgs& a, int grid, cudaStream_t s) {
+  constexpr size_t smem = (size_t)(kMsdSpans << FINE) * 4;
+  static PerDeviceOnce attr;
+  once_on_device(attr, [&](DeviceSetUp& u) {
+    u.smem(k_msd_map<FINE>, smem);
+  });
+  launch_pdl(k_msd_map<FINE>, grid, 1024, smem, s, a);
+}
+
 cudaError_t msd_run(const MsdArgs& a, const FallbackArgs& f, int num_sms, const ThreshArgs* ta, const ScanArgs* sa,
                     cudaStream_t s, FftProfile* prof) {
   const int sg = (int)std::max<int64_t>(1, std::min<int64_t>(num_sms * 2, (a.n + 8191) / 8192));
   prof_begin(prof, PK_SORT_HIST, s);
-  launch_pdl(k_msd_map, sg, 1024, 0, s, a);
+  if (a.fine == 5) launch_map<5>(a, sg, s);
+  else if (a.fine == 4) launch_map<4>(a, sg, s);
+  else launch_map<3>(a, sg, s);
   prof_end(prof, PK_SORT_HIST, s);
   const int g1 = msd_split_ctas(a.n, MsdPlan{a.nb1, a.nb2, a.cap1}, num_sms);
   prof_begin(prof, PK_SORT_PASS, s);
@@ -715,17 +780,21 @@ cudaError_t msd_run(const MsdArgs& a, const FallbackArgs& f, int num_sms, const 
 }
 
 cudaError_t msd_multi(const MsdMulti& m, int num_sms, cudaStream_t s) {
-  constexpr size_t ssmem = (size_t)kMsdTileA * 16 + kMsdKnots * 8 + 2 * kMsdMaxDigits * 4;
+  constexpr size_t msmem = (size_t)(kMsdSpans << kMsdMaxFine) * 4;
+  constexpr size_t ssmem = (size_t)kMsdTileA * 16 + kMsdKnots * 8 + kMsdSpans * 4 + 2 * kMsdMaxDigits * 4;
   constexpr size_t lsmem = (size_t)kMsdCap * 8 + (kMsdSub / 2 + 4) * 4;
   static PerDeviceOnce attr;  // per device
   once_on_device(attr, [&](DeviceSetUp& u) {
+    u.smem(k_msd_map_multi<5>, msmem);
     u.smem(k_msd_split_multi<true>, ssmem);
     u.smem(k_msd_split_multi<false>, ssmem);
     u.smem(k_msd_local_multi<true>, lsmem);
     u.smem(k_msd_local_multi<false>, lsmem);
   });
   const dim3 g((unsigned)m.split_ctas, (unsigned)m.M);
-  k_msd_map_multi<<<dim3((unsigned)num_sms, (unsigned)m.M), 1024, 0, s>>>(m.args);
+  const dim3 gm((unsigned)num_sms, (unsigned)m.M);
+  if (m.fine == 5) k_msd_map_multi<5><<<gm, 1024, msmem, s>>>(m.args);
+  else k_msd_map_multi<4><<<gm, 1024, msmem / 2, s>>>(m.args);  // (sizes from 64^3 up)
   k_msd_split_multi<true><<<g, 512, ssmem, s>>>(m.args);
   if (m.two_splits) k_msd_split_multi<false><<<g, 512, ssmem, s>>>(m.args);
   return sort_fallback_multi(m.fallback, m.M, m.tiles, num_sms, s);

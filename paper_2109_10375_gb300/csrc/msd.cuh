@@ -9,8 +9,12 @@
 
 namespace amber {
 
-constexpr int kMsdKnotBits = 11;
-constexpr int kMsdKnots = 1 << kMsdKnotBits;  // knots of the distribution map
+constexpr int kMsdSpans = 512;                // equal spans of the key range ...
+constexpr int kMsdKnots = 2048;               // ... that share the knots of the distribution map
+constexpr int kMsdMaxFine = 5;                // a span has up to 2^5 counters, and at most as many knots
+// log2 counters per span: the map kernel's CTAs clear and add them all, 6 us of
+// a 64^3 solve's 96 with 2^5; fewer cells need fewer for the same balance
+inline int msd_fine(int64_t n) { return n < 1 << 18 ? 3 : n < 1 << 25 ? 4 : kMsdMaxFine; }
 constexpr int kMsdMaxDigits = 1024;           // buckets one split can write
 // Tiles of a split: 4096 cells (two CTAs per SM), or 10240 (one) where there are
 // so many buckets that a small tile's runs would be short: with 529 buckets
@@ -30,8 +34,10 @@ struct MsdCtrl {
   uint32_t done;      // CTAs of the map kernel that finished
   uint32_t bar;       // grid barrier of the fallback
   uint32_t pad[61];
-  uint32_t hist[kMsdKnots];
+  uint32_t hist[kMsdSpans << kMsdMaxFine];
   uint32_t map[kMsdKnots + 4];
+  int32_t span[kMsdSpans];  // knot of key k in a span: (k >> (span & 31)) + (span >> 5)
+  int32_t equal;            // >= 0: all knots are 2^equal keys wide
   uint32_t cnt1[kMsdMaxDigits];
 };
 
@@ -45,6 +51,8 @@ struct MsdArgs {
   float* mass2;
   uint32_t cap1, nb1, nb2;
   int idx_shift;         // cell index << idx_shift fills 32 bits
+  int fine;              // log2 counters per span
+  unsigned long long scale;  // (2^32 - 1) 2^32 / n
   int digit_bits;        // for the pass count reported
   SortCtrl* ctrl;
   MsdCtrl* mc;
@@ -62,7 +70,7 @@ struct MsdArgs {
 
 struct MsdPlan {
   uint32_t nb1, nb2, cap1;
-  int idx_shift;
+  int idx_shift, fine;
   int64_t kv1, m1, kv2, m2;  // words of the sets (kv: 2 per cell)
 };
 MsdPlan msd_plan(int64_t n, bool with_mass, int num_sms);
@@ -90,6 +98,7 @@ struct FallbackArgs {
   const uint2* kv1;
   const float* mass1;
   uint32_t nb1, cap1;
+  int fine;
   uint32_t* order_to;  // or null: the ranking (and masses) are copied here
   float* mass_to;
 };
@@ -109,7 +118,7 @@ struct MsdMulti {
   const MsdArgs* args;
   const ScanArgs* scans;
   const FallbackArgs* fallback;
-  int split_ctas, buckets;
+  int split_ctas, buckets, fine;
   bool two_splits;
   int64_t tiles;  // sort tiles of one ranking
 };
@@ -117,19 +126,19 @@ cudaError_t msd_multi(const MsdMulti& m, int num_sms, cudaStream_t s);  // up to
 void msd_multi_match(const MsdMulti& m, cudaStream_t s);                // local sorts with the matching
 cudaError_t sort_fallback_multi(const FallbackArgs* f, int M, int64_t tiles, int num_sms, cudaStream_t s);
 
-// Knots are 2^L keys wide and aligned to them, so that no knot straddles two
-// octaves of the intensity (a float's keys are half as dense per unit value in
-// the next octave, which would bend the distribution inside the knot); kbase is
-// the smallest key rounded down to a knot.
+// Spans are 2^L keys wide and aligned to them, and so are their counters and
+// knots, so that none straddles two octaves of the intensity (a float's keys are
+// half as dense per unit value in the next octave, which would bend the
+// distribution inside a knot); kbase is the smallest key rounded down to a span.
 struct MsdRange {
   uint32_t kbase;
-  int L;
+  int L;  // fine <= L <= 23
 };
-__device__ __forceinline__ MsdRange msd_range(const SortCtrl* ctrl) {
+__device__ __forceinline__ MsdRange msd_range(const SortCtrl* ctrl, int fine) {
   const uint32_t lo = (uint32_t)ctrl->kmin, hi = (uint32_t)ctrl->kmax;
   const int bits = 32 - __clz((int)(hi - lo));
-  int L = bits > kMsdKnotBits ? bits - kMsdKnotBits : 0;
-  if ((hi >> L) - (lo >> L) >= (uint32_t)kMsdKnots) ++L;
+  int L = fine + max(bits - 9 - fine, 0);
+  if ((hi - (lo >> L << L)) >> L >= (uint32_t)kMsdSpans) ++L;
   return {lo >> L << L, L};
 }
 

@@ -552,7 +552,7 @@ __device__ __forceinline__ void sort_fallback_body(const FallbackArgs& f) {
   uint32_t round = 0;
   unsigned* status = f.pass[0].status;
   if (!(fell & 1u) && (f.J_restore || f.mass_restore)) {
-    const uint32_t kbase = msd_range(f.hist.ctrl).kbase;
+    const uint32_t kbase = msd_range(f.hist.ctrl, f.fine).kbase;
     const int64_t slots = (int64_t)f.nb1 * f.cap1;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < slots; i += (int64_t)gridDim.x * blockDim.x) {
       const uint32_t d = (uint32_t)(i / f.cap1);

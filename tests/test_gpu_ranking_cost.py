@@ -1,0 +1,82 @@
+"""What a ranking costs does not hang on where the intensities lie (needs a GB300).
+
+Medians of ten calls, timed on the device; each limit lies well above the
+run-to-run spread (a few per cent) and well below what the fault it guards
+against cost.  Orders are checked against a stable sort.
+"""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    import __graft_entry__ as g
+    g.build()
+    from paper_2109_10375_gb300 import binding
+    return binding
+
+
+def _ms(f):
+    times = []
+    for k in range(13):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        f()
+        b.record()
+        torch.cuda.synchronize()
+        if k >= 3:
+            times.append(a.elapsed_time(b))
+    return float(np.median(times))
+
+
+def _rank_ms(B, ctx, J):
+    order = torch.empty(J.numel(), dtype=torch.int32, device="cuda")
+    ms = _ms(lambda: ctx.rank(J, out=order))
+    assert ctx.sync_status() == 0
+    assert torch.equal(order, torch.sort(-(J + 0.0), stable=True).indices.to(torch.int32))
+    return ms
+
+
+def _octaves(n):
+    g = torch.Generator(device="cuda").manual_seed(n % 1000)
+    return torch.randn(n, generator=g, device="cuda").mul_(0.8).exp_()
+
+
+@pytest.mark.parametrize("n", [300_007, 10_000_019])
+@pytest.mark.parametrize("kind", ["one zero", "some negative", "both signs", "far outliers"])
+def test_rank_with_intensities_at_and_below_zero(B, n, kind):
+    # they stretch the key range over all exponents, which must not unbalance
+    # the buckets of the others (it took twice as long)
+    J = _octaves(n)
+    with B.Context(n) as ctx:
+        base = _rank_ms(B, ctx, J)
+        if kind == "one zero":
+            J[n // 3] = 0.0
+        elif kind == "some negative":
+            J[::1000] *= -1.0
+        elif kind == "both signs":
+            J[::2] *= -1.0
+        else:
+            J[5], J[n - 5] = 1e-30, 1e30
+        assert _rank_ms(B, ctx, J) < 1.35 * base
+
+
+@pytest.mark.parametrize("n,l_mfp", [(128, 1.0), (256, 1.0), (256, 1.6), (512, 2.0), (512, 1.0)])
+def test_solve_with_short_mean_free_paths(B, n, l_mfp):
+    # below l = 3 the FP32 transforms leave some cells with J <= 0
+    from paper_2109_10375_gb300 import synth
+    S, m = synth.realisation(n, 0.78125 * n, 4, device="cuda")
+    h = B.history(8.0, 4.0, 3.0)
+    z, J = torch.empty_like(S), torch.empty_like(S)
+    with B.Context(n ** 3) as ctx:
+        base = _ms(lambda: ctx.solve(S, m, 0.78125 * n, 5.0, h, out=z))
+        t = _ms(lambda: ctx.solve(S, m, 0.78125 * n, l_mfp, h, out=z, J_out=J))
+        ctx.set_tuning(n, sort_digit_bits=8, fuse_histogram=1)  # digit passes
+        ref = ctx.solve(S, m, 0.78125 * n, l_mfp, h)
+        assert ctx.sync_status() == 0
+    assert float(J.min()) < 1e-3 * float(J.median())
+    assert torch.equal(z, ref)
+    assert t < 1.25 * base
