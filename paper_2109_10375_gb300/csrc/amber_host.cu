@@ -313,8 +313,10 @@ namespace {
 // lie at its start, the second's after them; J (J_inside) is massB and the
 // masses (mass_inside) idxB, which only the second split may overwrite.  Their
 // values then come back from the first split's regions if it overflows.
+// in_place: matched in the local sort, which reads the fallback's ranking where
+// its passes leave it; else that goes to order (and mass_out) too, if given.
 bool msd_setup(amber_ctx* c, const float* J, bool J_inside, const float* mass, bool mass_inside, int64_t n,
-               uint32_t* order, float* mass_out, int digit_bits, MsdArgs* out, FallbackArgs* fb) {
+               uint32_t* order, float* mass_out, bool in_place, int digit_bits, MsdArgs* out, FallbackArgs* fb) {
   const Plan& pl = c->plan;
   if (sort_rank_env() >= 0) return false;
   const MsdPlan p = msd_plan(n, mass != nullptr, c->num_sms);
@@ -360,9 +362,8 @@ bool msd_setup(amber_ctx* c, const float* J, bool J_inside, const float* mass, b
   f = FallbackArgs{};
   f.mc = a.mc;
   uint32_t blocks;
-  // with masses the fallback leaves its ranking in the workspace for the matching
-  rank_args<float>(c->sortw, J, n, mass ? nullptr : order, mass, nullptr, nullptr, c->status, kSpinLimit, 8, &f.hist,
-                   &blocks, f.pass);
+  rank_args<float>(c->sortw, J, n, in_place ? nullptr : order, mass, in_place ? nullptr : mass_out, nullptr, c->status,
+                   kSpinLimit, 8, &f.hist, &blocks, f.pass);
   f.tiles = sort_tiles(n);
   if (p.nb2 > 1) {
     f.J_restore = J_inside ? const_cast<float*>(J) : nullptr;
@@ -383,15 +384,17 @@ bool msd_match(amber_ctx* c, const float* J, bool J_inside, const float* mass, b
                cudaStream_t s, cudaError_t* err) {
   MsdArgs ma;
   FallbackArgs fa;
-  if (!msd_setup(c, J, J_inside, mass, mass_inside, n, order_out, mass_rank_out, digit_bits, &ma, &fa)) return false;
   const Plan& pl = c->plan;
-  const int nsums = msd_split_ctas(n, MsdPlan{ma.nb1, ma.nb2, ma.cap1}, c->num_sms);
   const unsigned char* z = reinterpret_cast<const unsigned char*>(zre);
   // Matched in the local sort where redshifts are stored in place (assign.cu;
   // a result inside the workspace would lie among what the local sort reads).
   // With pairs and buckets to form as well it is slower than the scan on its
   // 8192-rank tiles (512^3: local sort with matching 2.31 ms, apart 1.13 + 0.92, now 1.16 + 0.72).
-  if (n <= kDirectMaxCells && (z < c->ws || z >= c->ws + pl.total)) {
+  const bool in_place = n <= kDirectMaxCells && (z < c->ws || z >= c->ws + pl.total);
+  if (!msd_setup(c, J, J_inside, mass, mass_inside, n, order_out, mass_rank_out, in_place, digit_bits, &ma, &fa))
+    return false;
+  const int nsums = msd_split_ctas(n, MsdPlan{ma.nb1, ma.nb2, ma.cap1}, c->num_sms);
+  if (in_place) {
     ThreshArgs ta;
     ScanArgs sa;
     ScatterArgs xa;
@@ -406,7 +409,8 @@ bool msd_match(amber_ctx* c, const float* J, bool J_inside, const float* mass, b
     return true;
   }
   // the ranking over the first split's regions (two splits: dead by then) or
-  // idxB and massA; the pairs in arrays that are free then
+  // idxB and massA; the pairs in arrays that are free then, or over the
+  // fallback's ranking (a tile's pairs go where its own ranks were read)
   uint32_t* block = reinterpret_cast<uint32_t*>(c->ws + pl.off_spec);
   AssignWork w = c->assw;
   if (ma.nb2 > 1) {
@@ -417,12 +421,15 @@ bool msd_match(amber_ctx* c, const float* J, bool J_inside, const float* mass, b
     ma.order = ma.nb2 > 1 ? block : c->sortw.idxB;
     ma.mass_out = ma.nb2 > 1 ? reinterpret_cast<float*>(block + (n + 63) / 64 * 64) : c->sortw.massA;
   }
-  fa.order_to = ma.order;
-  fa.mass_to = ma.mass_out;
+  const FellArgs fell{&ma.mc->overflow, c->sortw.idxA, c->sortw.massA};
   *err = msd_run(ma, fa, c->num_sms, nullptr, nullptr, s, &c->prof);
-  if (*err == cudaSuccess)
+  if (*err != cudaSuccess) return true;
+  if (order_out)
     *err = assign_impl(w, ma.order, ma.mass_out, true, ma.cta_mass, n, hc, zre, nullptr, c->status, s, &c->prof,
                        kSpinLimit, nullptr, nullptr, nullptr, nsums);
+  else
+    *err = assign_impl(w, ma.order, ma.mass_out, true, ma.cta_mass, n, hc, zre, nullptr, c->status, s, &c->prof,
+                       kSpinLimit, c->sortw.idxB, c->sortw.massB, &c->sortw.ctrl->npasses, nsums, &fell);
   return true;
 }
 
@@ -796,7 +803,7 @@ int amber_rank(amber_ctx* c, const float* d_J, int64_t ncells, uint32_t* d_order
   c->last_stream = s;
   MsdArgs ma;
   FallbackArgs fa;
-  if (msd_setup(c, d_J, false, nullptr, false, ncells, d_order, nullptr, KeyOf<float>::RB, &ma, &fa)) {
+  if (msd_setup(c, d_J, false, nullptr, false, ncells, d_order, nullptr, false, KeyOf<float>::RB, &ma, &fa)) {
     cudaError_t e = sort_ctrl_reset(c->sortw.ctrl, s);
     if (e == cudaSuccess) e = key_range_impl(d_J, ncells, c->sortw.ctrl, c->num_sms, c->status, s);
     if (e == cudaSuccess) e = msd_run(ma, fa, c->num_sms, nullptr, nullptr, s, &c->prof);

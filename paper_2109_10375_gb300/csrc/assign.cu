@@ -268,9 +268,10 @@ __device__ __forceinline__ void scan_assign_body(const ScanArgs& a) {
   const uint32_t start = tile * (uint32_t)TILE;
   const uint32_t n = (uint32_t)a.n;
   const int cnt = (int)(n - start < (uint32_t)TILE ? n - start : (uint32_t)TILE);
-  const bool side_b = a.pick && ((*a.pick - 1) & 1);
-  const uint32_t* order = side_b ? a.order_b : a.order;
-  const float* mass = side_b ? a.mass_b : a.mass;
+  const bool fell = a.fell && *a.fell;
+  const bool side_b = a.pick && fell == (a.fell != nullptr) && ((*a.pick - 1) & 1);
+  const uint32_t* order = side_b ? a.order_b : fell ? a.order_a : a.order;
+  const float* mass = side_b ? a.mass_b : fell ? a.mass_a : a.mass;
   if (tid == 0 && a.ahead) {
     // order and masses of the tile a.ahead tickets later into L2
     const uint32_t fs = (tile + a.ahead) * (uint32_t)TILE;
@@ -511,6 +512,9 @@ void assign_args(const AssignWork& w, const uint32_t* order, const float* mass, 
   a.order_b = order_b;
   a.mass_b = mass_b;
   a.pick = pick;
+  a.fell = nullptr;
+  a.order_a = nullptr;
+  a.mass_a = nullptr;
   a.n = n;
   a.Xq = w.Xq;
   a.qshift = qshift;
@@ -555,13 +559,19 @@ template <typename A, typename B> static bool disjoint(const A* a, int64_t na, c
 cudaError_t assign_impl(const AssignWork& w, const uint32_t* order, const float* mass, bool mass_in_rank_order,
                         const unsigned long long* tile_mass, int64_t n, const HistoryCoeffs& hc, float* zre, double* F,
                         unsigned int* status, cudaStream_t s, FftProfile* prof, unsigned int spin_limit,
-                        const uint32_t* order_b, const float* mass_b, const int* pick, int64_t nsums) {
+                        const uint32_t* order_b, const float* mass_b, const int* pick, int64_t nsums,
+                        const FellArgs* fell) {
   const int64_t tiles = (n + kScanTile - 1) / kScanTile;
   ThreshArgs ta;
   ScanArgs a;
   ScatterArgs xa;
   assign_args(w, order, mass, tile_mass, n, hc, zre, F, status, spin_limit, order_b, mass_b, pick, &ta, &a, &xa);
   if (tile_mass && nsums >= 0) ta.ntiles = nsums;
+  if (fell) {
+    a.fell = fell->fell;
+    a.order_a = fell->order_a;
+    a.mass_a = fell->mass_a;
+  }
   cudaError_t e = cudaMemsetAsync(w.ctrl, 0, kAssignCtrlBytes, s);
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(w.state, 0, (size_t)tiles * sizeof(unsigned long long), s);
@@ -590,7 +600,8 @@ cudaError_t assign_impl(const AssignWork& w, const uint32_t* order, const float*
   // and matching 1.0e6 cells 154 -> 145 us, 3.0e6 274 -> 272, 1.0e7 610 -> 618.
   // (Also when the result may overwrite what the scan reads.)
   const bool direct = n <= (gather ? kDirectGatherMaxCells : kDirectMaxCells) && disjoint(zre, n, order, n) && disjoint(zre, n, mass, n) &&
-                      disjoint(zre, n, order_b, n) && disjoint(zre, n, mass_b, n) && disjoint(zre, n, F, n);
+                      disjoint(zre, n, order_b, n) && disjoint(zre, n, mass_b, n) && disjoint(zre, n, a.order_a, n) && disjoint(zre, n, a.mass_a, n) &&
+                      disjoint(zre, n, F, n);
   if (direct) a.zre = zre;
   auto launch = [&](auto gt, auto ft, auto lt, auto dt) {
     launch_pdl(k_scan_assign<decltype(gt)::value, decltype(ft)::value, decltype(lt)::value, decltype(dt)::value>, g,

@@ -60,6 +60,9 @@ struct ScanArgs {
   const uint32_t* order_b;  // with pick: the sort's results sit in (order, mass)
   const float* mass_b;      // for an odd pass count and in (order_b, mass_b) else
   const int* pick;          // &SortCtrl::npasses or null
+  const uint32_t* fell;     // if not null, and *fell is 0, they sit in (order, mass) after all, and
+  const uint32_t* order_a;  // else for an odd pass count in (order_a, mass_a)
+  const float* mass_a;
   int64_t n;
   const unsigned long long* Xq;
   const int* qshift;                // fixed-point shift s of the masses
@@ -156,6 +159,13 @@ cudaError_t tomo_fill(float* z, int64_t n, int num_sms, cudaStream_t s);
 cudaError_t tomo_mask(float* J, const float* z, int64_t n, SortCtrl* ctrl, int num_sms, cudaStream_t s);
 cudaError_t tomo_merge(float* z, const float* ztmp, int64_t n, float z_low, bool last, int num_sms, cudaStream_t s);
 
+// A ranking by splitting (order, mass), or its fallback's (see ScanArgs).
+struct FellArgs {
+  const uint32_t* fell;
+  const uint32_t* order_a;
+  const float* mass_a;
+};
+
 // mass_in_rank_order: mass[n] belongs to rank n (sort payload) instead of to
 // cell n.  tile_mass: per-tile partial mass sums from the ranking (summed in
 // the thresholds kernel); null means one reduction pass over mass.
@@ -164,6 +174,6 @@ cudaError_t assign_impl(const AssignWork& w, const uint32_t* order, const float*
                         const unsigned long long* tile_mass, int64_t n, const HistoryCoeffs& hc, float* zre, double* F,
                         unsigned int* status, cudaStream_t s, FftProfile* prof, unsigned int spin_limit,
                         const uint32_t* order_b = nullptr, const float* mass_b = nullptr, const int* pick = nullptr,
-                        int64_t nsums = -1);
+                        int64_t nsums = -1, const FellArgs* fell = nullptr);
 
 }  // namespace amber

@@ -28,8 +28,9 @@
 //                  masses the bucket is also matched there (scan.cuh): its rank
 //                  order never goes to memory
 //   fallback     : a field the map does not balance (a bucket outgrows its
-//                  region) is ranked by the digit passes, in one cooperative
-//                  launch that otherwise ends at once
+//                  region, or the map sees it coming) is ranked by the digit
+//                  passes, in one cooperative launch that otherwise ends at
+//                  once: 8.3 ms a pass at 1024^3, 6.9 in launches of their own
 //
 // A stable digit pass pays for its order with eight ballots per cell and is
 // bound by instruction issue (6.6 ms each at 1024^3); a split needs none, carries
@@ -62,6 +63,7 @@ __device__ __forceinline__ void msd_map_body(const MsdArgs& a, uint32_t blk, uin
   if (gt == 0) {
     a.mc->overflow = 0;
     a.mc->bar = 0;
+    a.mc->given_up = 0;
     // what amber_sort_passes reports: the digits the key range would take
     const int bits = 32 - __clz((int)((uint32_t)a.ctrl->kmax - (uint32_t)a.ctrl->kmin));
     a.ctrl->npasses = max((bits + a.digit_bits - 1) / a.digit_bits, 1);
@@ -171,6 +173,7 @@ __device__ __forceinline__ void msd_map_body(const MsdArgs& a, uint32_t blk, uin
   for (uint32_t i = total + tid; i <= (uint32_t)kMsdKnots; i += NT) a.mc->map[i] = 0xffffffffu;
   if (tid == 0) {
     a.mc->equal = equal ? R.L - 2 : -1;
+    if (!equal && a.n > kMsdTieCells && H > (a.n > kMsdTieCells2 ? kMsdTieSpans2 : kMsdTieSpans)) a.mc->overflow = a.mc->given_up = 1;
     a.mc->done = 0;
   }
 }
@@ -225,7 +228,9 @@ __device__ __forceinline__ void msd_split_body(const MsdArgs& a, uint32_t blk, u
   bool bad = false;
   MassSum msum;
   uint32_t done = 0;
-  for (uint32_t tile = blk; tile < tiles; tile += nblk) {
+  // where the map has given up, the masses are summed and nothing is split
+  const bool given_up = FIRST && a.n > kMsdTieCells && a.mc->given_up;
+  for (uint32_t tile = blk; tile < tiles && !given_up; tile += nblk) {
     uint32_t start, have, bucket = 0;
     if (FIRST) {
       start = tile * (uint32_t)TILE;
@@ -354,6 +359,18 @@ __device__ __forceinline__ void msd_split_body(const MsdArgs& a, uint32_t blk, u
     if (FIRST && MASS && (++done & 511u) == 0) msum.flush();
   }
   if (FIRST && MASS) {
+    if (given_up) {  // fewer than 2^13 masses per thread
+      const uint32_t step = nblk * NT;
+      uint32_t i = blk * NT + tid;
+      for (; i + 7u * step < n; i += 8u * step) {  // (n <= 2^30)
+        float m[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) m[q] = min_[i + q * step];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) msum.add(m[q], bad);
+      }
+      for (; i < n; i += step) msum.add(min_[i], bad);
+    }
     msum.flush();
     u128 t = msum.slow;
 #pragma unroll

@@ -28,12 +28,23 @@ constexpr int kMsdAvg = kMsdCap * 5 / 6;                    // cells per final b
 constexpr int kMsdMinAvg = 320;                             // fewer where that leaves SMs idle
 constexpr int kMsdSub = 8192;                               // sub-buckets of a final bucket
 
+// Fields of so many cells with more heavy spans than this, but too few for equal
+// knots, reach down to zero through dozens of octaves.  There the transforms'
+// rounding leaves thousands of cells with one and the same intensity (multiples of
+// 2^-22; 1024^3 4276 cells at l = 1, 1177 at l = 1.5), which no map can spread
+// over buckets: they take the digit passes at once, before anything is split.
+// (Heavy spans at 512^3: 33 at l = 2, 59 at 1, 78 at 0.5; at 1024^3: 47 at 2, 68
+// at 1.5, 84 at 1.  Smaller fields leave no such ties.)
+constexpr int64_t kMsdTieCells = 1 << 26, kMsdTieCells2 = 1 << 28;
+constexpr uint32_t kMsdTieSpans = 64, kMsdTieSpans2 = 50;
+
 // Device control block; zero when created, left clean by every ranking.
 struct MsdCtrl {
-  uint32_t overflow;  // bit 0: a first-split bucket, bit 1: a second-split bucket outgrew its region
+  uint32_t overflow;  // bit 0: a first-split bucket outgrew its region (or given_up), bit 1: a second-split bucket did
   uint32_t done;      // CTAs of the map kernel that finished
   uint32_t bar;       // grid barrier of the fallback
-  uint32_t pad[61];
+  uint32_t given_up;  // by the map: ties that no map can spread
+  uint32_t pad[60];
   uint32_t hist[kMsdSpans << kMsdMaxFine];
   uint32_t map[kMsdKnots + 4];
   int32_t span[kMsdSpans];  // knot of key k in a span: (k >> (span & 31)) + (span >> 5)
@@ -99,8 +110,6 @@ struct FallbackArgs {
   const float* mass1;
   uint32_t nb1, cap1;
   int fine;
-  uint32_t* order_to;  // or null: the ranking (and masses) are copied here
-  float* mass_to;
 };
 cudaError_t sort_fallback(const FallbackArgs& f, bool with_mass, int num_sms, cudaStream_t s);
 

@@ -576,28 +576,17 @@ __device__ __forceinline__ void sort_fallback_body(const FallbackArgs& f) {
       else sort_pass_body<float, RB, false, MASS, false>(f.pass[p]);
       __syncthreads();
     }
-    if ((p < 3 || f.order_to) && !grid_barrier(&f.mc->bar, ++round, kSpinLimit, status)) return;
-  }
-  if (f.order_to) {
-    // pass p writes the A side if p is even
-    const int last = f.hist.ctrl->npasses - 1;
-    const uint32_t* v = f.pass[last].vout;
-    const float* m = f.pass[last].mout;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < f.hist.n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-      f.order_to[i] = v[i];
-      if (MASS) f.mass_to[i] = m[i];
-    }
+    if (p < 3 && !grid_barrier(&f.mc->bar, ++round, kSpinLimit, status)) return;
   }
 }
 
 template <bool MASS>
-__global__ void __launch_bounds__(kSortThreads, 2) k_sort_fallback(const FallbackArgs f) {
+__global__ void __launch_bounds__(kSortThreads, AMBER_SORT_MINB) k_sort_fallback(const FallbackArgs f) {
   sort_fallback_body<MASS>(f);
 }
 
 // Several rankings, one after another (each with its own barrier word).
-__global__ void __launch_bounds__(kSortThreads, 2) k_sort_fallback_multi(const FallbackArgs* __restrict__ args, int M) {
+__global__ void __launch_bounds__(kSortThreads, AMBER_SORT_MINB) k_sort_fallback_multi(const FallbackArgs* __restrict__ args, int M) {
   __shared__ FallbackArgs f;
   for (int i = 0; i < M; ++i) {
     if (*reinterpret_cast<volatile uint32_t*>(&args[i].mc->overflow) == 0) continue;  // the same on every thread

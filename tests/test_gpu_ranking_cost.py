@@ -80,3 +80,53 @@ def test_solve_with_short_mean_free_paths(B, n, l_mfp):
     assert float(J.min()) < 1e-3 * float(J.median())
     assert torch.equal(z, ref)
     assert t < 1.25 * base
+
+
+@pytest.mark.parametrize("source,l_mfp", [("recipe", 0.5), ("sparse", 0.6)])
+def test_solve_of_fields_that_ties_unbalance(B, source, l_mfp):
+    # mean free paths below a cell leave over a thousand cells with one intensity
+    # near zero (the transforms' rounding), sparse sources far more: the digit
+    # passes rank them, at little more than their own price, in each form
+    from paper_2109_10375_gb300 import synth
+    n, box = 512, 400.0
+    S, m = synth.realisation(n, box, 4, device="cuda")
+    if source == "sparse":
+        S = torch.zeros_like(S)
+        S.view(-1)[torch.randint(0, n ** 3, (1000,), generator=torch.Generator(device="cuda").manual_seed(1),
+                                 device="cuda")] = 1.0
+    h = B.history(8.0, 4.0, 3.0)
+    with B.Context(n ** 3) as ctx:
+        z, J, z2 = torch.empty_like(S), torch.empty_like(S), torch.empty_like(S)
+        t = _ms(lambda: ctx.solve(S, m, box, l_mfp, h, out=z))
+        t_J = _ms(lambda: ctx.solve(S, m, box, l_mfp, h, out=z2, J_out=J))
+        assert torch.equal(z2, z)
+        order, mass = torch.empty(n ** 3, dtype=torch.int32, device="cuda"), torch.empty(n ** 3, device="cuda")
+        ctx.solve_ex(S, m, box, l_mfp, h, z2, order, mass)
+        assert torch.equal(z2, z)
+        zh = torch.empty(S.shape).pin_memory()
+        ctx.solve_host(S.cpu().pin_memory(), m.cpu().pin_memory(), box, l_mfp, h, zh)
+        assert ctx.sync_status() == 0
+        assert torch.equal(zh.cuda(), z)
+        ref = torch.sort(-(J.view(-1) + 0.0), stable=True).indices
+        assert torch.equal(order, ref.to(torch.int32)) and torch.equal(mass, m.view(-1)[ref])
+        del ref, order, mass, zh
+        ctx.set_tuning(n, sort_digit_bits=8, fuse_histogram=1)  # digit passes
+        digits = _ms(lambda: ctx.solve(S, m, box, l_mfp, h, out=z2))
+        assert ctx.sync_status() == 0
+    assert torch.equal(z, z2)
+    if source == "recipe":
+        assert t < 1.35 * digits and t_J < 1.35 * digits
+
+
+@pytest.mark.parametrize("kind", ["lump", "small lump", "coarse"])
+@pytest.mark.parametrize("n", [1 << 24, 20_000_003])
+def test_rank_of_large_fields_that_overflow(B, n, kind):
+    J = _octaves(n)
+    if kind == "lump":
+        J[n // 4:n // 2] = 0.5
+    elif kind == "small lump":
+        J[n // 4:n // 4 + 6000] = 0.5
+    else:
+        J = J.mul(300.0).round_()
+    with B.Context(n) as ctx:
+        _rank_ms(B, ctx, J)
