@@ -24,8 +24,9 @@
 //   k_msd_local  : a final bucket (3840 cells on average, at most 4608) in
 //                  shared memory: a counting pass over 8192 sub-buckets, linear
 //                  in (key, cell) over the bucket's range, leaves each cell among
-//                  about 1.5; it then counts which of those precede it.  With the
-//                  masses the bucket is also matched there (scan.cuh): its rank
+//                  about 1.5; it then counts which of those precede it.  Where
+//                  ties share a sub-bucket they are counted again by cell, or
+//                  merge sorted (sort_ties).  With the masses the bucket is also matched there (scan.cuh): its rank
 //                  order never goes to memory
 //   fallback     : a field the map does not balance (a bucket outgrows its
 //                  region, or the map sees it coming) is ranked by the digit
@@ -402,6 +403,248 @@ __global__ void __launch_bounds__(512, 2) k_msd_split_multi(const MsdArgs* __res
   msd_split_body<512, kMsdTileA / 512, FIRST, true>(a, blockIdx.x, gridDim.x);
 }
 
+// A final bucket's sub-buckets: linear in (key, cell) over what it holds.
+struct SubMap {
+  int mode;  // 0: by key, 1: by key and cell, 2: by cell
+  int ishift;
+  uint32_t off, mul_k, mul_i, F;
+  __device__ __forceinline__ uint32_t sub(uint32_t key, uint32_t idx) const {
+    if (mode == 0) return __umulhi(key - off, mul_k);
+    if (mode == 1) return (key - off) * F + __umulhi(idx << ishift, F);
+    return mul_i ? __umulhi(idx - off, mul_i) : idx - off;
+  }
+  // of cells with one key: the place in their sub-bucket as a fraction of 2^32
+  __device__ __forceinline__ uint32_t frac(uint32_t idx) const {
+    return mode == 0 ? idx << ishift : mode == 1 ? (idx << ishift) * F : (idx - off) * mul_i;
+  }
+};
+
+// A sub-bucket of more cells than kMsdTies, mostly ties, sends its bucket to
+// sort_ties: counting each against all others is quadratic.  Up to kMsdTiesMost it
+// may still be counted there.  (With 12 the tails of ordinary fields take it too
+// often, 512^3 l = 3 5.47 -> 5.52 ms, with 16 5.48; ranking 1.0e7 cells with 20 a
+// value 0.30 ms, with 24 0.37, with 64 0.36.)
+constexpr uint32_t kMsdTies = 16, kMsdTiesMost = 64;
+
+// The counts of S sub-buckets (packed 16-bit words) become starts, with the end
+// behind the last one; true if one holds more than `limit`.  Called by the whole
+// CTA, with a barrier at its end.
+template <int NT, int S>
+__device__ __forceinline__ bool counts_to_starts(uint32_t* sc, uint32_t* wsum, uint32_t limit) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint4* sc4 = reinterpret_cast<uint4*>(sc);
+  constexpr int PER = S / 2 / NT;
+  static_assert(PER % 4 == 0, "whole 16-byte words per thread");
+  uint32_t w[PER], sum = 0;
+#pragma unroll
+  for (int q = 0; q < PER / 4; ++q) {
+    const uint4 v = sc4[tid * (PER / 4) + q];
+    w[4 * q] = v.x;
+    w[4 * q + 1] = v.y;
+    w[4 * q + 2] = v.z;
+    w[4 * q + 3] = v.w;
+  }
+  uint32_t most = 0;
+#pragma unroll
+  for (int q = 0; q < PER; ++q) most = __vmaxu2(most, w[q]);
+#pragma unroll
+  for (int q = 0; q < PER; ++q) sum += w[q];  // both 16-bit halves at once (each below 2^13)
+  sum = (sum & 0xffffu) + (sum >> 16);
+  uint32_t x = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) wsum[warp] = x;
+  __syncthreads();
+  uint32_t st = x - sum + warps_before(wsum, NT / 32, lane, warp);
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const uint32_t c0 = w[q] & 0xffffu, c1 = w[q] >> 16;
+    w[q] = st | (st + c0) << 16;
+    st += c0 + c1;
+  }
+#pragma unroll
+  for (int q = 0; q < PER / 4; ++q)
+    sc4[tid * (PER / 4) + q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+  if (tid == NT - 1) sc[S / 2] = st;
+  return __syncthreads_or((most & 0xffffu) > limit || (most >> 16) > limit);
+}
+
+// The rest of the local sort where a sub-bucket holds more than kMsdTies cells, from
+// the starts and the `have` composites in shared memory.  Where the cells of each
+// such sub-bucket share one key, they are counted once more, into as many places as
+// they are by their cells' fractions.  Where that leaves more than kMsdTiesMost in
+// one, or was not possible, the composites are merge sorted: a run of IT per thread in registers, then runs
+// pairwise by merge path, pairs that follow on each other untouched; each cell then
+// finds its rank by bisection.  Cells and masses end in sidx and smass (over the
+// composites).  The cells are read again: kept over the call they would spill in
+// every bucket.  Called by the whole CTA.
+// Ranking seven octaves with 150 and 600 cells a value, counted against one another
+// and now (no ties; digit passes): 2^22 cells 0.49 and 1.16 -> 0.15 ms (0.13;
+// 0.19), 1.0e7 1.06 and 2.45 -> 0.28 (0.23; 0.32), 2^27 4.8 and 8.5 -> 3.0 (2.57;
+// 2.9).
+template <int NT, int IT, int S, bool MASS>
+__device__ __noinline__ void sort_ties(uint32_t have, const uint2* __restrict__ kv, const float* __restrict__ mass,
+                                       const SubMap* shared_map) {
+  static_assert((NT & (NT - 1)) == 0, "runs double up to the whole array");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  unsigned long long* comp = reinterpret_cast<unsigned long long*>(smem_raw);  // [NT IT]
+  uint32_t* sc = reinterpret_cast<uint32_t*>(comp + NT * IT);                  // [S/2 + 4]
+  const uint16_t* st16 = reinterpret_cast<const uint16_t*>(sc);
+  __shared__ uint32_t wsum[NT / 32];
+  const int tid = threadIdx.x;
+  const SubMap sub = *shared_map;
+  uint32_t idx[IT], rank[IT];
+  bool sorted;
+  {
+    uint32_t key[IT];
+    bool differ = false, most = false;
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const uint32_t p = it * NT + tid;
+      if (p < have) {
+        const uint2 c = kv[p];
+        key[it] = c.x;
+        idx[it] = c.y;
+      }
+    }
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const uint32_t p = it * NT + tid;
+      if (p < have) {
+        const uint32_t s = sub.sub(key[it], idx[it]), b0 = st16[s], c = st16[s + 1] - b0;
+        rank[it] = b0;
+        if (c > kMsdTies) {
+          rank[it] += __umulhi(sub.frac(idx[it]), c);
+          differ |= key[it] != (uint32_t)(comp[b0] >> 32);
+          most |= c > kMsdTiesMost;
+        }
+      }
+    }
+    if (__syncthreads_or(differ)) {
+      sorted = !__syncthreads_or(most);
+#pragma unroll
+      for (int it = 0; it < IT; ++it)
+        if (it * NT + tid < have) rank[it] = sub.sub(key[it], idx[it]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < S / 8 / NT; ++i) reinterpret_cast<uint4*>(sc)[i * NT + tid] = make_uint4(0, 0, 0, 0);
+      __syncthreads();
+#pragma unroll
+      for (int it = 0; it < IT; ++it) {
+        const uint32_t p = it * NT + tid;
+        if (p < have) {
+          const uint32_t s = rank[it];  // below `have`
+          const int sh = (s & 1u) * 16;
+          rank[it] = s << 16 | ((atomicAdd(&sc[s >> 1], 1u << sh) >> sh) & 0xffffu);
+        }
+      }
+      __syncthreads();
+      sorted = !counts_to_starts<NT, S>(sc, wsum, kMsdTiesMost);
+#pragma unroll
+      for (int it = 0; it < IT; ++it) {
+        const uint32_t p = it * NT + tid;
+        if (p < have) {
+          const uint32_t s = rank[it] >> 16;
+          comp[st16[s] + (rank[it] & 0xffffu)] = (unsigned long long)key[it] << 32 | idx[it];
+          rank[it] = s;
+        }
+      }
+      __syncthreads();
+    }
+    if (sorted) {
+#pragma unroll
+      for (int it = 0; it < IT; ++it) {
+        const uint32_t p = it * NT + tid;
+        if (p < have) {
+          const uint32_t b0 = st16[rank[it]], b1 = st16[rank[it] + 1];
+          const unsigned long long me = (unsigned long long)key[it] << 32 | idx[it];
+          uint32_t r = b0;
+          if (b1 - b0 > 1u)
+            for (uint32_t q = b0; q < b1; ++q) r += comp[q] < me;
+          rank[it] = r;
+        }
+      }
+    }
+  }
+  if (!sorted) {
+    unsigned long long v[IT];
+#pragma unroll
+    for (int i = 0; i < IT; ++i) v[i] = (uint32_t)(tid * IT + i) < have ? comp[tid * IT + i] : ~0ull;
+#pragma unroll
+    for (int r = 0; r < IT; ++r)
+#pragma unroll
+      for (int i = r & 1; i + 1 < IT; i += 2) {
+        const unsigned long long x = v[i], y = v[i + 1];
+        v[i] = x < y ? x : y;
+        v[i + 1] = x < y ? y : x;
+      }
+#pragma unroll
+    for (int i = 0; i < IT; ++i) comp[tid * IT + i] = v[i];
+    __syncthreads();
+#pragma unroll 1
+    for (int w = 1; w < NT; w *= 2) {
+      const int la = w * IT, d = (tid & (2 * w - 1)) * IT;
+      const unsigned long long *A = comp + (tid & ~(2 * w - 1)) * IT, *B = A + la;
+      const bool apart = A[la - 1] <= B[0];
+      if (!apart) {
+        int lo = max(0, d - la), hi = min(d, la);  // before this thread's first output: lo of A, d - lo of B
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (A[mid] <= B[d - 1 - mid]) lo = mid + 1;
+          else hi = mid;
+        }
+        int b = d - lo;
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+          const bool from_a = b >= la || (lo < la && A[lo] <= B[b]);
+          v[i] = from_a ? A[lo++] : B[b++];
+        }
+      }
+      __syncthreads();
+      if (!apart) {
+#pragma unroll
+        for (int i = 0; i < IT; ++i) comp[tid * IT + i] = v[i];
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const uint32_t p = it * NT + tid;
+      if (p < have) {
+        const uint2 c = kv[p];
+        const unsigned long long me = (unsigned long long)c.x << 32 | c.y;
+        uint32_t lo = 0, hi = have - 1;
+        while (lo < hi) {
+          const uint32_t mid = (lo + hi) >> 1;
+          if (comp[mid] < me) lo = mid + 1;
+          else hi = mid;
+        }
+        idx[it] = c.y;
+        rank[it] = lo;
+      }
+    }
+  }
+  uint32_t* sidx = reinterpret_cast<uint32_t*>(smem_raw);
+  float* smass = reinterpret_cast<float*>(sidx + NT * IT);
+  float m[IT];
+  if (MASS) {
+#pragma unroll
+    for (int it = 0; it < IT; ++it)
+      if (it * NT + tid < have) m[it] = mass[it * NT + tid];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    if (it * NT + tid < have) {
+      sidx[rank[it]] = idx[it];
+      if (MASS) smass[rank[it]] = m[it];
+    }
+  }
+}
+
 // SCAN: with the masses, matched here as well (LIN: see scan.cuh), each redshift
 // stored in its place.
 template <bool MASS, bool SCAN, bool LIN>
@@ -417,6 +660,7 @@ __device__ __forceinline__ void msd_local_body(const MsdArgs& a, const ScanArgs&
   __shared__ uint32_t wsum[NT / 32], wlo[NT / 32], whi[NT / 32], wbase[NT / 32];
   __shared__ unsigned long long wmass[NT / 32];
   __shared__ uint32_t s_tile;
+  __shared__ SubMap s_map;
   const bool fell = *reinterpret_cast<volatile uint32_t*>(&a.mc->overflow) != 0;
   if (!SCAN && fell) return;  // the fallback has written the ranking
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -512,16 +756,14 @@ __device__ __forceinline__ void msd_local_body(const MsdArgs& a, const ScanArgs&
       lb.start(sa, b, t, lane);
     }
     const uint32_t span = hi - lo;
-    uint32_t off = lo, mul_k = 0, mul_i = 0, F = 0;
-    int mode;  // 0: by key, 1: by key and cell, 2: by cell
+    SubMap sub{0, a.idx_shift, lo, 0, 0, 0};
     if (span >= (uint32_t)S - 1u) {
-      mode = 0;
-      mul_k = __float2uint_rz((float)S * 4294967296.0f / ((float)span + 1.0f) * 0.9999f);
+      sub.mul_k = __float2uint_rz((float)S * 4294967296.0f / ((float)span + 1.0f) * 0.9999f);
     } else if (span > 0) {
-      mode = 1;
-      F = (uint32_t)S / (span + 1u);
+      sub.mode = 1;
+      sub.F = (uint32_t)S / (span + 1u);
     } else {
-      mode = 2;
+      sub.mode = 2;
       uint32_t ilo = 0xffffffffu, ihi = 0;
 #pragma unroll
       for (int it = 0; it < IT; ++it) {
@@ -541,62 +783,25 @@ __device__ __forceinline__ void msd_local_body(const MsdArgs& a, const ScanArgs&
       __syncthreads();
       ilo = __reduce_min_sync(0xffffffffu, lane < NT / 32 ? wlo[lane] : 0xffffffffu);
       ihi = __reduce_max_sync(0xffffffffu, lane < NT / 32 ? whi[lane] : 0u);
-      off = ilo;
+      sub.off = ilo;
       const uint32_t isp = ihi - ilo;
-      mul_i = isp >= (uint32_t)S - 1u
+      sub.mul_i = isp >= (uint32_t)S - 1u
                   ? __float2uint_rz((float)S * 4294967296.0f / ((float)isp + 1.0f) * 0.9999f)
                   : 0u;  // 0: the offset itself
     }
+    if (tid == 0) s_map = sub;
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
       const uint32_t p = it * NT + tid;
       if (p < have) {
-        uint32_t s;
-        if (mode == 0) s = __umulhi(key[it] - off, mul_k);
-        else if (mode == 1) s = (key[it] - off) * F + __umulhi(idx[it] << a.idx_shift, F);
-        else s = mul_i ? __umulhi(idx[it] - off, mul_i) : idx[it] - off;
+        const uint32_t s = sub.sub(key[it], idx[it]);
         const int sh = (s & 1u) * 16;
         ss[it] = s << 16 | ((atomicAdd(&sc[s >> 1], 1u << sh) >> sh) & 0xffffu);
       }
     }
     if (SCAN && warp == 0) lb.poll(sa, lane);
     __syncthreads();
-    {
-      constexpr int PER = S / 2 / NT;
-      static_assert(PER % 4 == 0, "whole 16-byte words per thread");
-      uint32_t w[PER], sum = 0;
-#pragma unroll
-      for (int q = 0; q < PER / 4; ++q) {
-        const uint4 v = sc4[tid * (PER / 4) + q];
-        w[4 * q] = v.x;
-        w[4 * q + 1] = v.y;
-        w[4 * q + 2] = v.z;
-        w[4 * q + 3] = v.w;
-      }
-#pragma unroll
-      for (int q = 0; q < PER; ++q) sum += w[q];  // both 16-bit halves at once (each below 2^13)
-      sum = (sum & 0xffffu) + (sum >> 16);
-      uint32_t x = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-      }
-      if (lane == 31) wsum[warp] = x;
-      __syncthreads();
-      uint32_t st = x - sum + warps_before(wsum, NT / 32, lane, warp);
-#pragma unroll
-      for (int q = 0; q < PER; ++q) {
-        const uint32_t c0 = w[q] & 0xffffu, c1 = w[q] >> 16;
-        w[q] = st | (st + c0) << 16;
-        st += c0 + c1;
-      }
-#pragma unroll
-      for (int q = 0; q < PER / 4; ++q)
-        sc4[tid * (PER / 4) + q] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
-      if (tid == NT - 1) sc[S / 2] = st;
-    }
-    __syncthreads();
+    const bool ties = counts_to_starts<NT, S>(sc, wsum, kMsdTies);
     const uint16_t* st16 = reinterpret_cast<const uint16_t*>(sc);
 #pragma unroll
     for (int it = 0; it < IT; ++it) {
@@ -609,27 +814,32 @@ __device__ __forceinline__ void msd_local_body(const MsdArgs& a, const ScanArgs&
     }
     if (SCAN && warp == 0) lb.poll(sa, lane);
     __syncthreads();
+    if (ties) {  // uniform
+      sort_ties<NT, IT, S, MASS>(have, kv, mv_in, &s_map);
+      if (SCAN && warp == 0) lb.poll(sa, lane);
+    } else {
 #pragma unroll
-    for (int it = 0; it < IT; ++it) {
-      const uint32_t p = it * NT + tid;
-      if (p < have) {
-        const uint32_t b0 = ss[it] & 0xffffu, b1 = st16[(ss[it] >> 16) + 1];
-        uint32_t r = b0;
-        if (b1 - b0 > 1u) {
-          const unsigned long long me = (unsigned long long)key[it] << 32 | idx[it];
-          for (uint32_t q = b0; q < b1; ++q) r += comp[q] < me;
+      for (int it = 0; it < IT; ++it) {
+        const uint32_t p = it * NT + tid;
+        if (p < have) {
+          const uint32_t b0 = ss[it] & 0xffffu, b1 = st16[(ss[it] >> 16) + 1];
+          uint32_t r = b0;
+          if (b1 - b0 > 1u) {
+            const unsigned long long me = (unsigned long long)key[it] << 32 | idx[it];
+            for (uint32_t q = b0; q < b1; ++q) r += comp[q] < me;
+          }
+          ss[it] = r;
         }
-        ss[it] = r;
       }
-    }
-    if (SCAN && warp == 0) lb.poll(sa, lane);
-    __syncthreads();
+      if (SCAN && warp == 0) lb.poll(sa, lane);
+      __syncthreads();
 #pragma unroll
-    for (int it = 0; it < IT; ++it) {
-      const uint32_t p = it * NT + tid;
-      if (p < have) {
-        sidx[ss[it]] = idx[it];
-        if (MASS) smass[ss[it]] = m[it];
+      for (int it = 0; it < IT; ++it) {
+        const uint32_t p = it * NT + tid;
+        if (p < have) {
+          sidx[ss[it]] = idx[it];
+          if (MASS) smass[ss[it]] = m[it];
+        }
       }
     }
   }

@@ -130,3 +130,32 @@ def test_rank_of_large_fields_that_overflow(B, n, kind):
         J = J.mul(300.0).round_()
     with B.Context(n) as ctx:
         _rank_ms(B, ctx, J)
+
+
+@pytest.mark.parametrize("n", [1 << 22, 10_000_019])
+@pytest.mark.parametrize("ties", [150, 600])
+def test_rank_of_fields_with_many_cells_per_value(B, n, ties):
+    # a bucket of the local sort then holds a few values, far apart and with
+    # hundreds of cells each; ranking them within the bucket must not grow with
+    # the square of that (the digit passes take 1.3 times what no ties take)
+    u = torch.rand(n, generator=torch.Generator(device="cuda").manual_seed(ties), device="cuda")
+    with B.Context(n) as ctx:
+        base = _rank_ms(B, ctx, u.mul(7.0).exp2_())
+        values = n // ties
+        t = _rank_ms(B, ctx, u.mul(values).floor_().mul_(7.0 / values).exp2_())
+        assert t < 1.6 * base
+
+
+def test_rank_of_one_bucket_of_ties_among_others(B):
+    # sub-buckets at and above the counts from which they are counted again, and sorted
+    with B.Context(1 << 20) as ctx:
+        for n in (4096, 4600, 100_003, 1 << 20):
+            x = _octaves(n)
+            for lump in (16, 17, 64, 65, 130, 2000, 4000):
+                y = x.clone()
+                at = torch.randperm(n, generator=torch.Generator(device="cuda").manual_seed(lump), device="cuda")
+                y[at[:lump]] = 0.75
+                y[at[lump:lump + 90]] = 0.75000006
+                order = ctx.rank(y)
+                assert ctx.sync_status() == 0
+                assert torch.equal(order, torch.sort(-(y + 0.0), stable=True).indices.to(torch.int32)), (n, lump)
