@@ -243,12 +243,12 @@ __global__ void __launch_bounds__(kThreshThreads) k_thresholds(const ThreshArgs 
   thresholds_body(A, (int)blockIdx.x);
 }
 
-// CTA (x, y): points of CTA x of item y's table.
+// CTA (x, y): points of CTA y of item x's table (a grid's y ends at 65535).
 __global__ void __launch_bounds__(kThreshThreads) k_thresholds_multi(const ThreshArgs* __restrict__ args) {
   __shared__ ThreshArgs A;
-  if (threadIdx.x == 0) A = args[blockIdx.y];
+  if (threadIdx.x == 0) A = args[blockIdx.x];
   __syncthreads();
-  if ((int)blockIdx.x * kThreshPoints < A.M) thresholds_body(A, (int)blockIdx.x);
+  if ((int)blockIdx.y * kThreshPoints < A.M) thresholds_body(A, (int)blockIdx.y);
 }
 
 // ---------------------------------------------------------------------------
@@ -630,7 +630,7 @@ cudaError_t assign_impl(const AssignWork& w, const uint32_t* order, const float*
 }
 
 cudaError_t assign_multi(const AssignMulti& m, cudaStream_t s) {
-  k_thresholds_multi<<<dim3((unsigned)((m.max_table + kThreshPoints - 1) / kThreshPoints), (unsigned)m.M),
+  k_thresholds_multi<<<dim3((unsigned)m.M, (unsigned)((m.max_table + kThreshPoints - 1) / kThreshPoints)),
                        kThreshThreads, 0, s>>>(m.thresh);
   if (m.scan_tiles[0]) k_scan_assign_multi<false><<<m.scan_tiles[0], kScanThreads, 0, s>>>(m.scan[0], m.scan_prefix[0], m.Mg[0]);
   if (m.scan_tiles[1]) k_scan_assign_multi<true><<<m.scan_tiles[1], kScanThreads, 0, s>>>(m.scan[1], m.scan_prefix[1], m.Mg[1]);
