@@ -1233,10 +1233,12 @@ static int batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, con
   };
   std::vector<ItemWs> iw(nitems);
   int64_t cells = 0, digit_cells = 0;
+  int64_t of_size[11] = {};  // cells by log2 of the grid size
   for (int i : ord) {
     ItemWs& w = iw[i];
     w.C = (int64_t)items[i].params.n * items[i].params.n * items[i].params.n;
     cells += w.C;
+    of_size[ilog2i(items[i].params.n)] += w.C;
   }
   for (int i : ord) {
     // Rankings by splitting share their launches where they are of one size and
@@ -1245,10 +1247,8 @@ static int batch_create(amber_batch** out, amber_ctx* const* ctxs, int nctx, con
     // batch).  The other items stay with the digit passes, which take mixed
     // sizes in one launch.
     ItemWs& w = iw[i];
-    int64_t of_size = 0;
-    for (int k : ord) of_size += items[k].params.n == items[i].params.n ? w.C : 0;
-    w.msd = split && items[i].params.n >= 64 && w.C <= kDirectMaxCells && of_size > kBatchSplitCells &&
-            sort_rank_env() < 0;
+    w.msd = split && items[i].params.n >= 64 && w.C <= kDirectMaxCells &&
+            of_size[ilog2i(items[i].params.n)] > kBatchSplitCells && sort_rank_env() < 0;
     if (w.msd) w.plan = msd_plan(w.C, true, c0->num_sms);
     else digit_cells += w.C;
   }
