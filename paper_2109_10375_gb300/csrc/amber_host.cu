@@ -204,8 +204,8 @@ static Plan make_plan(int64_t max_cells) {
   const size_t lb = 2 * sort_lookback_words(max_cells) * 4;
   // scan tiles of a given ranking, or final buckets of a ranking by splitting
   const int64_t buckets = msd_most_buckets(max_cells);
-  const int64_t rows = std::max<int64_t>((max_cells + kScanTile - 1) / kScanTile, buckets);
-  const size_t stt = (size_t)rows * sizeof(unsigned long long);
+  const int64_t tiles = (max_cells + kScanTile - 1) / kScanTile;
+  const size_t stt = (size_t)std::max(tiles, buckets) * sizeof(unsigned long long);
   size_t o = 0;
   auto take = [&](size_t bytes) { const size_t at = o; o += align256(bytes); return at; };
   p.off_spec = take(spec);
@@ -222,7 +222,7 @@ static Plan make_plan(int64_t max_cells) {
   p.off_invdx = take((size_t)kMaxTable * sizeof(float));
   p.off_lin = take((size_t)4 * kMaxTable * sizeof(float));
   p.off_state = take(stt);
-  p.off_btab = take((size_t)rows * (kMaxBuckets + 1) * sizeof(uint16_t));
+  p.off_btab = take((size_t)tiles * (kMaxBuckets + 1) * sizeof(uint16_t));  // (the local sort stores in place)
   p.off_tilemass = take(std::max<size_t>((size_t)sort_tiles(max_cells) * 16, 4096 * 16));
   p.off_msd = take(sizeof(MsdCtrl));
   p.off_msd_cnt2 = take((size_t)buckets * 4);

@@ -79,6 +79,16 @@ def test_workspace_plan(B):
         B.workspace_bytes((1 << 30) + 1)
 
 
+def test_workspace_holds_little_beyond_its_per_cell_arrays(B):
+    # 2^30 cells: half spectrum, six 4-byte arrays, look-back words of 2^18 digit
+    # tiles; the rest is the bucket table (2^17 scan tiles of 129 16-bit starts,
+    # 34 MB) and under 15 MB of counters, sums and tables
+    cells = 1 << 30
+    rest = B.workspace_bytes(cells) - (4 * 1024 * 1024 * 1028 + 24 * cells + 2 * (cells // 4096) * 512 * 4)
+    table = 2 * 129 * (cells // 8192)
+    assert table < rest < table + 15e6
+
+
 def test_create_without_gpu_reports_cuda_error(B):
     import torch
     if torch.cuda.is_available():
