@@ -257,8 +257,10 @@ int amber_solve_spectrum(amber_ctx *ctx, const void *d_spec, const float *d_mass
  *                    512 as 16 x 32, 256 as 32 x 8, 128 as 8 x 16);
  *   (FP32 rankings split their cells into buckets of like intensity and sort
  *   those on chip.  The three sort choices are those of the radix sort that
- *   ranks with fuse_histogram 1, in a batch, in the later intervals of a
- *   tomographic matching, and when AMBER_SORT_RANK is set.)
+ *   ranks with fuse_histogram 1, in a batch the sizes below 64^3, above 256^3
+ *   or with at most 2^23 cells in all, in the later intervals of a tomographic
+ *   matching, and everything when AMBER_SORT_RANK is set.  amber_autotune
+ *   times that radix sort.)
  *   sort_digit_bits  9 or 8: digit width of the radix sort (a few-octave
  *                    intensity field needs 27 bits: 3 passes of 9 bits, 4 of 8;
  *                    a 24-bit range takes 3 of either, the 8-bit ones cheaper);
@@ -329,9 +331,9 @@ int amber_get_tuning(amber_ctx *ctx, int n, amber_tuning_t *out);
  *    ranked by splitting (amber_batch_kernel_nodes).
  *  - The batch allocates its own workspace at creation (about 30 bytes per
  *    cell of all items together, 37 for those ranked by splitting, which are
- *    laid out for digit passes where that does not fit, plus the items'
- *    arguments); amber_batch_create
- *    and amber_create are the only calls that allocate.
+ *    laid out for digit passes where that does not fit or AMBER_SORT_RANK is
+ *    set, plus the items' arguments); amber_batch_create and amber_create are
+ *    the only calls that allocate.
  *  - ctxs[0] gives the device, the FFT twiddles (its max_cells must hold the
  *    largest grid), the status word that amber_sync_status(ctxs[0]) reads and
  *    the tuning; each grid size not yet tuned on ctxs[0] is autotuned on its

@@ -329,7 +329,6 @@ bool msd_setup(amber_ctx* c, const float* J, bool J_inside, const float* mass, b
   const bool small = n < kMsdSmallCells;
   if (small && p.kv1 + p.m1 > (int64_t)msd_small_words(c->max_cells)) return false;
   if (!small && (p.kv1 + p.m1 > inside || p.kv1 + p.m1 + p.kv2 + p.m2 > words)) return false;
-  if (n > c->max_cells) return false;
   uint32_t* at = small ? reinterpret_cast<uint32_t*>(c->ws + pl.off_msd_small) : block;
   MsdArgs& a = *out;
   a = MsdArgs{};

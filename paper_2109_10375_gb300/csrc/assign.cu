@@ -326,10 +326,10 @@ __global__ void __launch_bounds__(kScanThreads, AMBER_SCAN_MINB)
 }
 
 // z_re[cell] = z, bucket after bucket: CTA (bucket b, tile group g) copies
-// bucket b's run of every tile in its group (one tile per warp at the
-// default group size).  A warp takes its runs in rounds of four 32-pair
-// chunks: all the round's loads (lanes read a run coalesced), then its
-// stores, so the dependent load -> store chains overlap.  A
+// bucket b's run of every tile in its group, a tile per warp.  A warp takes
+// its run in rounds of four 32-pair chunks: all the round's loads (lanes read
+// a run coalesced), then its stores, so the dependent load -> store chains
+// overlap.  A
 // bucket's cells span a bounded region of z_re, so the permuted writes of
 // the CTAs working on it stay close together.
 __device__ __forceinline__ void scatter_back_body(const ScatterArgs& x, uint32_t blk) {
@@ -339,49 +339,31 @@ __device__ __forceinline__ void scatter_back_body(const ScatterArgs& x, uint32_t
   float* __restrict__ zre = x.zre;
   const int nbuckets = x.nbuckets, groups = x.groups;
   const int64_t tiles = x.tiles;
-  constexpr int TPW = 1;  // tiles per warp
   const int b = blk / groups;
   const int64_t g = blk - (int64_t)b * groups;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned long long stream_pol = l2_evict_first(), keep_pol = l2_evict_last();
-  const int64_t t0 = g * kBackTilesPerCta + warp;
-  // lane 0 fetches the tile's run bounds
-  int s_l = 0, e_l = 0;
-  if (lane < TPW && t0 + lane < tiles) {
-    const uint16_t* row = btab + (t0 + lane) * (nbuckets + 1);
-    s_l = row[b];
-    e_l = row[b + 1];
-  }
-  // rounds of 4 x 32 pairs per run: the loads of all the warp's runs, then the stores
-  constexpr int G = 4;
-  int len = e_l - s_l;
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) len = max(len, __shfl_xor_sync(0xffffffffu, len, o));
-  int s_k[TPW], e_k[TPW];
-#pragma unroll
-  for (int k = 0; k < TPW; ++k) {
-    s_k[k] = __shfl_sync(0xffffffffu, s_l, k);
-    e_k[k] = __shfl_sync(0xffffffffu, e_l, k);
-  }
+  const int64_t t = g * kBackTilesPerCta + warp;
+  if (t >= tiles) return;
+  const uint16_t* row = btab + t * (nbuckets + 1);
+  const int start = row[b], end = row[b + 1];
+  const int64_t base = t * kScanTile;
+  constexpr int G = 4;  // 32-pair chunks per round
 #pragma unroll 1
-  for (int j0 = 0; j0 < len; j0 += 32 * G) {
-    uint32_t c[TPW * G];
-    float zz[TPW * G];
+  for (int j0 = start; j0 < end; j0 += 32 * G) {
+    uint32_t c[G];
+    float zz[G];
 #pragma unroll
-    for (int k = 0; k < TPW; ++k) {
-#pragma unroll
-      for (int q = 0; q < G; ++q) {
-        const int i = s_k[k] + j0 + 32 * q + lane;
-        c[k * G + q] = 0xffffffffu;
-        if (i < e_k[k]) {
-          const int64_t at = (t0 + k) * kScanTile + i;
-          c[k * G + q] = ld_hint(bcell + at, stream_pol);
-          zz[k * G + q] = ld_hint(bz + at, stream_pol);
-        }
+    for (int q = 0; q < G; ++q) {
+      const int i = j0 + 32 * q + lane;
+      c[q] = 0xffffffffu;
+      if (i < end) {
+        c[q] = ld_hint(bcell + base + i, stream_pol);
+        zz[q] = ld_hint(bz + base + i, stream_pol);
       }
     }
 #pragma unroll
-    for (int q = 0; q < TPW * G; ++q)
+    for (int q = 0; q < G; ++q)
       if (c[q] != 0xffffffffu) st_hint(zre + c[q], zz[q], keep_pol);
   }
 }

@@ -59,16 +59,6 @@ __device__ __forceinline__ void count_ge_round(const unsigned long long* __restr
 
 constexpr int kScanWin = 64;  // thresholds one tile may span, staged in shared memory
 
-// LIN: a linear weighting (growth or volume).  The exact-integer threshold
-// test of the mass weighting is replaced by the margins h_j(n) in FP32: a
-// cell takes the largest table point j with h_j >= 0.  A margin is linear in
-// (n, M_n), so its extremes over the box that a run of ranks spans lie at the
-// corners.  Per tile every point is classified: jall is the largest one that
-// ionizes all of its cells, jtop the largest one that can ionize any.  From
-// jtop each warp walks down 32 points at a time to the first one its own box
-// allows, each thread from there to the first one its 16 ranks allow, and only
-// then each cell tests margins.  (The first tile of 128^3 spans over 1000 of
-// 2000 points; with every cell testing all of the tile's points it took 1.06 ms.)
 // Largest j in (jall, js] whose margin at (u, v) is not negative, jall if none,
 // for the lanes that ask: lane after lane, the warp testing 32 points at once.
 // (One lane stepping down 253 points for each of its cells took 120 us.)
@@ -181,6 +171,16 @@ struct LookBack {
 // The pairs go to bcell, bz + start.
 // DIRECT: the redshifts go straight to a.zre in cell order instead (bcell, bz
 // and the staging words unused): for fields that stay in L2.
+// LIN: a linear weighting (growth or volume).  The exact-integer threshold
+// test of the mass weighting is replaced by the margins h_j(n) in FP32: a
+// cell takes the largest table point j with h_j >= 0.  A margin is linear in
+// (n, M_n), so its extremes over the box that a run of ranks spans lie at the
+// corners.  Per tile every point is classified: jall is the largest one that
+// ionizes all of its cells, jtop the largest one that can ionize any.  From
+// jtop each warp walks down 32 points at a time to the first one its own box
+// allows, each thread from there to the first one its 16 ranks allow, and only
+// then each cell tests margins.  (The first tile of 128^3 spans over 1000 of
+// 2000 points; with every cell testing all of the tile's points it took 1.06 ms.)
 template <int NT, int IT, bool PAD, bool EARLY, bool DIRECT, bool WANT_F, bool LIN>
 __device__ __forceinline__ void scan_tile(const ScanArgs& a, ScanShared& S, LookBack& lb, uint32_t tile, uint32_t start,
                                           int cnt, const uint32_t* cell, const float* mv, unsigned long long run,
