@@ -26,8 +26,8 @@
 //                  in (key, cell) over the bucket's range, leaves each cell among
 //                  about 1.5; it then counts which of those precede it.  Where
 //                  ties share a sub-bucket they are counted again by cell, or
-//                  merge sorted (sort_ties).  With the masses the bucket is also matched there (scan.cuh): its rank
-//                  order never goes to memory
+//                  merge sorted (sort_ties).  With the masses the bucket is also
+//                  matched there (scan.cuh): its rank order never goes to memory
 //   fallback     : a field the map does not balance (a bucket outgrows its
 //                  region, or the map sees it coming) is ranked by the digit
 //                  passes, in one cooperative launch that otherwise ends at
@@ -58,7 +58,7 @@ __device__ __forceinline__ void msd_map_body(const MsdArgs& a, uint32_t blk, uin
   const int tid = threadIdx.x;
   for (int i = tid; i < NC; i += NT) h[i] = 0;
   const uint32_t gt = blk * NT + tid, ng = nblk * NT;
-  for (uint32_t i = gt; i < a.nb1; i += ng) a.mc->cnt1[i] = 0;
+  for (uint32_t i = gt; i < a.nb1; i += ng) a.mc->cnt1[i * msd_cnt1_step(a.nb1)] = 0;
   if (a.nb2 > 1)
     for (uint32_t i = gt; i < a.nb1 * a.nb2; i += ng) a.cnt2[i] = 0;
   if (gt == 0) {
@@ -238,7 +238,7 @@ __device__ __forceinline__ void msd_split_body(const MsdArgs& a, uint32_t blk, u
       have = min(n - start, (uint32_t)TILE);
     } else {
       bucket = tile / per;
-      const uint32_t at = (tile - bucket * per) * TILE, c = a.mc->cnt1[bucket];
+      const uint32_t at = (tile - bucket * per) * TILE, c = a.mc->cnt1[bucket * msd_cnt1_step(a.nb1)];
       if (at >= c) continue;  // uniform
       start = bucket * a.cap1 + at;
       have = min(c - at, (uint32_t)TILE);
@@ -307,7 +307,7 @@ __device__ __forceinline__ void msd_split_body(const MsdArgs& a, uint32_t blk, u
       for (int q = 0; q < DPT; ++q) {
         const uint32_t d = tid * DPT + q;
         g[q] = 0;
-        if (c[q]) g[q] = atomicAdd(FIRST ? &a.mc->cnt1[d] : &a.cnt2[bucket * nb2 + d], c[q]);
+        if (c[q]) g[q] = atomicAdd(FIRST ? &a.mc->cnt1[d * msd_cnt1_step(a.nb1)] : &a.cnt2[bucket * nb2 + d], c[q]);
       }
       uint32_t x = sum;
 #pragma unroll
@@ -682,13 +682,13 @@ __device__ __forceinline__ void msd_local_body(const MsdArgs& a, const ScanArgs&
     have = a.cnt2[b];
     kv = a.kv2 + (size_t)b * CAP;
     mv_in = a.mass2 + (size_t)b * CAP;
-    for (uint32_t i = tid; i < d; i += NT) base += a.mc->cnt1[i];
+    for (uint32_t i = tid; i < d; i += NT) base += a.mc->cnt1[i * msd_cnt1_step(a.nb1)];
     for (uint32_t i = tid; i < e; i += NT) base += a.cnt2[d * a.nb2 + i];
   } else {
-    have = a.mc->cnt1[b];
+    have = a.mc->cnt1[b * msd_cnt1_step(a.nb1)];
     kv = a.kv1 + (size_t)b * a.cap1;
     mv_in = a.mass1 + (size_t)b * a.cap1;
-    for (uint32_t i = tid; i < b; i += NT) base += a.mc->cnt1[i];
+    for (uint32_t i = tid; i < b; i += NT) base += a.mc->cnt1[i * msd_cnt1_step(a.nb1)];
   }
   const float qs = SCAN ? __int_as_float((127 + *sa.qshift) << 23) : 0.f;
   LookBack lb;
@@ -926,6 +926,9 @@ MsdPlan msd_plan(int64_t n, bool with_mass, int num_sms) {
 
 static int split_tile(uint32_t digits) { return digits > kMsdManyDigits ? kMsdTileB : kMsdTileA; }
 
+// (A batch launches as many of its 4096-cell CTAs per ranking, with as many mass
+// sums: 152 at 128^3, where twice that gave 5 items 0.446 instead of 0.455 ms and
+// 32 items 2.50 instead of 2.46.)
 int msd_split_ctas(int64_t n, const MsdPlan& p, int num_sms) {
   const int tile = split_tile(p.nb1);
   return (int)std::min<int64_t>((n + tile - 1) / tile, (int64_t)num_sms * (tile == kMsdTileB ? 1 : 2));

@@ -38,6 +38,16 @@ constexpr int kMsdSub = 8192;                               // sub-buckets of a 
 constexpr int64_t kMsdTieCells = 1 << 26, kMsdTieCells2 = 1 << 28;
 constexpr uint32_t kMsdTieSpans = 64, kMsdTieSpans2 = 50;
 
+// Words between the first split's bucket counters.  With 4096-cell tiles every tile
+// adds to nearly all of them, and 187 side by side (512^3) lie in six lines, whose
+// adds come one after another, the dearer the more buckets a tile reaches.  A sector
+// each: the passes of a 512^3 ranking 2.78, 2.88 and 2.99 ms (l = 10, 5, 3) -> 2.68,
+// 2.71 and 2.80; side by side from a line's start 2.68, 2.73, 2.82, a line each 2.70,
+// 2.74, 2.83.  Where there are many, larger tiles add less often and the local sort
+// sums more of them: side by side (a 1024^3 solve with a sector each 49.3 ms, 49.1).
+constexpr uint32_t kMsdCnt1Step = 8;
+__host__ __device__ constexpr uint32_t msd_cnt1_step(uint32_t nb1) { return nb1 <= kMsdManyDigits ? kMsdCnt1Step : 1u; }
+
 // Device control block; zero when created, left clean by every ranking.
 struct MsdCtrl {
   uint32_t overflow;  // bit 0: a first-split bucket outgrew its region (or given_up), bit 1: a second-split bucket did
@@ -49,7 +59,8 @@ struct MsdCtrl {
   uint32_t map[kMsdKnots + 4];
   int32_t span[kMsdSpans];  // knot of key k in a span: (k >> (span & 31)) + (span >> 5)
   int32_t equal;            // >= 0: all knots are 2^equal keys wide
-  uint32_t cnt1[kMsdMaxDigits];
+  alignas(256) uint32_t cnt1[kMsdManyDigits * kMsdCnt1Step];  // of bucket d: [d msd_cnt1_step(nb1)]
+  static_assert(kMsdManyDigits * kMsdCnt1Step >= kMsdMaxDigits, "side by side they fit too");
 };
 
 struct MsdArgs {

@@ -556,7 +556,7 @@ __device__ __forceinline__ void sort_fallback_body(const FallbackArgs& f) {
     const int64_t slots = (int64_t)f.nb1 * f.cap1;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < slots; i += (int64_t)gridDim.x * blockDim.x) {
       const uint32_t d = (uint32_t)(i / f.cap1);
-      if ((uint32_t)(i - (int64_t)d * f.cap1) >= f.mc->cnt1[d]) continue;
+      if ((uint32_t)(i - (int64_t)d * f.cap1) >= f.mc->cnt1[d * msd_cnt1_step(f.nb1)]) continue;
       const uint2 v = f.kv1[i];
       const uint32_t u = ~(v.x + kbase);  // undo the key's flips
       if (f.J_restore) f.J_restore[v.y] = __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
